@@ -340,9 +340,207 @@ __global__ void k_init_uniform(float* __restrict__ p, size_t n, unsigned long lo
 
 // ------------------------------------------------------------------ top-k joint bins
 // score(q, d) = log_softmax(lq)[q] + log_softmax(ld)[d]; the k best joint bins q * nd + d of each
-// sample, best first; ties to the lower bin.
-__global__ void __launch_bounds__(kT) k_topk_joint(const float* __restrict__ lq, int nq, const float* __restrict__ ld,
-                                                   int nd, int k, int* __restrict__ bins, float* __restrict__ scores) {
+// sample, best first; ties to the lower bin.  Bins whose score is NaN are left out, and what is then
+// missing of the k is (0x7fffffff, -inf).
+
+// ln sum exp of both heads' logits into *lse_q, *lse_d and d - lse_d into dls, by the first kT threads of
+// the block in a fixed order (every thread of the block takes part in the barriers).
+__device__ void joint_log_norms(const float* q, int nq, const float* d, int nd, float* rv, float* lse_q, float* lse_d,
+                                float* dls) {
+    const int t = threadIdx.x;
+    for (int head = 0; head < 2; ++head) {
+        const float* l = head ? d : q;
+        const int n = head ? nd : nq;
+        float m = -INFINITY;
+        if (t < kT) {
+            for (int i = t; i < n; i += kT) m = fmaxf(m, l[i]);
+            rv[t] = m;
+        }
+        __syncthreads();
+        for (int st = kT / 2; st > 0; st >>= 1) {
+            if (t < st) rv[t] = fmaxf(rv[t], rv[t + st]);
+            __syncthreads();
+        }
+        m = rv[0];
+        __syncthreads();
+        if (t < kT) {
+            float s = 0.f;
+            for (int i = t; i < n; i += kT) s += expf(l[i] - m);
+            rv[t] = s;
+        }
+        __syncthreads();
+        for (int st = kT / 2; st > 0; st >>= 1) {
+            if (t < st) rv[t] += rv[t + st];
+            __syncthreads();
+        }
+        if (t == 0) *(head ? lse_d : lse_q) = m + logf(rv[0]);
+        __syncthreads();
+    }
+    for (int i = t; i < nd; i += blockDim.x) dls[i] = d[i] - *lse_d;
+    __syncthreads();
+}
+
+// Selection and sort, one block per sample: a radix selection finds the k-th largest score (each pass
+// histograms kSelBits more bits of the order-preserving integer form of the scores, starting below
+// the bits they all share), the k bins are compacted into shared memory and sorted there by (score,
+// bin) with a bitonic network, whose steps inside a warp's own 64 entries need no block barrier.
+// Bound by the sort's shared-memory passes: 0.5 log2(k)^2 of them, against one pass over all nq nd
+// scores for every bin picked before (k = 4096 of 18,432, 256 samples: 54.2 ms).
+constexpr int kTopT = 1024, kSelBits = 11;
+constexpr int kTopMaxK = 32768, kTopMaxBins = 65536;   // 6 bytes per sorted entry in shared memory; 16-bit bins
+
+// a before b: larger score first, then the lower bin
+__device__ __forceinline__ bool topk_before(uint32_t ka, uint32_t ia, uint32_t kb, uint32_t ib) {
+    return ka > kb || (ka == kb && ia < ib);
+}
+
+__global__ void __launch_bounds__(kTopT) k_topk_joint(const float* __restrict__ lq, int nq, const float* __restrict__ ld,
+                                                      int nd, int k, int n2, int* __restrict__ bins,
+                                                      float* __restrict__ scores) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    uint32_t* key = reinterpret_cast<uint32_t*>(sm_raw);             // [n2]
+    uint16_t* idx = reinterpret_cast<uint16_t*>(key + n2);           // [n2]
+    __shared__ uint32_t hist[1 << kSelBits];
+    __shared__ float rv[kT], dls[64], lse_q, lse_d;
+    __shared__ uint32_t s_min, s_max, s_valid, s_bin, s_above, s_taken;
+    const int t = threadIdx.x, lane = t & 31;
+    const float* q = lq + (size_t)blockIdx.x * nq;
+    const float* d = ld + (size_t)blockIdx.x * nd;
+    if (t == 0) { s_min = 0xffffffffu; s_max = 0u; s_valid = 0u; s_taken = 0u; }
+    joint_log_norms(q, nq, d, nd, rv, &lse_q, &lse_d, dls);
+    const float lse = lse_q;
+    // order-preserving integer of a score (-0 as +0); 0 for NaN, which is below every score's
+    auto ord = [&](float v) -> uint32_t {
+        const uint32_t u = __float_as_uint(v + 0.f);
+        return v != v ? 0u : (u & 0x80000000u) ? ~u : u | 0x80000000u;
+    };
+    {
+        uint32_t lo = 0xffffffffu, hi = 0u, c = 0;
+        for (int i = t; i < nq; i += kTopT) {
+            const float base = q[i] - lse;
+            for (int e = 0; e < nd; ++e) {
+                const uint32_t o = ord(base + dls[e]);
+                if (o) { lo = min(lo, o); hi = max(hi, o); ++c; }
+            }
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) { atomicMin(&s_min, lo); atomicMax(&s_max, hi); atomicAdd(&s_valid, c); }
+    }
+    __syncthreads();
+    const uint32_t valid = s_valid;
+    const uint32_t need = valid < (uint32_t)k ? valid : (uint32_t)k;
+    // scores with (o >> shift) > prefix are all taken; of those equal to it, the next `left`
+    uint32_t prefix = 0, left = 0;
+    int shift = 32;
+    bool split = need < valid;   // some valid scores stay out
+    if (split) {
+        const uint32_t diff = s_min ^ s_max;
+        shift = diff ? 32 - __clz(diff) : 0;
+        prefix = shift < 32 ? s_max >> shift : 0u;
+        left = need;
+        while (shift > 0) {
+            const int w = min(shift, kSelBits), ns = shift - w;
+            for (int i = t; i < (1 << kSelBits); i += kTopT) hist[i] = 0;
+            __syncthreads();
+            for (int i = t; i < nq; i += kTopT) {
+                const float base = q[i] - lse;
+                for (int e = 0; e < nd; ++e) {
+                    const uint32_t o = ord(base + dls[e]);
+                    if (o && (shift == 32 || (o >> shift) == prefix)) atomicAdd(&hist[(o >> ns) & ((1u << w) - 1u)], 1u);
+                }
+            }
+            __syncthreads();
+            if (t < 32) {   // the bin, from the top, in which the count reaches `left`
+                uint32_t above = 0;
+                for (int b0 = (1 << w) - 1; b0 >= 0; b0 -= 32) {
+                    const int b = b0 - lane;
+                    const uint32_t c = b >= 0 ? hist[b] : 0u;
+                    uint32_t run = c;
+#pragma unroll
+                    for (int off = 1; off < 32; off <<= 1) {
+                        const uint32_t v = __shfl_up_sync(0xffffffffu, run, off);
+                        if (lane >= off) run += v;
+                    }
+                    const unsigned hit = __ballot_sync(0xffffffffu, above + run >= left);
+                    if (hit) {
+                        if (lane == __ffs(hit) - 1) { s_bin = (uint32_t)b; s_above = above + run - c; }
+                        break;
+                    }
+                    above += __shfl_sync(0xffffffffu, run, 31);
+                }
+            }
+            __syncthreads();
+            prefix = (shift == 32 ? 0u : prefix << w) | s_bin;
+            left -= s_above;
+            shift = ns;
+            const bool whole = hist[s_bin] == left;   // the bin is taken whole: no finer threshold needed
+            __syncthreads();
+            if (whole) { split = false; break; }
+        }
+    }
+    // compact: everything above the threshold prefix, and the prefix's own unless only some are taken
+    const bool all = need == valid && shift == 32;
+    for (int i = t; i < nq; i += kTopT) {
+        const float base = q[i] - lse;
+        for (int e = 0; e < nd; ++e) {
+            const uint32_t o = ord(base + dls[e]);
+            const uint32_t top = all ? 0u : o >> shift;
+            if (o && (all || top > prefix || (top == prefix && !split))) {
+                const uint32_t at = atomicAdd(&s_taken, 1u);
+                key[at] = o;
+                idx[at] = (uint16_t)(i * nd + e);
+            }
+        }
+    }
+    __syncthreads();
+    if (split && t < 32) {   // equal scores at the threshold (shift = 0): the lowest bins
+        uint32_t at = s_taken;
+        const int total = nq * nd;
+        for (int j0 = 0; j0 < total && at < need; j0 += 32) {
+            const int j = j0 + lane;
+            const bool tie = j < total && ord((q[j / nd] - lse) + dls[j % nd]) == prefix;
+            const unsigned bal = __ballot_sync(0xffffffffu, tie);
+            const uint32_t my = at + __popc(bal & ((1u << lane) - 1u));
+            if (tie && my < need) {
+                key[my] = prefix;
+                idx[my] = (uint16_t)j;
+            }
+            at += __popc(bal);
+        }
+    }
+    for (int i = need + t; i < n2; i += kTopT) { key[i] = 0u; idx[i] = 0xffffu; }   // after every score
+    __syncthreads();
+    for (int size = 2; size <= n2; size <<= 1) {
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int e = t; e < n2 / 2; e += kTopT) {
+                const int i = 2 * e - (e & (stride - 1)), j = i + stride;
+                const uint32_t ka = key[i], kb = key[j], ia = idx[i], ib = idx[j];
+                if (topk_before(ka, ia, kb, ib) != ((i & size) == 0)) {
+                    key[i] = kb; key[j] = ka;
+                    idx[i] = (uint16_t)ib; idx[j] = (uint16_t)ia;
+                }
+            }
+            // the next step's pairs of a warp lie within its own 64 entries while its stride is at most 32
+            if (stride > 32 || (stride == 1 && size >= 64)) __syncthreads();
+            else __syncwarp();
+        }
+    }
+    __syncthreads();
+    for (int r = t; r < k; r += kTopT) {
+        const bool ok = (uint32_t)r < need;
+        const int j = ok ? (int)idx[r] : 0x7fffffff;
+        bins[(size_t)blockIdx.x * k + r] = j;
+        if (scores) scores[(size_t)blockIdx.x * k + r] = ok ? (q[j / nd] - lse) + dls[j % nd] : -INFINITY;
+    }
+}
+
+// Any nq, nd and k: one pass over the scores for each of the k picks (a sort of more than kTopMaxK
+// entries or of bins beyond 16 bits does not fit in shared memory).
+__global__ void __launch_bounds__(kT) k_topk_joint_scan(const float* __restrict__ lq, int nq,
+                                                        const float* __restrict__ ld, int nd, int k,
+                                                        int* __restrict__ bins, float* __restrict__ scores) {
     const int b = blockIdx.x;
     const float* q = lq + (size_t)b * nq;
     const float* d = ld + (size_t)b * nd;
@@ -350,36 +548,7 @@ __global__ void __launch_bounds__(kT) k_topk_joint(const float* __restrict__ lq,
     __shared__ int ri[kT];
     __shared__ float lse_q, lse_d;
     __shared__ float dls[64];
-    // log-sum-exp of both heads
-    for (int head = 0; head < 2; ++head) {
-        const float* l = head ? d : q;
-        const int n = head ? nd : nq;
-        float m = -INFINITY;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) m = fmaxf(m, l[i]);
-        rv[threadIdx.x] = m;
-        __syncthreads();
-        for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-            if (threadIdx.x < st) rv[threadIdx.x] = fmaxf(rv[threadIdx.x], rv[threadIdx.x + st]);
-            __syncthreads();
-        }
-        m = rv[0];
-        __syncthreads();
-        float s = 0.f;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) s += expf(l[i] - m);
-        rv[threadIdx.x] = s;
-        __syncthreads();
-        for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-            if (threadIdx.x < st) rv[threadIdx.x] += rv[threadIdx.x + st];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            if (head) lse_d = m + logf(rv[0]);
-            else lse_q = m + logf(rv[0]);
-        }
-        __syncthreads();
-    }
-    for (int i = threadIdx.x; i < nd; i += blockDim.x) dls[i] = d[i] - lse_d;
-    __syncthreads();
+    joint_log_norms(q, nq, d, nd, rv, &lse_q, &lse_d, dls);
     const int total = nq * nd;
     int last = -1;
     float last_v = INFINITY;
@@ -709,13 +878,23 @@ int bioem_cnn_train_step(bioem_cnn* n, const float* d_images, const int* d_label
 int bioem_propose(bioem_cnn* n, const float* d_images, int n_img, int k, int* d_bins, float* d_scores) {
     if (!n || !d_images || n_img < 0 || k < 1 || k > n->n_q * n->n_d || !d_bins) return BIOEM_ERR_INVALID_ARG;
     cudaSetDevice(n->ctx->device);
+    const bool sorted = k <= kTopMaxK && (long long)n->n_q * n->n_d <= kTopMaxBins;
+    int n2 = 64;   // entries of the sorting network: a power of two, at least a warp's 64
+    while (sorted && n2 < k) n2 *= 2;
+    const size_t sm = (size_t)n2 * 6;
+    if (sorted && cudaFuncSetAttribute(k_topk_joint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+        return bioem_check_cuda(n->ctx, cudaGetLastError(), "top-k shared memory");
     for (int b0 = 0; b0 < n_img; b0 += n->max_batch) {
         const int B = n_img - b0 < n->max_batch ? n_img - b0 : n->max_batch;
         int rc = prepare_input(n, d_images + (size_t)b0 * n->n_in * n->n_in, B);
         if (!rc) rc = forward(n, B);
         if (rc) return rc;
-        k_topk_joint<<<B, kT, 0, n->ctx->stream>>>(n->d_lq, n->n_q, n->d_ld, n->n_d, k, d_bins + (size_t)b0 * k,
-                                                   d_scores ? d_scores + (size_t)b0 * k : nullptr);
+        int* bins = d_bins + (size_t)b0 * k;
+        float* scores = d_scores ? d_scores + (size_t)b0 * k : nullptr;
+        if (sorted)
+            k_topk_joint<<<B, kTopT, sm, n->ctx->stream>>>(n->d_lq, n->n_q, n->d_ld, n->n_d, k, n2, bins, scores);
+        else
+            k_topk_joint_scan<<<B, kT, 0, n->ctx->stream>>>(n->d_lq, n->n_q, n->d_ld, n->n_d, k, bins, scores);
         n->ctx->n_launches++;
         rc = check(n->ctx, "propose");
         if (rc) return rc;
