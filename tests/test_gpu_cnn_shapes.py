@@ -1,5 +1,6 @@
-"""GPU: the proposal network's kernels where their tiles end: the top-k at the edges of its sorting
-network, with equal and undefined scores."""
+"""GPU: the proposal network's kernels where their tiles end: image sizes and channel counts that are no
+multiple of a thread's or a block's share, column tiles beyond the first, and the top-k at the edges of
+its sorting network, with equal and undefined scores."""
 import numpy as np
 import pytest
 
@@ -22,6 +23,38 @@ def env():
 def _dev(x):
     import torch
     return torch.from_numpy(np.ascontiguousarray(x)).to("cuda:0")
+
+
+# (image px, downsample, channels, orientation bins, defocus bins, batch): 8 px leaves 1 px outputs; 24 px
+# rows are no whole groups of four at the last layers; 33 and 64 channels take a second channel block;
+# 72 px rows take a second column tile of the weight gradients
+@pytest.mark.parametrize("px,down,C,nq,nd,B", [(8, 1, 3, 5, 1, 2), (24, 1, 5, 70, 3, 3), (32, 1, 33, 9, 2, 2),
+                                               (32, 1, 64, 130, 64, 1), (144, 2, 4, 7, 5, 2), (64, 1, 17, 65, 4, 67)])
+def test_network_shapes(env, px, down, C, nq, nd, B):
+    """Logits, losses and gradients against float64.  Tolerance: the sums run over at most a few 1e5
+    FP32 terms (relative error below 1e-4); a ReLU input that rounds across zero moves a gradient by a
+    share of one sample's part, below the 2e-3 that the other network tests allow."""
+    bioem, ctx = env
+    rng = np.random.default_rng(100 + px + C)
+    net = bioem.CNN(ctx, image_px=px, downsample=down, channels=C, n_qbins=nq, n_dbins=nd, max_batch=B, seed=1)
+    _, _, _, n = ocnn.layout(px // down, C, nq, nd)
+    theta = (rng.standard_normal(n) * (1.5 / np.sqrt(9 * C))).astype(np.float16).astype(np.float64)
+    imgs = rng.standard_normal((B, px, px)).astype(np.float32)
+    yq, yd = rng.integers(0, nq, B).astype(np.int32), rng.integers(0, nd, B).astype(np.int32)
+    net.set_params(_dev(theta.astype(np.float32)))
+    lq, ld = net.forward(_dev(imgs))
+    g, loss = net.gradients(_dev(imgs), _dev(yq), _dev(yd))
+    want_loss, want_g = ocnn.loss_and_grad(theta, imgs.astype(np.float64), yq, yd, down, C, nq, nd)
+    wq, wd, _ = ocnn.forward(theta, imgs.astype(np.float64), down, C, nq, nd)
+    np.testing.assert_allclose(lq.cpu().numpy(), wq, rtol=0, atol=1e-4 * np.abs(wq).max())
+    np.testing.assert_allclose(ld.cpu().numpy(), wd, rtol=0, atol=1e-4 * np.abs(wd).max())
+    np.testing.assert_allclose(loss.cpu().numpy(), want_loss, rtol=2e-4)
+    offs, heads, _, _ = ocnn.layout(px // down, C, nq, nd)
+    got = g.cpu().numpy().astype(np.float64)
+    for off, shape in [o for pair in offs for o in pair] + list(heads):
+        sl = slice(off, off + int(np.prod(shape)))
+        err = np.linalg.norm(got[sl] - want_g[sl]) / max(np.linalg.norm(want_g[sl]), 1e-12)
+        assert err < 2e-3, (off, shape, err)
 
 
 # sorting networks of 64 (the smallest), 128, 2048 and 4096 entries, whole and partly filled; 70,000 bins
