@@ -23,176 +23,305 @@
 
 namespace {
 
-constexpr int kThreads = 256;
+// Threads of the transform kernels: two blocks per SM up to 128 px; at 192 px a block's spectrum fills
+// the SM's shared memory, so it has 512.
+template <int N>
+struct Dft {
+    static constexpr int T = N == 192 ? 512 : 256;
+    static constexpr int NC = N / 2, H = NC + 1;
+    // Register tiles: 16 lanes share a group's KY rows (or frequencies) and take KX columns each, 16
+    // apart.  A dense sum costs N multiply-adds per output either way; the tile is what lets a value
+    // loaded from shared memory serve 8 (x KX) or 4 (x KY) of them at 128 px instead of one.
+    static constexpr int G = T / 16, KY = N / G, KX = NC / 16;
+    static_assert(KY * G == N && KX * 16 == NC, "whole tiles; the kx = N/2 column is summed apart");
+    static constexpr int PER = (N * H + T - 1) / T;   // coefficients per thread in the passes over a spectrum
+};
 
-// Deterministic block sum of two doubles (fixed tree order).
-__device__ void block_sum2(double& a, double& b, double* red) {
-    const int tid = threadIdx.x;
-    red[tid] = a;
-    red[blockDim.x + tid] = b;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (tid < s) {
-            red[tid] += red[tid + s];
-            red[blockDim.x + tid] += red[blockDim.x + tid + s];
-        }
-        __syncthreads();
+// Deterministic block sums of two doubles (fixed order: lanes, then warps); red holds 2 T / 32 doubles.
+template <int T>
+__device__ __forceinline__ void block_sum2(double& a, double& b, double* red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, off);
+        b += __shfl_xor_sync(0xffffffffu, b, off);
     }
+    if (lane == 0) {
+        red[warp] = a;
+        red[T / 32 + warp] = b;
+    }
+    __syncthreads();
     a = red[0];
-    b = red[blockDim.x];
+    b = red[T / 32];
+    for (int w = 1; w < T / 32; ++w) {
+        a += red[w];
+        b += red[T / 32 + w];
+    }
     __syncthreads();
 }
 
-// F[y][kx] = sum_x (img[y][x] - mean) W^(kx x), kx = 0..N/2 (row pass of a real 2-D transform).
+// Largest value over the block, in every thread; red holds T / 32 floats.
+template <int T>
+__device__ __forceinline__ float block_max(float v, float* red) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    v = red[0];
+    for (int w = 1; w < T / 32; ++w) v = fmaxf(v, red[w]);
+    __syncthreads();
+    return v;
+}
+
+// (idx + step) mod N for idx, step < N: the smaller of the two candidates as unsigned numbers
 template <int N>
-__device__ void r2c_rows(const float* __restrict__ img, float mean, float2* F, const float2* tw) {
-    constexpr int H = N / 2 + 1;
-    for (int o = threadIdx.x; o < N * H; o += blockDim.x) {
-        const int y = o / H, kx = o - y * H;
-        const float* row = img + y * N;
-        float re = 0.f, im = 0.f;
-        int idx = 0;
-#pragma unroll 8
-        for (int x = 0; x < N; ++x) {
-            const float v = row[x] - mean;
-            const float2 w = tw[idx];
-            re = fmaf(v, w.x, re);
-            im = fmaf(v, w.y, im);
-            idx += kx;
-            idx -= (idx >= N) ? N : 0;
+__device__ __forceinline__ unsigned step_mod(unsigned idx, unsigned step) {
+    if constexpr ((N & (N - 1)) == 0) return (idx + step) & (N - 1);
+    else return min(idx + step, idx + step - N);
+}
+
+// Shared memory of the transform kernels.
+template <int N>
+struct DftSm {
+    float2* F;      // [N][H]
+    float2* tw;     // [N] exp(-2 pi i t / N)
+    float2* ts;     // [N] the same with its parts exchanged: (w.y, w.x)
+    double* red;    // [4 T / 32]
+    __device__ __forceinline__ explicit DftSm(unsigned char* smem) {
+        F = reinterpret_cast<float2*>(smem);
+        tw = F + N * Dft<N>::H;
+        ts = tw + N;
+        red = reinterpret_cast<double*>(ts + N);
+    }
+    // the twiddle pair of the forward transform, or of the inverse (conjugates)
+    __device__ __forceinline__ void twiddles(const float2* __restrict__ g_tw, bool inverse) const {
+        for (int i = threadIdx.x; i < N; i += Dft<N>::T) {
+            const float2 w = g_tw[i];
+            const float y = inverse ? -w.y : w.y;
+            tw[i] = make_float2(w.x, y);
+            ts[i] = make_float2(y, w.x);
         }
-        F[o] = make_float2(re, im);
+    }
+    static constexpr size_t bytes() {
+        return (size_t)(N * Dft<N>::H + 2 * N) * sizeof(float2) + 4 * (Dft<N>::T / 32) * sizeof(double);
+    }
+};
+
+// F[y][kx] = sum_x (img[y][x] - mean) W^(kx x), kx = 0..N/2 (row pass of a real 2-D transform), x ascending
+// in one FP32 accumulator per output.
+template <int N, bool VEC = true>
+__device__ __forceinline__ void r2c_rows(const float* __restrict__ img, float mean, const DftSm<N>& sm) {
+    // four pixels of a row; VEC: img is 16-byte aligned
+    auto load4 = [](const float* p) {
+        if constexpr (VEC) return __ldg(reinterpret_cast<const float4*>(p));
+        else return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+    };
+    using D = Dft<N>;
+    constexpr int H = D::H, KY = D::KY, KX = D::KX;
+    const int g = threadIdx.x >> 4, l = threadIdx.x & 15;
+    float2 acc[KY][KX];
+    unsigned idx[KX];
+#pragma unroll
+    for (int k = 0; k < KX; ++k) {
+        idx[k] = 0;
+#pragma unroll
+        for (int i = 0; i < KY; ++i) acc[i][k] = make_float2(0.f, 0.f);
+    }
+#pragma unroll 1
+    for (int x0 = 0; x0 < N; x0 += 4) {
+        float v[KY][4];
+#pragma unroll
+        for (int i = 0; i < KY; ++i) {
+            const float4 q = load4(img + (size_t)(g * KY + i) * N + x0);
+            v[i][0] = q.x - mean; v[i][1] = q.y - mean; v[i][2] = q.z - mean; v[i][3] = q.w - mean;
+        }
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int k = 0; k < KX; ++k) {
+                const float2 w = sm.tw[idx[k]];
+                idx[k] = step_mod<N>(idx[k], l + 16 * k);
+#pragma unroll
+                for (int i = 0; i < KY; ++i) acc[i][k] = __ffma2_rn(make_float2(v[i][x], v[i][x]), w, acc[i][k]);
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < KY; ++i)
+#pragma unroll
+        for (int k = 0; k < KX; ++k) sm.F[(g * KY + i) * H + l + 16 * k] = acc[i][k];
+    if (threadIdx.x < N) {   // kx = N/2: the twiddles alternate between t = 0 and N/2
+        const float* row = img + (size_t)threadIdx.x * N;
+        float2 a = make_float2(0.f, 0.f);
+        const float2 w0 = sm.tw[0], w1 = sm.tw[N / 2];
+        for (int x0 = 0; x0 < N; x0 += 4) {
+            const float4 q = load4(row + x0);
+            const float v[4] = {q.x - mean, q.y - mean, q.z - mean, q.w - mean};
+#pragma unroll
+            for (int x = 0; x < 4; ++x) a = __ffma2_rn(make_float2(v[x], v[x]), (x & 1) ? w1 : w0, a);
+        }
+        sm.F[threadIdx.x * H + N / 2] = a;
     }
 }
 
-// In place over shared memory: F[ky][kx] <- sum_y F[y][kx] W^(ky y) (column pass), or with the
-// conjugate twiddle when inverse is true.  Processed in blocks of columns so that every read of
-// a column precedes every write to it.
-template <int N, bool INVERSE>
-__device__ void c2c_columns_inplace(float2* F, const float2* tw) {
-    constexpr int H = N / 2 + 1;
-    constexpr int CB = 8;                               // columns per block
-    constexpr int PER = (N * CB + kThreads - 1) / kThreads;
-    for (int c0 = 0; c0 < H; c0 += CB) {
-        const int ncol = min(CB, H - c0);
-        float2 res[PER];
+// In place over shared memory: F[ky][kx] <- sum_y F[y][kx] W^(ky y) with the twiddles in sm.tw (column
+// pass; the inverse with conjugate twiddles), y ascending, re and im each in one FP32 accumulator.  All
+// outputs are held in registers until every read is done.
+template <int N>
+__device__ __forceinline__ void c2c_columns_inplace(const DftSm<N>& sm) {
+    using D = Dft<N>;
+    constexpr int H = D::H, KY = D::KY, KX = D::KX;
+    const int g = threadIdx.x >> 4, l = threadIdx.x & 15;
+    float2 acc[KY][KX];
+    unsigned idx[KY];
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int o = threadIdx.x + i * kThreads;
-            res[i] = make_float2(0.f, 0.f);
-            if (o < N * ncol) {
-                const int ky = o / ncol, kx = c0 + (o - (o / ncol) * ncol);
-                float re = 0.f, im = 0.f;
-                int idx = 0;
-#pragma unroll 8
-                for (int y = 0; y < N; ++y) {
-                    const float2 v = F[y * H + kx];
-                    float2 w = tw[idx];
-                    if (INVERSE) w.y = -w.y;
-                    re = fmaf(v.x, w.x, fmaf(-v.y, w.y, re));
-                    im = fmaf(v.x, w.y, fmaf(v.y, w.x, im));
-                    idx += ky;
-                    idx -= (idx >= N) ? N : 0;
-                }
-                res[i] = make_float2(re, im);
+    for (int i = 0; i < KY; ++i) {
+        idx[i] = 0;
+#pragma unroll
+        for (int k = 0; k < KX; ++k) acc[i][k] = make_float2(0.f, 0.f);
+    }
+#pragma unroll 2
+    for (int y = 0; y < N; ++y) {
+        float2 v[KX];
+#pragma unroll
+        for (int k = 0; k < KX; ++k) v[k] = sm.F[y * H + l + 16 * k];
+#pragma unroll
+        for (int i = 0; i < KY; ++i) {
+            const float2 w = sm.tw[idx[i]], ws = sm.ts[idx[i]];
+            idx[i] = step_mod<N>(idx[i], g * KY + i);
+#pragma unroll
+            for (int k = 0; k < KX; ++k) {
+                // re += -v.y w.y, then v.x w.x; im += v.y w.x, then v.x w.y
+                acc[i][k] = __ffma2_rn(make_float2(-v[k].y, v[k].y), ws, acc[i][k]);
+                acc[i][k] = __ffma2_rn(make_float2(v[k].x, v[k].x), w, acc[i][k]);
             }
         }
-        __syncthreads();
-#pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int o = threadIdx.x + i * kThreads;
-            if (o < N * ncol) {
-                const int ky = o / ncol, kx = c0 + (o - (o / ncol) * ncol);
-                F[ky * H + kx] = res[i];
-            }
+    }
+    float2 last = make_float2(0.f, 0.f);   // kx = N/2, one ky per thread
+    if (threadIdx.x < N) {
+        unsigned t = 0;
+        for (int y = 0; y < N; ++y) {
+            const float2 v = sm.F[y * H + N / 2];
+            const float2 w = sm.tw[t], ws = sm.ts[t];
+            t = step_mod<N>(t, threadIdx.x);
+            last = __ffma2_rn(make_float2(-v.y, v.y), ws, last);
+            last = __ffma2_rn(make_float2(v.x, v.x), w, last);
         }
-        __syncthreads();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < KY; ++i)
+#pragma unroll
+        for (int k = 0; k < KX; ++k) sm.F[(g * KY + i) * H + l + 16 * k] = acc[i][k];
+    if (threadIdx.x < N) sm.F[threadIdx.x * H + N / 2] = last;
+    __syncthreads();
+}
+
+// The inverse row pass: real[y][x] = G(0) + (-1)^x G(N/2) + 2 sum_{0 < kx < N/2} Re(G(kx) exp(+2 pi i kx x / N)) of the
+// rows G of sm.F, kx ascending; put(y, x, value) for every pixel.  sm.tw holds the FORWARD twiddles.
+template <int N, class PUT>
+__device__ __forceinline__ void c2r_rows(const DftSm<N>& sm, PUT&& put) {
+    using D = Dft<N>;
+    constexpr int H = D::H, KY = D::KY, KX = N / 16;
+    const int g = threadIdx.x >> 4, l = threadIdx.x & 15;
+    float acc[KY][KX];
+    unsigned idx[KX];
+#pragma unroll
+    for (int k = 0; k < KX; ++k) {
+        idx[k] = l + 16 * k;
+#pragma unroll
+        for (int i = 0; i < KY; ++i) acc[i][k] = 0.f;
+    }
+#pragma unroll 1
+    for (int kx = 1; kx < N / 2; ++kx) {
+        float2 v[KY];
+#pragma unroll
+        for (int i = 0; i < KY; ++i) v[i] = sm.F[(g * KY + i) * H + kx];
+#pragma unroll
+        for (int k = 0; k < KX; ++k) {
+            const float2 w = sm.tw[idx[k]];   // exp(-2 pi i kx x / N); conjugated below
+            idx[k] = step_mod<N>(idx[k], l + 16 * k);
+#pragma unroll
+            for (int i = 0; i < KY; ++i) acc[i][k] = fmaf(v[i].x, w.x, fmaf(v[i].y, w.y, acc[i][k]));
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < KY; ++i) {
+        const int y = g * KY + i;
+        const float g0 = sm.F[y * H].x, gn = sm.F[y * H + N / 2].x;
+#pragma unroll
+        for (int k = 0; k < KX; ++k) {
+            const int x = l + 16 * k;
+            const float v = g0 + ((x & 1) ? -gn : gn);
+            put(y, x, v + 2.f * acc[i][k]);
+        }
     }
 }
 
+// Write F * T * scale (T may be null; DC zeroed) to a [N][N/2 + 1] half spectrum; returns the calling thread's
+// largest |coefficient|.
 template <int N>
-__device__ void load_twiddles(const float2* __restrict__ g_tw, float2* tw) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = g_tw[i];
-}
-
-// Write F * T * scale (DC zeroed) to a [N][N/2 + 1] half spectrum; returns (to thread 0) the largest
-// |coefficient| written (block reduction over red, which must hold blockDim.x floats).
-template <int N>
-__device__ float store_half_spectrum(const float2* F, const float* __restrict__ T, float scale,
-                                     float2* __restrict__ spec, float* red) {
-    constexpr int H = N / 2 + 1;
+__device__ __forceinline__ float store_half_spectrum(const float2* F, const float* __restrict__ T, float scale,
+                                                     float2* __restrict__ spec) {
     float amax = 0.f;
-    for (int o = threadIdx.x; o < N * H; o += blockDim.x) {
+    for (int o = threadIdx.x; o < N * Dft<N>::H; o += Dft<N>::T) {
         float2 v = F[o];
-        if (T) v = c_scale(v, T[o]);
+        if (T) v = c_scale(v, __ldg(T + o));
         v = c_scale(v, scale);
         if (o == 0) v = make_float2(0.f, 0.f);
         spec[o] = v;
         amax = fmaxf(amax, fmaxf(fabsf(v.x), fabsf(v.y)));
     }
-    red[threadIdx.x] = amax;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) red[threadIdx.x] = fmaxf(red[threadIdx.x], red[threadIdx.x + st]);
-        __syncthreads();
-    }
-    const float r = red[0];
-    __syncthreads();
-    return r;
+    return amax;
 }
 
-// sum over k != 0 of w_kx |F T|^2 over the full spectrum (w = 1 on the kx = 0 and N/2 columns,
-// 2 elsewhere: the Hermitian partners of the half spectrum), in float64.
+// k != 0 of the half spectrum stands for w_kx of the full one's coefficients: 1 on the kx = 0 and kx = N/2
+// columns, 2 elsewhere (their Hermitian partners); 0 at DC.
 template <int N>
-__device__ double half_spectrum_energy(const float2* F, const float* __restrict__ T, double* red) {
-    constexpr int H = N / 2 + 1;
-    double e = 0.0, dummy = 0.0;
-    for (int o = threadIdx.x; o < N * H; o += blockDim.x) {
-        if (o == 0) continue;
-        const int kx = o % H;
-        float2 v = F[o];
-        if (T) v = c_scale(v, T[o]);
-        const double m = (double)v.x * v.x + (double)v.y * v.y;
-        e += (kx == 0 || kx == N / 2) ? m : 2.0 * m;
-    }
-    block_sum2(e, dummy, red);
-    return e;
+__device__ __forceinline__ double half_weight(int o) {
+    const int kx = o % Dft<N>::H;
+    return o == 0 ? 0.0 : (kx == 0 || kx == N / 2) ? 1.0 : 2.0;
 }
 
-template <int N>
-__global__ void __launch_bounds__(kThreads) k_prepare_images(const float* __restrict__ images,
+// VEC: the images start on a 16-byte boundary (a caller's tensor may be a view that does not).
+template <int N, bool VEC>
+__global__ void __launch_bounds__(Dft<N>::T) k_prepare_images(const float* __restrict__ images,
                                                               const float2* __restrict__ g_tw,
                                                               float2* __restrict__ spec,
                                                               double* __restrict__ kA, float* __restrict__ amax,
                                                               double cn,
                                                               int* __restrict__ status) {
-    constexpr int H = N / 2 + 1;
+    constexpr int H = Dft<N>::H, T = Dft<N>::T;
     extern __shared__ __align__(16) unsigned char smem[];
-    float2* F = reinterpret_cast<float2*>(smem);
-    float2* tw = F + N * H;
-    double* red = reinterpret_cast<double*>(tw + N);
+    const DftSm<N> sm(smem);
     const int w = blockIdx.x;
     const float* img = images + (size_t)w * N * N;
-    load_twiddles<N>(g_tw, tw);
+    sm.twiddles(g_tw, false);
 
     double s1 = 0.0, s2 = 0.0;
-    for (int i = threadIdx.x; i < N * N; i += blockDim.x) {
+    for (int i = threadIdx.x; i < N * N; i += T) {
         const double v = img[i];
         s1 += v;
         s2 += v * v;
     }
-    block_sum2(s1, s2, red);
+    block_sum2<T>(s1, s2, sm.red);
     const double n = (double)N * N;
     const double A = n * s2 - s1 * s1;   // n C_oo - C_o^2
     const float mean = (float)(s1 / n);
 
-    r2c_rows<N>(img, mean, F, tw);
+    r2c_rows<N, VEC>(img, mean, sm);
     __syncthreads();
-    c2c_columns_inplace<N, false>(F, tw);
-    const double e = half_spectrum_energy<N>(F, nullptr, red);
+    c2c_columns_inplace<N>(sm);
+    double e = 0.0, dummy = 0.0;
+    for (int o = threadIdx.x; o < N * H; o += T) {
+        const float2 v = sm.F[o];
+        e += half_weight<N>(o) * ((double)v.x * v.x + (double)v.y * v.y);
+    }
+    block_sum2<T>(e, dummy, sm.red);
     const bool bad = !(A > 0.0) || !(e > 0.0);
     const float scale = bad ? 0.f : (float)(1.0 / sqrt(e));
-    const float mx = store_half_spectrum<N>(F, nullptr, scale, spec + (size_t)w * N * H, reinterpret_cast<float*>(red));
+    const float mx = block_max<T>(store_half_spectrum<N>(sm.F, nullptr, scale, spec + (size_t)w * N * H),
+                                  reinterpret_cast<float*>(sm.red));
     if (threadIdx.x == 0) {
         amax[w] = mx;
         if (bad) {
@@ -397,56 +526,144 @@ __global__ void __launch_bounds__(ProjCfg<N>::T) k_project(const float4* __restr
 }
 
 // T[c][ky][kx] = CTF(s) Env(s) for PSF c on the half-spectrum grid, evaluated in float64.
-// coef[3c..3c+2] = (a, A, b); s = 2 pi (kx~, ky~) / (N pixel) with signed frequency indices.
+// coef[3c..3c+2] = (a, A, b); s = 2 pi (kx~, ky~) / (N pixel) with signed frequency indices.  The value depends on kx~^2 + ky~^2 only, so each unordered pair {|kx~|, |ky~|} is
+// evaluated once and written to its (up to four) places: bound by float64 arithmetic, a quarter of
+// evaluating every coefficient (1.20 ms for 1024 PSFs at 128 px before).
 __global__ void k_ctf_table(const double* __restrict__ coef, int nctf, int N, double pixel,
                             float* __restrict__ T) {
-    const int H = N / 2 + 1;
-    const int total = nctf * N * H;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-        const int c = i / (N * H);
-        const int r = i - c * N * H;
-        const int ky = r / H, kx = r - (r / H) * H;
-        const double fy = (ky <= N / 2) ? ky : ky - N;
-        const double f = 2.0 * 3.14159265358979323846 / (N * pixel);
-        const double s2 = f * f * ((double)kx * kx + fy * fy);
+    const int H = N / 2 + 1, tri = H * (H + 1) / 2;
+    const long long total = (long long)nctf * tri;
+    const double f = 2.0 * 3.14159265358979323846 / (N * pixel);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+        const int c = (int)(i / tri);
+        const int r = (int)(i - (long long)c * tri);
+        // r = hi (hi + 1) / 2 + lo, lo <= hi
+        int hi = (int)((sqrtf(8.f * (float)r + 1.f) - 1.f) * 0.5f);
+        while ((hi + 1) * (hi + 2) / 2 <= r) ++hi;
+        while (hi * (hi + 1) / 2 > r) --hi;
+        const int lo = r - hi * (hi + 1) / 2;
+        const double s2 = f * f * ((double)lo * lo + (double)hi * hi);
         const double a = coef[3 * c], A = coef[3 * c + 1], b = coef[3 * c + 2];
         const double ctf = -A * cos(0.5 * a * s2) - sqrt(1.0 - A * A) * sin(0.5 * a * s2);
-        T[i] = (float)(ctf * exp(-0.5 * b * s2));
+        const float v = (float)(ctf * exp(-0.5 * b * s2));
+        auto put = [&](int ky, int kx) { T[(size_t)c * N * H + (size_t)ky * H + kx] = v; };
+        put(lo, hi);
+        if (lo > 0 && lo < N / 2) put(N - lo, hi);
+        if (lo != hi) {
+            put(hi, lo);
+            if (hi < N / 2) put(N - hi, lo);
+        }
     }
 }
 
+// (hi, lo) += w x^2 in FP32 pairs, w a power of two: the square and the sum with their rounding errors
+// (error-free transforms of Dekker and Knuth), the errors summed in lo.
+__device__ __forceinline__ void add_square(float& hi, float& lo, float x, float w) {
+    const float p0 = x * x, e = fmaf(x, x, -p0) * w, p = p0 * w;
+    const float s = hi + p, b = s - hi;
+    lo += (hi - (s - b)) + (p - b) + e;
+    hi = s;
+}
+
+// One orientation per block: transform I0, and for every PSF c the energy B_c = sum_{k != 0} w_kx |F T_c|^2 (of
+// the FP32 products that are stored) and the normalised product.
+// GB300's float64 rate is 1/70 of its FP32 rate, and squaring every product in float64 (two conversions
+// and three operations) took most of the kernel's 1.5 us per orientation (128 px, 8 PSFs).  Each thread now
+// sums its squares in runs of kRun as FP32 pairs (relative error about 2^-46 per run, independent between
+// the ~800 runs of a spectrum, so 1e-16 of B) and adds the runs in float64.  The products are scaled by a
+// power of two so that the largest |F| is near 1; a B so small against it that squares may have lost bits
+// to underflow (below kSmall) is summed again in float64 throughout.
+constexpr int kPsfChunk = 16;   // PSFs whose energies are reduced together
+constexpr int kRun = 11;
+constexpr double kSmall = 1e-12;
+
 template <int N>
-__global__ void __launch_bounds__(kThreads) k_psf_spectra(const float* __restrict__ img0,
+__device__ __forceinline__ double psf_energy64(const float2* F, const float* __restrict__ T) {
+    double e = 0.0;
+    for (int o = threadIdx.x; o < N * Dft<N>::H; o += Dft<N>::T) {
+        const float2 v = c_scale(F[o], __ldg(T + o));
+        e += half_weight<N>(o) * ((double)v.x * v.x + (double)v.y * v.y);
+    }
+    return e;
+}
+
+template <int N>
+__global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(const float* __restrict__ img0,
                                                            const float2* __restrict__ g_tw,
                                                            const float* __restrict__ T, int nctf,
                                                            float2* __restrict__ spec,
                                                            double* __restrict__ kB, float* __restrict__ amax,
                                                            int* __restrict__ status) {
-    constexpr int H = N / 2 + 1;
+    constexpr int H = Dft<N>::H, TH = Dft<N>::T, PER = Dft<N>::PER;
     extern __shared__ __align__(16) unsigned char smem[];
-    float2* F = reinterpret_cast<float2*>(smem);
-    float2* tw = F + N * H;
-    double* red = reinterpret_cast<double*>(tw + N);
+    __shared__ double part[kPsfChunk][TH / 32];
+    const DftSm<N> sm(smem);
     const int q = blockIdx.x;
-    load_twiddles<N>(g_tw, tw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    sm.twiddles(g_tw, false);
     __syncthreads();
-    r2c_rows<N>(img0 + (size_t)q * N * N, 0.f, F, tw);
+    r2c_rows<N>(img0 + (size_t)q * N * N, 0.f, sm);
     __syncthreads();
-    c2c_columns_inplace<N, false>(F, tw);
-    for (int c = 0; c < nctf; ++c) {
-        const float* Tc = T + (size_t)c * N * H;
-        const double B = half_spectrum_energy<N>(F, Tc, red);   // n C_cc - C_c^2 (Plancherel)
-        const bool bad = !(B > 0.0);
-        const size_t p = (size_t)q * nctf + c;
-        const float mx = store_half_spectrum<N>(F, Tc, bad ? 0.f : (float)(1.0 / sqrt(B)), spec + p * N * H,
-                                                reinterpret_cast<float*>(red));
-        if (threadIdx.x == 0) {
-            amax[p] = mx;
-            if (bad) {
-                atomicOr(status, BIOEM_DEV_NUMERIC);
-                kB[p] = -INFINITY;
-            } else {
-                kB[p] = -0.5 * log(B);
+    c2c_columns_inplace<N>(sm);
+    // power of two near 1 / max |F| over k != 0 (1 for an empty or non-finite spectrum)
+    float fm = 0.f;
+    for (int o = threadIdx.x; o < N * H; o += TH)
+        if (o > 0) fm = fmaxf(fm, fmaxf(fabsf(sm.F[o].x), fabsf(sm.F[o].y)));
+    fm = block_max<TH>(fm, reinterpret_cast<float*>(sm.red));
+    int ex = 0;
+    if (fm > 0.f && fm < INFINITY) frexpf(fm, &ex);
+    ex = max(-120, min(120, ex));
+    const float sc = ldexpf(1.f, -ex);
+    for (int c0 = 0; c0 < nctf; c0 += kPsfChunk) {
+        const int nc = min(kPsfChunk, nctf - c0);
+        for (int c = 0; c < nc; ++c) {
+            const float* Tc = T + (size_t)(c0 + c) * N * H;
+            double e = 0.0;
+#pragma unroll
+            for (int i0 = 0; i0 < PER; i0 += kRun) {
+                float hi = 0.f, lo = 0.f;
+#pragma unroll
+                for (int i = i0; i < i0 + kRun && i < PER; ++i) {
+                    const int o = threadIdx.x + i * TH;
+                    if (o < N * H) {
+                        const int kx = o % H;
+                        const float2 v = c_scale(c_scale(sm.F[o], __ldg(Tc + o)), o == 0 ? 0.f : sc);
+                        const float w = kx == 0 || kx == N / 2 ? 1.f : 2.f;
+                        add_square(hi, lo, v.x, w);
+                        add_square(hi, lo, v.y, w);
+                    }
+                }
+                e += (double)hi + (double)lo;
+            }
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
+            if (lane == 0) part[c][warp] = e;
+        }
+        __syncthreads();
+        for (int c = 0; c < nc; ++c) {
+            const float* Tc = T + (size_t)(c0 + c) * N * H;
+            double B = part[c][0];
+            for (int w = 1; w < TH / 32; ++w) B += part[c][w];
+            if (B > kSmall && B < INFINITY) {
+                B = ldexp(B, 2 * ex);
+            } else {   // uniform over the block
+                double dummy = 0.0;
+                B = psf_energy64<N>(sm.F, Tc);
+                block_sum2<TH>(B, dummy, sm.red);
+            }
+            const bool bad = !(B > 0.0);   // B = n C_cc - C_c^2 (Plancherel)
+            const size_t p = (size_t)q * nctf + c0 + c;
+            const float mx = block_max<TH>(store_half_spectrum<N>(sm.F, Tc, bad ? 0.f : (float)(1.0 / sqrt(B)),
+                                                                  spec + p * N * H),
+                                           reinterpret_cast<float*>(sm.red));
+            if (threadIdx.x == 0) {
+                amax[p] = mx;
+                if (bad) {
+                    atomicOr(status, BIOEM_DEV_NUMERIC);
+                    kB[p] = -INFINITY;
+                } else {
+                    kB[p] = -0.5 * log(B);
+                }
             }
         }
     }
@@ -454,41 +671,29 @@ __global__ void __launch_bounds__(kThreads) k_psf_spectra(const float* __restric
 
 // Synthetic map for pair i: I1 = Re F^-1[F(I0_i) T_i] with F^-1 normalised by 1/N^2.
 template <int N>
-__global__ void __launch_bounds__(kThreads) k_psf_real(const float* __restrict__ img0,
+__global__ void __launch_bounds__(Dft<N>::T) k_psf_real(const float* __restrict__ img0,
                                                         const float2* __restrict__ g_tw,
                                                         const float* __restrict__ T,
                                                         float* __restrict__ out) {
-    constexpr int H = N / 2 + 1;
+    constexpr int H = Dft<N>::H, TH = Dft<N>::T;
     extern __shared__ __align__(16) unsigned char smem[];
-    float2* F = reinterpret_cast<float2*>(smem);
-    float2* tw = F + N * H;
+    const DftSm<N> sm(smem);
     const int i = blockIdx.x;
-    load_twiddles<N>(g_tw, tw);
+    sm.twiddles(g_tw, false);
     __syncthreads();
-    r2c_rows<N>(img0 + (size_t)i * N * N, 0.f, F, tw);
+    r2c_rows<N>(img0 + (size_t)i * N * N, 0.f, sm);
     __syncthreads();
-    c2c_columns_inplace<N, false>(F, tw);
+    c2c_columns_inplace<N>(sm);
     const float* Ti = T + (size_t)i * N * H;
-    for (int o = threadIdx.x; o < N * H; o += blockDim.x) F[o] = c_scale(F[o], Ti[o]);
+    for (int o = threadIdx.x; o < N * H; o += TH) sm.F[o] = c_scale(sm.F[o], __ldg(Ti + o));
+    sm.twiddles(g_tw, true);
     __syncthreads();
-    c2c_columns_inplace<N, true>(F, tw);
-    // rows: I(y, x) = (1/N^2) [G0 + GN (-1)^x + 2 sum_{0<kx<N/2} Re(G(kx) exp(+2 pi i kx x / N))]
+    c2c_columns_inplace<N>(sm);
+    sm.twiddles(g_tw, false);
+    __syncthreads();
     float* o = out + (size_t)i * N * N;
     const float inv = 1.0f / ((float)N * N);
-    for (int p = threadIdx.x; p < N * N; p += blockDim.x) {
-        const int y = p / N, x = p - (p / N) * N;
-        const float2* G = F + y * H;
-        float v = G[0].x + ((x & 1) ? -G[N / 2].x : G[N / 2].x);
-        float acc = 0.f;
-        int idx = x;
-        for (int kx = 1; kx < N / 2; ++kx) {
-            const float2 w = tw[idx];          // exp(-2 pi i kx x / N); conjugated below
-            acc = fmaf(G[kx].x, w.x, fmaf(G[kx].y, w.y, acc));
-            idx += x;
-            idx -= (idx >= N) ? N : 0;
-        }
-        o[p] = (v + 2.f * acc) * inv;
-    }
+    c2r_rows<N>(sm, [&](int y, int x, float v) { o[y * N + x] = v * inv; });
 }
 
 // Real-space image of a stored unit-norm half spectrum S (Eq. 3, inverse transform):
@@ -497,60 +702,36 @@ __global__ void __launch_bounds__(kThreads) k_psf_real(const float* __restrict__
 // transforms above this is the zero-mean, unit-norm image whose correlations the scoring kernels
 // evaluate: sum_r o'(r) c'(r + d) = rho(d).  Writes x [N][N] and max |x|.
 template <int N>
-__global__ void __launch_bounds__(kThreads) k_spec_to_real(const float2* __restrict__ spec,
+__global__ void __launch_bounds__(Dft<N>::T) k_spec_to_real(const float2* __restrict__ spec,
                                                            const float2* __restrict__ g_tw, float* __restrict__ out,
                                                            float* __restrict__ amax) {
-    constexpr int H = N / 2 + 1;
+    constexpr int H = Dft<N>::H, TH = Dft<N>::T;
     extern __shared__ __align__(16) unsigned char smem[];
-    float2* F = reinterpret_cast<float2*>(smem);
-    float2* tw = F + N * H;
-    double* red = reinterpret_cast<double*>(tw + N);
+    const DftSm<N> sm(smem);
     const int i = blockIdx.x;
-    load_twiddles<N>(g_tw, tw);
+    sm.twiddles(g_tw, true);
     const float2* S = spec + (size_t)i * N * H;
-    for (int o = threadIdx.x; o < N * H; o += blockDim.x) F[o] = S[o];
+    for (int o = threadIdx.x; o < N * H; o += TH) sm.F[o] = S[o];
     __syncthreads();
-    c2c_columns_inplace<N, true>(F, tw);
+    c2c_columns_inplace<N>(sm);
+    sm.twiddles(g_tw, false);
+    __syncthreads();
     float* xo = out + (size_t)i * N * N;
     double e = 0.0, dummy = 0.0;
-    for (int p = threadIdx.x; p < N * N; p += blockDim.x) {
-        const int y = p / N, x = p - (p / N) * N;
-        const float2* G = F + y * H;
-        const float v = G[0].x + ((x & 1) ? -G[N / 2].x : G[N / 2].x);
-        float acc = 0.f;
-        int idx = x;
-        for (int kx = 1; kx < N / 2; ++kx) {
-            const float2 w = tw[idx];   // exp(-2 pi i kx x / N); conjugated below
-            acc = fmaf(G[kx].x, w.x, fmaf(G[kx].y, w.y, acc));
-            idx += x;
-            idx -= (idx >= N) ? N : 0;
-        }
-        const float r = v + 2.f * acc;
-        xo[p] = r;
-        e += (double)r * r;
-    }
-    block_sum2(e, dummy, red);
+    c2r_rows<N>(sm, [&](int y, int x, float v) {
+        xo[y * N + x] = v;
+        e += (double)v * v;
+    });
+    block_sum2<TH>(e, dummy, sm.red);   // its barriers also order the stores before the reads below
     const float scale = e > 0.0 ? (float)(1.0 / sqrt(e)) : 0.f;
     float mx = 0.f;
-    for (int p = threadIdx.x; p < N * N; p += blockDim.x) {   // the same elements this thread wrote
+    for (int p = threadIdx.x; p < N * N; p += TH) {
         const float r = xo[p] * scale;
         xo[p] = r;
         mx = fmaxf(mx, fabsf(r));
     }
-    float* redf = reinterpret_cast<float*>(red);
-    __syncthreads();
-    redf[threadIdx.x] = mx;
-    __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) redf[threadIdx.x] = fmaxf(redf[threadIdx.x], redf[threadIdx.x + st]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) amax[i] = redf[0];
-}
-
-template <int N>
-size_t fwd_smem() {
-    return (size_t)(N * (N / 2 + 1) + N) * sizeof(float2) + 2 * kThreads * sizeof(double);
+    mx = block_max<TH>(mx, reinterpret_cast<float*>(sm.red));
+    if (threadIdx.x == 0) amax[i] = mx;
 }
 
 template <int N>
@@ -583,7 +764,8 @@ int build_ctf_table(bioem_ctx* ctx, const bioem_ctf* ctfs, int nctf, int npix, d
     }
     e = cudaMemcpyAsync(d_coef, h, sizeof(double) * 3 * nctf, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) {
-        const int blocks = (int)((tsize + 255) / 256 < 4096 ? (tsize + 255) / 256 : 4096);
+        const size_t work = (tsize / 4 + 255) / 256 + 1;
+        const int blocks = (int)(work < 4096 ? work : 4096);
         bioem_launch_begin(ctx, KID_CTF_TABLE);
         k_ctf_table<<<blocks, 256, 0, ctx->stream>>>(d_coef, nctf, npix, pixel_A, *d_T);
         e = cudaGetLastError();
@@ -602,12 +784,13 @@ int build_ctf_table(bioem_ctx* ctx, const bioem_ctf* ctfs, int nctf, int npix, d
 
 template <int N>
 int launch_prepare_n(bioem_ctx* ctx, const float* d_images, bioem_images* im) {
-    const size_t sm = fwd_smem<N>();
-    if (set_smem<N>((const void*)k_prepare_images<N>, sm)) return bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");
+    const size_t sm = DftSm<N>::bytes();
+    auto kern = (uintptr_t)d_images % 16 == 0 ? k_prepare_images<N, true> : k_prepare_images<N, false>;
+    if (set_smem<N>((const void*)kern, sm)) return bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");
     const double cn = bioem_log_norm_constant(N * N);
     bioem_launch_begin(ctx, KID_PREPARE);
-    k_prepare_images<N><<<im->n_img, kThreads, sm, ctx->stream>>>(d_images, bioem_twiddles(ctx, N), im->d_spec,
-                                                                    im->d_kA, im->d_amax, cn, ctx->d_status);
+    kern<<<im->n_img, Dft<N>::T, sm, ctx->stream>>>(d_images, bioem_twiddles(ctx, N), im->d_spec, im->d_kA,
+                                                    im->d_amax, cn, ctx->d_status);
     bioem_launch_end(ctx, KID_PREPARE);
     return bioem_check_cuda(ctx, cudaGetLastError(), "k_prepare_images");
 }
@@ -626,7 +809,7 @@ int launch_project_n(bioem_ctx* ctx, const float* d_atoms, int n_atoms, double s
         cudaFreeAsync(d_T, ctx->stream);
         return bioem_set_error(ctx, BIOEM_ERR_OOM, "cudaMallocAsync(projection scratch)");
     }
-    const size_t sm = fwd_smem<N>();
+    const size_t sm = DftSm<N>::bytes();
     if (set_smem<N>((const void*)k_project<N>, ProjCfg<N>::SMEM) || set_smem<N>((const void*)k_psf_spectra<N>, sm)) rc = bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");
     for (int q0 = 0; q0 < nq && rc == BIOEM_OK; q0 += qw) {
         const int nb = nq - q0 < qw ? nq - q0 : qw;
@@ -639,7 +822,7 @@ int launch_project_n(bioem_ctx* ctx, const float* d_atoms, int n_atoms, double s
         if (rc) break;
         const size_t p0 = (size_t)q0 * nctf;
         bioem_launch_begin(ctx, KID_PSF_SPECTRA);
-        k_psf_spectra<N><<<nb, kThreads, sm, ctx->stream>>>(d_I0, bioem_twiddles(ctx, N), d_T, nctf,
+        k_psf_spectra<N><<<nb, Dft<N>::T, sm, ctx->stream>>>(d_I0, bioem_twiddles(ctx, N), d_T, nctf,
                                                              ps->d_spec + p0 * N * (N / 2 + 1), ps->d_kB + p0,
                                                              ps->d_amax + p0, ctx->d_status);
         bioem_launch_end(ctx, KID_PSF_SPECTRA);
@@ -671,11 +854,11 @@ int launch_synthetic_n(bioem_ctx* ctx, const float* d_atoms, int n_atoms, double
                                                    reinterpret_cast<const float4*>(d_quats), sigma_A, pixel_A, d_I0);
     bioem_launch_end(ctx, KID_PROJECT);
     rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_project");
-    const size_t sm = fwd_smem<N>();
+    const size_t sm = DftSm<N>::bytes();
     if (!rc && set_smem<N>((const void*)k_psf_real<N>, sm)) rc = bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");
     if (!rc) {
         bioem_launch_begin(ctx, KID_PSF_REAL);
-        k_psf_real<N><<<n, kThreads, sm, ctx->stream>>>(d_I0, bioem_twiddles(ctx, N), d_T, d_out);
+        k_psf_real<N><<<n, Dft<N>::T, sm, ctx->stream>>>(d_I0, bioem_twiddles(ctx, N), d_T, d_out);
         bioem_launch_end(ctx, KID_PSF_REAL);
         rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_psf_real");
     }
@@ -686,10 +869,10 @@ int launch_synthetic_n(bioem_ctx* ctx, const float* d_atoms, int n_atoms, double
 
 template <int N>
 int launch_spec_to_real_n(bioem_ctx* ctx, const float2* spec, int count, float* out, float* amax) {
-    const size_t sm = fwd_smem<N>();
+    const size_t sm = DftSm<N>::bytes();
     if (set_smem<N>((const void*)k_spec_to_real<N>, sm)) return bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");
     bioem_launch_begin(ctx, KID_GEMM_OPS);
-    k_spec_to_real<N><<<count, kThreads, sm, ctx->stream>>>(spec, bioem_twiddles(ctx, N), out, amax);
+    k_spec_to_real<N><<<count, Dft<N>::T, sm, ctx->stream>>>(spec, bioem_twiddles(ctx, N), out, amax);
     bioem_launch_end(ctx, KID_GEMM_OPS);
     return bioem_check_cuda(ctx, cudaGetLastError(), "k_spec_to_real");
 }
