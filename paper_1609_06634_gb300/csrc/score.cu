@@ -672,97 +672,192 @@ struct Acc {
     int bd;      // its displacement index
 };
 
-__device__ __forceinline__ void acc_add(Acc& a, double m, double s, int p, int d) {
-    if (!(m > -INFINITY)) return;
-    if (m > a.M) {
-        a.S = a.S * exp(a.M - m) + s;
-        a.M = m;
-    } else {
-        a.S += s * exp(m - a.M);
-    }
-    if (m > a.bv || (m == a.bv && p < a.bp)) {
-        a.bv = m;
-        a.bp = p;
-        a.bd = d;
-    }
-}
-
-__device__ __forceinline__ void acc_merge(Acc& a, const Acc& b) {
-    if (b.M > -INFINITY) {
-        if (b.M > a.M) {
-            a.S = a.S * exp(a.M - b.M) + b.S;
-            a.M = b.M;
-        } else {
-            a.S += b.S * exp(b.M - a.M);
-        }
-    }
-    if (b.bv > a.bv || (b.bv == a.bv && b.bp < a.bp)) {
-        a.bv = b.bv;
-        a.bp = b.bp;
-        a.bd = b.bd;
-    }
-}
-
 constexpr int kRedThreads = 256;
+constexpr int kExpBits = 6;   // table of 2^(j / 64)
+constexpr double kExpMin = -100.0;
 
-// One block per image: fold the wave's pair records into the image's running accumulator and,
-// if requested, write the per-orientation posteriors of the wave's orientations.
+// exp(x) for x in [kExpMin, 0]: x = (64 q + j) ln2 / 64 + r, |r| <= ln2 / 128, exp(x) = 2^q 2^(j/64) e^r with the Taylor
+// series of e^r to r^5 (truncation below 4e-17), the table-driven scheme of Tang (ACM TOMS 15, 1989).  Ten
+// float64 operations; the reductions below are bound by the float64 pipe (1/70 of the FP32 rate).
+__device__ __forceinline__ double exp_neg(double x, const double* tab) {
+    const double big = 6755399441055744.0;   // 1.5 * 2^52: adding it rounds to an integer in the low word
+    const double kd = fma(x, 92.33248261689366, big);   // 64 / ln 2
+    const int k = __double2loint(kd);
+    const double n = kd - big;
+    double r = fma(n, -1.0830424696249145e-2, x);            // ln 2 / 64, leading part and the rest
+    r = fma(n, -3.623510646634843e-19, r);
+    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    p = fma(r, p, 1.0 / 6.0);
+    p = fma(r, p, 0.5);
+    p = fma(r, p, 1.0);
+    const double t = tab[k & 63];
+    const double v = fma(t, r * p, t);
+    return __hiloint2double(__double2hiint(v) + (k >> kExpBits) * (1 << 20), __double2loint(v));
+}
+
+// Folds four terms s_i exp(m_i) (m = -inf: none) into (M, S), ln sum = M + ln S; returns the index of the first
+// term that is a new maximum, or -1.  Terms more than 100 below the maximum cannot change S (S >= 1: the
+// maximum's own s is at least 1) and are left out.
+__device__ __forceinline__ int lse_add4(double& M, double& S, const double (&m)[4], const float (&s)[4], const double* tab) {
+    int at = -1;
+    const double mx = fmax(fmax(m[0], m[1]), fmax(m[2], m[3]));
+    if (mx > M) {
+        at = m[0] == mx ? 0 : m[1] == mx ? 1 : m[2] == mx ? 2 : 3;
+        S = M - mx > kExpMin ? S * exp_neg(M - mx, tab) : 0.0;
+        M = mx;
+    }
+    bool any = false;
+    double d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        d[i] = m[i] - M;
+        any |= d[i] > kExpMin;
+    }
+    if (__any_sync(__activemask(), any)) {
+        double e[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) e[i] = exp_neg(d[i] > kExpMin ? d[i] : 0.0, tab);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) S = fma(d[i] > kExpMin ? (double)s[i] : 0.0, e[i], S);
+    }
+    return at;
+}
+
+__device__ __forceinline__ void exp_table(double* tab) {
+    if (threadIdx.x < (1 << kExpBits)) tab[threadIdx.x] = exp2((double)threadIdx.x / (1 << kExpBits));
+}
+
+// The warp's (M, S, best set) merged into every lane, lanes in a fixed order; bp = the lowest set of the maximum.
+__device__ __forceinline__ void warp_lse(double& M, double& S, int& bp) {
+    double mx = M;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    S = (M > -INFINITY) ? S * exp(M - mx) : 0.0;
+    if (!(M == mx)) bp = 0x7fffffff;
+    M = mx;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        S += __shfl_xor_sync(0xffffffffu, S, off);
+        bp = min(bp, __shfl_xor_sync(0xffffffffu, bp, off));
+    }
+}
+
+// The same over a block of kRedThreads, valid in warp 0.
+__device__ __forceinline__ void block_lse(double& M, double& S, int& bp) {
+    constexpr int W = kRedThreads / 32;
+    __shared__ double rM[W], rS[W];
+    __shared__ int rb[W];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    warp_lse(M, S, bp);
+    if (lane == 0) { rM[warp] = M; rS[warp] = S; rb[warp] = bp; }
+    __syncthreads();
+    if (warp == 0) {
+        M = lane < W ? rM[lane] : -INFINITY;
+        S = lane < W ? rS[lane] : 0.0;
+        bp = lane < W ? rb[lane] : 0x7fffffff;
+        warp_lse(M, S, bp);
+    }
+}
+
+// r merged with the running accumulator of earlier waves (which hold the lower parameter sets).
+__device__ __forceinline__ void acc_merge_prev(Acc& r, const Acc& prev) {
+    if (!(prev.M > -INFINITY)) return;
+    if (r.M > prev.M) {
+        r.S += prev.S * exp(prev.M - r.M);
+    } else {
+        r.S = r.M > -INFINITY ? prev.S + r.S * exp(r.M - prev.M) : prev.S;
+        r.M = prev.M;
+    }
+    if (prev.bv >= r.bv) { r.bv = prev.bv; r.bp = prev.bp; r.bd = prev.bd; }
+}
+
+// One block per (image, part): fold the part's share of the wave's pair records into parts[image][part]
+// and, if requested, write the per-orientation posteriors of the share's orientations.  Parts are whole
+// orientations; an image is cut into enough of them to occupy the GPU (reduce_parts).  An image in one part
+// is folded in place (parts = prev = the running accumulators; prev null: the first wave).  Bound by the
+// float64 pipe: one exponential per record for each of the two outputs (REDUCE_NOTE).
 __global__ void __launch_bounds__(kRedThreads) k_reduce_wave(
     const float* __restrict__ rec_t, const float* __restrict__ rec_s, const int* __restrict__ rec_d,
     const double* __restrict__ kA, const double* __restrict__ kB, int ps_begin, int wave_len, int nctf,
-    int nq, double c1, double log_norm_orient, Acc* __restrict__ acc, int first, double* __restrict__ logP_orient) {
-    __shared__ Acc red[kRedThreads];
-    const int w = blockIdx.x;
+    int nq, double c1, double log_norm_orient, Acc* parts, int n_parts, const Acc* prev,
+    double* __restrict__ logP_orient) {
+    __shared__ double tab[1 << kExpBits];
+    const int w = blockIdx.x / n_parts, part = blockIdx.x - w * n_parts;
+    const int q_all = wave_len / nctf, q_per = (q_all + n_parts - 1) / n_parts;
+    const int q0 = min(part * q_per, q_all), q1 = min(q0 + q_per, q_all);
     const double ka = kA[w];
-    Acc a{-INFINITY, 0.0, -INFINITY, 0x7fffffff, 0};
     const size_t base = (size_t)w * wave_len;
-    for (int p = threadIdx.x; p < wave_len; p += blockDim.x) {
-        const double m = ka + kB[ps_begin + p] + c1 * (double)rec_t[base + p];
-        acc_add(a, m, (double)rec_s[base + p], ps_begin + p, rec_d[base + p]);
-    }
-    red[threadIdx.x] = a;
+    exp_table(tab);
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) acc_merge(red[threadIdx.x], red[threadIdx.x + st]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        Acc r = red[0];
-        if (!first) {
-            Acc prev = acc[w];
-            acc_merge(prev, r);
-            r = prev;
+    double M = -INFINITY, S = 0.0;
+    int bp = 0x7fffffff;
+    const int lo = q0 * nctf, hi = q1 * nctf;
+    for (int p = lo + threadIdx.x; p < hi; p += 4 * kRedThreads) {
+        double m[4];
+        float sv[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int pi = p + i * kRedThreads;
+            m[i] = pi < hi ? ka + kB[ps_begin + pi] + c1 * (double)rec_t[base + pi] : -INFINITY;
+            sv[i] = pi < hi ? rec_s[base + pi] : 0.f;
         }
-        acc[w] = r;
+        const int at = lse_add4(M, S, m, sv, tab);
+        if (at >= 0) bp = p + at * kRedThreads;
+    }
+    block_lse(M, S, bp);
+    if (threadIdx.x == 0) {
+        const bool any = bp != 0x7fffffff;
+        Acc r{M, S, any ? M : -INFINITY, any ? ps_begin + bp : 0x7fffffff, any ? rec_d[base + bp] : 0};
+        if (prev) acc_merge_prev(r, prev[w]);
+        parts[blockIdx.x] = r;
     }
     if (logP_orient) {
-        const int q0 = ps_begin / nctf;
-        for (int ql = threadIdx.x; ql < wave_len / nctf; ql += blockDim.x) {
-            double M = -INFINITY, S = 0.0;
-            for (int c = 0; c < nctf; ++c) {
-                const int p = ql * nctf + c;
-                const double m = ka + kB[ps_begin + p] + c1 * (double)rec_t[base + p];
-                const double s = rec_s[base + p];
-                if (!(m > -INFINITY)) continue;
-                if (m > M) { S = S * exp(M - m) + s; M = m; }
-                else S += s * exp(m - M);
+        for (int ql = q0 + threadIdx.x; ql < q1; ql += kRedThreads) {
+            double Mq = -INFINITY, Sq = 0.0;
+            for (int c = 0; c < nctf; c += 4) {
+                double m[4];
+                float sv[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int p = ql * nctf + c + i;
+                    m[i] = c + i < nctf ? ka + kB[ps_begin + p] + c1 * (double)rec_t[base + p] : -INFINITY;
+                    sv[i] = c + i < nctf ? rec_s[base + p] : 0.f;
+                }
+                lse_add4(Mq, Sq, m, sv, tab);
             }
-            logP_orient[(size_t)w * nq + q0 + ql] = M + log(S) - log_norm_orient;
+            logP_orient[(size_t)w * nq + ps_begin / nctf + ql] = Mq + log(Sq) - log_norm_orient;
         }
     }
 }
 
-__global__ void k_finalize(const Acc* __restrict__ acc, int n_img, double log_norm, int nctf, int nsk, int smax,
-                           double* logP, int* best_q, int* best_ctf, int* best_dx, int* best_dy, double* best_logL) {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+// One warp per image: the wave's parts (at most 32, one per lane) and, unless this is the first wave, the
+// running accumulator, merged into acc[image]; after the last wave the outputs.  parts null: acc is complete.
+__global__ void __launch_bounds__(kRedThreads) k_finalize(Acc* acc, const Acc* parts,
+                                                          int n_parts, int first, int last, int n_img, double log_norm,
+                                                          int nctf, int nsk, int smax, double* logP, int* best_q,
+                                                          int* best_ctf, int* best_dx, int* best_dy, double* best_logL) {
+    const int w = blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (w >= n_img) return;
-    const Acc a = acc[w];
-    if (logP) logP[w] = a.M + log(a.S) - log_norm;
-    if (best_q) best_q[w] = a.bp / nctf;
-    if (best_ctf) best_ctf[w] = a.bp % nctf;
-    if (best_dy) best_dy[w] = a.bd / nsk - smax;
-    if (best_dx) best_dx[w] = a.bd % nsk - smax;
-    if (best_logL) best_logL[w] = a.bv;
+    Acc a{-INFINITY, 0.0, -INFINITY, 0x7fffffff, 0};
+    if (lane < n_parts) a = (parts ? parts : acc)[(size_t)w * n_parts + lane];
+    Acc prev{-INFINITY, 0.0, -INFINITY, 0x7fffffff, 0};
+    if (!first) prev = acc[w];
+    double M = a.M, S = a.S;
+    int bp = a.bp;
+    warp_lse(M, S, bp);
+    const int src = __ffs(__ballot_sync(0xffffffffu, bp != 0x7fffffff && a.bp == bp)) - 1;
+    const int bd = __shfl_sync(0xffffffffu, a.bd, src < 0 ? 0 : src);
+    if (lane != 0) return;
+    Acc r{M, S, bp != 0x7fffffff ? M : -INFINITY, bp, bd};
+    acc_merge_prev(r, prev);
+    acc[w] = r;
+    if (!last) return;
+    if (logP) logP[w] = r.M + log(r.S) - log_norm;
+    if (best_q) best_q[w] = r.bp / nctf;
+    if (best_ctf) best_ctf[w] = r.bp % nctf;
+    if (best_dy) best_dy[w] = r.bd / nsk - smax;
+    if (best_dx) best_dx[w] = r.bd % nsk - smax;
+    if (best_logL) best_logL[w] = r.bv;
 }
 
 // pair_max[w][col0 + p] = max_d ln L and pair_lse[w][col0 + p] = ln sum_d L for the wave's records.
@@ -799,6 +894,45 @@ __global__ void k_fold_acc(const Acc* __restrict__ acc, int n_img, double* __res
 }
 
 // ---------------------------------------------------------------------------- host side
+// Parts per image of the wave reduction: about four blocks per SM over all images, each of at least 512
+// records and one orientation, at most 32 (one lane each in k_finalize).
+int reduce_parts(const bioem_ctx* ctx, int n_img, long long wave, int nctf) {
+    long long n = 4ll * ctx->num_sms / n_img;
+    if (n > wave / 512) n = wave / 512;
+    if (n > wave / nctf) n = wave / nctf;
+    return (int)(n < 1 ? 1 : n > 32 ? 32 : n);
+}
+
+// Accumulators and parts of n_img images in one array: [n_img] accumulators, then with more than one part
+// per image [n_img][n_parts].
+size_t reduce_bytes(int n_img, int n_parts) {
+    return sizeof(Acc) * (size_t)n_img * (n_parts > 1 ? 1 + n_parts : 1);
+}
+
+// The reductions of one wave's records into acc (laid out as in reduce_bytes), and after the last wave the
+// outputs.
+int launch_reduce(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, int max_shift, int smax, int wbegin,
+                  int wl, const float* rec_t, const float* rec_s, const int* rec_d, Acc* acc, int n_parts, bool first,
+                  bool last, const bioem_score_out& out) {
+    const int n_img = im->n_img, nctf = ps->nctf;
+    Acc* parts = n_parts > 1 ? acc + n_img : nullptr;
+    const double c1 = 0.5 * (3.0 - (double)(im->nx * im->ny));
+    const int S = (2 * max_shift + 1) * (2 * max_shift + 1);
+    bioem_launch_begin(ctx, KID_REDUCE_WAVE);
+    k_reduce_wave<<<n_img * n_parts, kRedThreads, 0, ctx->stream>>>(rec_t, rec_s, rec_d, im->d_kA, ps->d_kB, wbegin, wl,
+                                                                    nctf, ps->nq, c1, log((double)nctf * S),
+                                                                    parts ? parts : acc, n_parts,
+                                                                    parts || first ? nullptr : acc, out.logP_orient);
+    bioem_launch_end(ctx, KID_REDUCE_WAVE);
+    if (!parts && !last) return bioem_check_cuda(ctx, cudaGetLastError(), "reduction");
+    bioem_launch_begin(ctx, KID_FINALIZE);
+    k_finalize<<<(n_img + kRedThreads / 32 - 1) / (kRedThreads / 32), kRedThreads, 0, ctx->stream>>>(
+        acc, parts, n_parts, first || !parts, last, n_img, log((double)ps->n_ps * S), nctf, 2 * smax + 1, smax, out.logP,
+        out.best_q, out.best_ctf, out.best_dx, out.best_dy, out.best_logL);
+    bioem_launch_end(ctx, KID_FINALIZE);
+    return bioem_check_cuda(ctx, cudaGetLastError(), "reduction");
+}
+
 // The wave loop shared by the scoring forms: parameter sets [range) in waves whose per-pair records
 // (n_img x wave) fit the scratch limit; `records(wbegin, wl, rec_t, rec_s, rec_d)` enqueues the
 // kernel(s) writing the records of sets [wbegin, wbegin + wl), then the float64 reductions fold
@@ -811,7 +945,6 @@ int run_waves(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, i
               const bioem_score_out& out, Records&& records) {
     const int n_img = im->n_img;
     const int n = im->nx * im->ny;
-    const int nsk = 2 * smax + 1;
     const bool pairs_mode = out.pair_max != nullptr;
     const int range_begin = pairs_mode ? out.ps_begin : 0;
     const int range_len = pairs_mode ? out.ps_count : ps->n_ps;
@@ -835,7 +968,8 @@ int run_waves(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, i
             return bioem_set_error(ctx, BIOEM_ERR_OOM, "record scratch of %zu bytes", rec_need);
         ctx->rec_bytes = rec_need;
     }
-    const size_t acc_need = sizeof(Acc) * (size_t)n_img;
+    const int n_parts = pairs_mode ? 1 : reduce_parts(ctx, n_img, wave, nctf);
+    const size_t acc_need = reduce_bytes(n_img, n_parts);
     if (!pairs_mode && ctx->acc_bytes < acc_need) {
         if (ctx->d_acc) cudaFreeAsync(ctx->d_acc, ctx->stream);
         ctx->d_acc = nullptr;
@@ -848,7 +982,7 @@ int run_waves(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, i
     float* rec_s = rec_t + (size_t)n_img * wave;
     int* rec_d = reinterpret_cast<int*>(rec_s + (size_t)n_img * wave);
     const double c1 = 0.5 * (3.0 - (double)n);
-    const int S = (2 * max_shift + 1) * (2 * max_shift + 1);
+    Acc* acc = reinterpret_cast<Acc*>(ctx->d_acc);
 
     for (long long w0 = 0; w0 < range_len; w0 += wave) {
         const int wl = (int)(range_len - w0 < wave ? range_len - w0 : wave);
@@ -861,31 +995,19 @@ int run_waves(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, i
                                                        out.pair_max, out.pair_lse, range_len, (int)w0);
             bioem_launch_end(ctx, KID_PAIRS_OUT);
         } else {
-            const double log_norm_orient = log((double)nctf * S);
-            bioem_launch_begin(ctx, KID_REDUCE_WAVE);
-            k_reduce_wave<<<n_img, kRedThreads, 0, ctx->stream>>>(rec_t, rec_s, rec_d, im->d_kA, ps->d_kB, wbegin, wl,
-                                                                  nctf, ps->nq, c1, log_norm_orient,
-                                                                  reinterpret_cast<Acc*>(ctx->d_acc), w0 == 0,
-                                                                  out.logP_orient);
-            bioem_launch_end(ctx, KID_REDUCE_WAVE);
+            rc = launch_reduce(ctx, im, ps, max_shift, smax, wbegin, wl, rec_t, rec_s, rec_d, acc, n_parts,
+                               w0 == 0, w0 + wl == range_len, out);
         }
-        rc = bioem_check_cuda(ctx, cudaGetLastError(), "reduction");
+        if (!rc) rc = bioem_check_cuda(ctx, cudaGetLastError(), "reduction");
         if (rc) return rc;
     }
     if (!pairs_mode) {
-        const double log_norm = log((double)ps->n_ps * S);
-        bioem_launch_begin(ctx, KID_FINALIZE);
-        k_finalize<<<(n_img + 255) / 256, 256, 0, ctx->stream>>>(reinterpret_cast<const Acc*>(ctx->d_acc), n_img, log_norm,
-                                                                  nctf, nsk, smax, out.logP, out.best_q, out.best_ctf,
-                                                                  out.best_dx, out.best_dy, out.best_logL);
-        bioem_launch_end(ctx, KID_FINALIZE);
         if (out.acc2) {
             bioem_launch_begin(ctx, KID_FINALIZE);
-            k_fold_acc<<<(n_img + 255) / 256, 256, 0, ctx->stream>>>(reinterpret_cast<const Acc*>(ctx->d_acc), n_img,
-                                                                     out.acc2, out.acc_first);
+            k_fold_acc<<<(n_img + 255) / 256, 256, 0, ctx->stream>>>(acc, n_img, out.acc2, out.acc_first);
             bioem_launch_end(ctx, KID_FINALIZE);
         }
-        return bioem_check_cuda(ctx, cudaGetLastError(), "k_finalize");
+        return bioem_check_cuda(ctx, cudaGetLastError(), "k_fold_acc");
     }
     return BIOEM_OK;
 }
@@ -1106,38 +1228,35 @@ int run_score_noalloc(bioem_ctx* ctx, const bioem_images* im, const bioem_projse
     void* base = nullptr;
     int rc = noalloc_scratch(ctx, &base);
     if (rc) return rc;
-    long long wave = (long long)((kNoAllocBytes - acc_bytes) / per_ps);
+    // the reduction's parts follow the accumulators where they leave the records room
+    int n_parts = reduce_parts(ctx, n_img, ps->n_ps, nctf);
+    size_t head = (reduce_bytes(n_img, n_parts) + 255) / 256 * 256;
+    if (head + per_ps * nctf > kNoAllocBytes) {
+        n_parts = 1;
+        head = acc_bytes;
+    }
+    long long wave = (long long)((kNoAllocBytes - head) / per_ps);
     wave -= wave % nctf;
     if (wave > ps->n_ps) wave = ps->n_ps;
     Acc* acc = reinterpret_cast<Acc*>(base);
-    float* rec_t = reinterpret_cast<float*>(static_cast<unsigned char*>(base) + acc_bytes);
+    float* rec_t = reinterpret_cast<float*>(static_cast<unsigned char*>(base) + head);
     float* rec_s = rec_t + (size_t)n_img * wave;
     int* rec_d = reinterpret_cast<int*>(rec_s + (size_t)n_img * wave);
 
     int slots = 0;
     rc = score_slots<C>(ctx, &slots);
     if (rc) return rc;
-    const int n = C::N * C::N;
-    const double c1 = 0.5 * (3.0 - (double)n);
-    const int S = (2 * max_shift + 1) * (2 * max_shift + 1);
+    bioem_score_out out{};
+    out.logP = logP;
     for (long long w0 = 0; w0 < ps->n_ps; w0 += wave) {
         const int wl = (int)(ps->n_ps - w0 < wave ? ps->n_ps - w0 : wave);
         rc = launch_score_records<C>(ctx, im, ps, slots, (int)w0, wl, max_shift, rec_t, rec_s, rec_d);
-        if (rc) return rc;
-        bioem_launch_begin(ctx, KID_REDUCE_WAVE);
-        k_reduce_wave<<<n_img, kRedThreads, 0, ctx->stream>>>(rec_t, rec_s, rec_d, im->d_kA, ps->d_kB, (int)w0, wl,
-                                                              nctf, ps->nq, c1, log((double)nctf * S), acc, w0 == 0,
-                                                              nullptr);
-        bioem_launch_end(ctx, KID_REDUCE_WAVE);
-        rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_reduce_wave");
+        if (!rc)
+            rc = launch_reduce(ctx, im, ps, max_shift, C::SMAX, (int)w0, wl, rec_t, rec_s, rec_d, acc, n_parts, w0 == 0,
+                               w0 + wl == ps->n_ps, out);
         if (rc) return rc;
     }
-    bioem_launch_begin(ctx, KID_FINALIZE);
-    k_finalize<<<(n_img + 255) / 256, 256, 0, ctx->stream>>>(acc, n_img, log((double)ps->n_ps * S), nctf, C::NS,
-                                                              C::SMAX, logP, nullptr, nullptr, nullptr, nullptr,
-                                                              nullptr);
-    bioem_launch_end(ctx, KID_FINALIZE);
-    return bioem_check_cuda(ctx, cudaGetLastError(), "k_finalize");
+    return BIOEM_OK;
 }
 
 }  // namespace
@@ -1264,40 +1383,32 @@ k_score_multi(const SegDesc* __restrict__ segs, int n_segs, long long n_items, i
 // into out[model][column].
 __global__ void __launch_bounds__(kRedThreads) k_reduce_multi(const SegDesc* __restrict__ segs, int n_segs,
                                                               float* __restrict__ out, int out_ld) {
-    __shared__ double redM[kRedThreads], redS[kRedThreads];
+    __shared__ double tab[1 << kExpBits];
     const long long row = blockIdx.x;
     const int g = find_seg(segs, n_segs, row, true);
     const SegDesc& sd = segs[g];
     const int w = (int)(row - sd.row_begin);
     const double ka = sd.kA[w];
     const double c1 = (double)sd.c1;
-    double M = -INFINITY, S = 0.0;
-    const size_t base = (size_t)w * sd.n_ps;
-    for (int p = threadIdx.x; p < sd.n_ps; p += blockDim.x) {
-        const double m = ka + sd.kB[p] + c1 * (double)sd.rec_t[base + p];
-        const double s = sd.rec_s[base + p];
-        if (!(m > -INFINITY)) continue;
-        if (m > M) { S = S * exp(M - m) + s; M = m; }
-        else S += s * exp(m - M);
-    }
-    redM[threadIdx.x] = M;
-    redS[threadIdx.x] = S;
+    exp_table(tab);
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) {
-            const double m2 = redM[threadIdx.x + st], s2 = redS[threadIdx.x + st];
-            double m1 = redM[threadIdx.x], s1 = redS[threadIdx.x];
-            if (m2 > -INFINITY) {
-                if (m2 > m1) { s1 = s1 * exp(m1 - m2) + s2; m1 = m2; }
-                else s1 += s2 * exp(m2 - m1);
-            }
-            redM[threadIdx.x] = m1;
-            redS[threadIdx.x] = s1;
+    double M = -INFINITY, S = 0.0;
+    int bp = 0x7fffffff;
+    const size_t base = (size_t)w * sd.n_ps;
+    for (int p = threadIdx.x; p < sd.n_ps; p += 4 * kRedThreads) {
+        double m[4];
+        float sv[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int pi = p + i * kRedThreads;
+            m[i] = pi < sd.n_ps ? ka + sd.kB[pi] + c1 * (double)sd.rec_t[base + pi] : -INFINITY;
+            sv[i] = pi < sd.n_ps ? sd.rec_s[base + pi] : 0.f;
         }
-        __syncthreads();
+        lse_add4(M, S, m, sv, tab);
     }
+    block_lse(M, S, bp);
     if (threadIdx.x == 0)
-        out[(size_t)sd.out_row * out_ld + sd.out_col + w] = (float)(redM[0] + log(redS[0]) - sd.log_norm);
+        out[(size_t)sd.out_row * out_ld + sd.out_col + w] = (float)(M + log(S) - sd.log_norm);
 }
 
 struct TuneEntry {
@@ -1705,44 +1816,30 @@ __global__ void __launch_bounds__(kRedThreads) k_fold_gathered(const int* __rest
                                                                const double* __restrict__ kA,
                                                                const double* __restrict__ kB, double c1,
                                                                double* __restrict__ acc, int first) {
-    __shared__ double redM[kRedThreads], redS[kRedThreads];
+    __shared__ double tab[1 << kExpBits];
     const int w = blockIdx.x;
     const int b0 = offsets[w], b1 = offsets[w + 1];
-    double M = -INFINITY, S = 0.0;
-    for (int i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
-        const double m = kA[w] + kB[ps_idx[i]] + c1 * (double)rec_t[i];
-        const double sv = rec_s[i];
-        if (!(m > -INFINITY)) continue;
-        if (m > M) { S = S * exp(M - m) + sv; M = m; }
-        else S += sv * exp(m - M);
-    }
-    redM[threadIdx.x] = M;
-    redS[threadIdx.x] = S;
+    exp_table(tab);
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) {
-            const double m2 = redM[threadIdx.x + st], s2 = redS[threadIdx.x + st];
-            double m1 = redM[threadIdx.x], s1 = redS[threadIdx.x];
-            if (m2 > -INFINITY) {
-                if (m2 > m1) { s1 = s1 * exp(m1 - m2) + s2; m1 = m2; }
-                else s1 += s2 * exp(m2 - m1);
-            }
-            redM[threadIdx.x] = m1;
-            redS[threadIdx.x] = s1;
+    double M = -INFINITY, S = 0.0;
+    int bp = 0x7fffffff;
+    for (int i0 = b0 + threadIdx.x; i0 < b1; i0 += 4 * kRedThreads) {
+        double m[4];
+        float sv[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = i0 + k * kRedThreads;
+            m[k] = i < b1 ? kA[w] + kB[ps_idx[i]] + c1 * (double)rec_t[i] : -INFINITY;
+            sv[k] = i < b1 ? rec_s[i] : 0.f;
         }
-        __syncthreads();
+        lse_add4(M, S, m, sv, tab);
     }
+    block_lse(M, S, bp);
     if (threadIdx.x == 0) {
-        double m1 = redM[0], s1 = redS[0];
-        if (!first) {
-            const double m2 = acc[2 * w], s2 = acc[2 * w + 1];
-            if (m2 > -INFINITY) {
-                if (m2 > m1) { s1 = s1 * exp(m1 - m2) + s2; m1 = m2; }
-                else s1 += s2 * exp(m2 - m1);
-            }
-        }
-        acc[2 * w] = m1;
-        acc[2 * w + 1] = s1;
+        Acc r{M, S, -INFINITY, 0, 0};
+        if (!first) acc_merge_prev(r, Acc{acc[2 * w], acc[2 * w + 1], -INFINITY, 0, 0});
+        acc[2 * w] = r.M;
+        acc[2 * w + 1] = r.S;
     }
 }
 
