@@ -134,87 +134,76 @@ __host__ __device__ constexpr int bitrev(int u, int bits) {
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
 __host__ __device__ constexpr int pmod(int a, int m) { return ((a % m) + m) % m; }
 
-template <int N_, int SMAX_, int PB_, int THREADS_, bool ALLOW_PACK_ = true, int BSPLIT_ = 1>
+template <int N_, int SMAX_, int NG_, int GT_, int GPB_, bool PACK_, int BSPLIT_ = 1>
 struct Cfg {
     static constexpr int N = N_;
     static constexpr int SMAX = SMAX_;
-    static constexpr int PB = PB_;             // pairs per batch
     static constexpr int NC = N / 2;
     static constexpr int H = NC + 1;           // half-spectrum row length (kx = 0..N/2)
     static constexpr int NS = 2 * SMAX + 1;    // displacements per axis
     static constexpr int NROW = 2 * SMAX;      // stage-B transform rows per pair (dy < SMAX)
     static constexpr int R = N / L;            // sub-sequences per transform
-    static constexpr int THREADS = THREADS_;   // threads doing the work (a block may have more)
-    static constexpr int NWARPS = THREADS / 32;  // full warps (combine step)
-    // stage-B threads per row: 2 when the block has two threads for every row (each sums half
-    // of the sub-sequences, the halves are exchanged by a lane shuffle, and each evaluates the
-    // likelihood for half of the dx outputs)
-    static constexpr int BSPLIT = BSPLIT_;
-    static_assert((BSPLIT == 1 || BSPLIT == 2) && THREADS >= PB * 2 * SMAX_ * BSPLIT, "stage-B threads");
-    static constexpr bool PREFETCH = THREADS <= 320;   // stage-A projection prefetch (registers)
-    static_assert(THREADS >= PB * NROW, "one stage-B row per thread");
-    static_assert(NWARPS >= 1, "at least one full warp");
     static_assert(N % L == 0, "sub-transform length divides N");
+    // Decoupled groups: the block's threads form NGROUP groups of GT threads.  A group takes batches of
+    // GPB pairs from the item's counter and runs all their phases (packed edge columns, stage A, stage B,
+    // the dy = +SMAX row, the combine) by itself, waiting only on its own named barrier, so that one
+    // group's projection loads, barrier waits and short phases overlap the others' transform arithmetic.
+    // The image spectrum and the twiddle tables are shared by the block.
+    static constexpr int NGROUP = NG_, GT = GT_, GPB = GPB_;
+    static constexpr int THREADS = NGROUP * GT;
+    static constexpr int PB = NGROUP * GPB;    // pairs in flight per block
+    static_assert(GT % 32 == 0 && THREADS <= 1024 && NGROUP <= 15, "whole warps; named barriers 1 .. 15");
+    // stage-B threads per row: 2 when the group has two threads for every row (each sums half of the
+    // sub-sequences, the halves are exchanged by a lane shuffle, and each evaluates the likelihood
+    // for half of the dx outputs)
+    static constexpr int BSPLIT = BSPLIT_;
+    static constexpr int ROWS = GPB * NROW * BSPLIT;   // stage-B tasks per batch
+    static_assert(BSPLIT == 1 || (BSPLIT == 2 && ROWS == GT), "split rows: one per thread");
+    static constexpr bool PREFETCH = THREADS <= 320;   // stage-A projection prefetch (registers)
     static constexpr int QS = H;               // Q row stride (complex); odd -> conflict-free columns
-    static constexpr int NDIR = PB * NS;       // outputs of the dy = +SMAX row, evaluated directly
+    static constexpr int NDIR = GPB * NS;      // outputs of the dy = +SMAX row, evaluated directly
     static constexpr size_t SM_IMG = (size_t)N * H * sizeof(float2);
     static constexpr size_t SM_Q = (size_t)PB * NS * QS * sizeof(float2);
     static constexpr size_t SM_QA = (SM_Q + 15) / 16 * 16;   // the twiddle table starts 16-byte aligned
     // twiddle table twc[b][d] = W_N^(b d), d = 0..SMAX (the outputs -d use the conjugate), rows of
     // an even length TWS so that pairs (d, d + 1), d even, are read as one 16-byte load
     static constexpr int TWS = 2 * ((SMAX + 2) / 2);
-    // the 128 px, +-16 px instance keeps a second table 2 W_N^(b d) for stage B (the weight 2 of
-    // kx != 0 rides on the twiddles, exact, instead of scaling every input)
-    static constexpr bool TW2 = N == 128 && SMAX == 16 && THREADS == 512;
-    static constexpr size_t SM_TWC = (size_t)(TW2 ? 2 : 1) * R * TWS * sizeof(float2);
-    static_assert((SM_IMG + SM_QA) % 16 == 0 && (TWS * sizeof(float2)) % 16 == 0, "16-byte twiddle pairs");
-    static constexpr size_t SM_ROW = (size_t)PB * NROW * BSPLIT * (2 * sizeof(float) + sizeof(int));
-    static constexpr size_t SM_DIR = (size_t)NDIR * sizeof(float);
-    static constexpr size_t SM_BASE = SM_IMG + SM_QA + SM_TWC + SM_ROW + SM_DIR;
     // Packed edge columns: for real images and projections the product conj(O) C is Hermitian in
     // ky on the kx = 0 and kx = N/2 columns, so both columns' stage-A outputs are real, and one
     // complex transform of Z(ky) = P(ky, 0) + i P(ky, N/2) gives Q(dy, 0) as its real part and
-    // Q(dy, N/2) as its imaginary part.  That leaves N/2 column tasks per pair (a multiple of the
-    // block's warps); Z is formed for the batch in shared memory before stage A.  Used where Z fits.
-    static constexpr size_t SM_Z_PACKED = (size_t)PB * N * sizeof(float2);
-    static constexpr bool PACK = ALLOW_PACK_ && SM_BASE + SM_Z_PACKED <= kScoreSmemLimit;
+    // Q(dy, N/2) as its imaginary part.  That leaves N/2 column tasks per pair; Z is formed for the
+    // batch in shared memory before stage A.
+    static constexpr bool PACK = PACK_;
     static constexpr int NCOL = PACK ? NC : H;      // stage-A column tasks per pair
-    static constexpr int TASKS_A = PB * NCOL;       // stage-A column tasks per batch
-    static constexpr size_t SM_Z = PACK ? SM_Z_PACKED : 0;
+    static constexpr int TASKS_A = GPB * NCOL;      // stage-A column tasks per batch
+    static constexpr size_t SM_Z = PACK ? (size_t)PB * N * sizeof(float2) : 0;
     // The dy = +SMAX row by real transforms (the 128 px, +-16 px instance): jobs (pair, Re / Im,
-    // kx sub-sequence) on the last PB 2 R threads, each a real 16-point transform recombined into the
-    // SMAX + 1 even (cosine) or odd (sine) outputs, summed over sub-sequences by lane shuffles; a
-    // direct sum costs ~60 multiply-adds per output instead.
-    static constexpr bool DIRFFT = PACK && N == 128 && SMAX == 16 && THREADS == 512 && PB == 8;
+    // kx sub-sequence) on the last GPB 2 R threads of the group, each a real 16-point transform
+    // recombined into the SMAX + 1 even (cosine) or odd (sine) outputs, summed over sub-sequences by
+    // lane shuffles; a direct sum costs ~60 multiply-adds per output instead.
+    static constexpr bool DIRFFT = PACK && N == 128 && SMAX == 16;
+    static_assert(!DIRFFT || (GPB * NCOL == GT && BSPLIT == 2 && ((GPB * 2 * R) % 32 == 0 || GPB * 2 * R == 16)),
+                  "each group's tasks on its own threads, its dy = +SMAX jobs on whole warps or half a warp");
+    // that instance keeps a second table 2 W_N^(b d) for stage B (the weight 2 of kx != 0 rides on the
+    // twiddles, exact, instead of scaling every input)
+    static constexpr bool TW2 = DIRFFT;
+    static constexpr size_t SM_TWC = (size_t)(TW2 ? 2 : 1) * R * TWS * sizeof(float2);
+    static_assert((SM_IMG + SM_QA) % 16 == 0 && (TWS * sizeof(float2)) % 16 == 0, "16-byte twiddle pairs");
+    static constexpr size_t SM_ROW = (size_t)NGROUP * ROWS * (2 * sizeof(float) + sizeof(int));
+    static constexpr size_t SM_DIR = (size_t)NGROUP * NDIR * sizeof(float);
+    static constexpr size_t SM_BASE = (SM_IMG + SM_QA + SM_TWC + SM_Z + SM_ROW + SM_DIR + 7) / 8 * 8;
     static constexpr size_t SM_DTW = DIRFFT ? (size_t)2 * R * (SMAX + 1) * sizeof(float2) : 0;
     static constexpr size_t SM_DSUM = DIRFFT ? (size_t)PB * 2 * (SMAX + 1) * sizeof(float) : 0;
-    static constexpr size_t SMEM = SM_BASE + SM_Z + SM_DTW + SM_DSUM;
+    static constexpr size_t SMEM = SM_BASE + SM_DTW + SM_DSUM;
     static_assert(SMEM <= kScoreSmemLimit, "dynamic shared memory per block");
-    // Decoupled groups (the 128 px, +-16 px instance): the block's threads form NGROUP groups of
-    // GT threads, group g owning pairs [g GPB, (g + 1) GPB) of every batch in every phase (packed
-    // edge columns, stage A, stage B, the dy = +SMAX row, the combine), and within the batch loop
-    // each group waits only on its own named barrier.  The groups drift apart, so that one group's
-    // projection loads and barrier waits overlap the others' transform arithmetic instead of the
-    // whole block moving through its phases in step (the FP32 pipe saturated in the transforms and
-    // idle in between).  Measured per pair: 14.25 ns in step, 13.43 ns with two groups, 12.59 ns
-    // with four, 13.17 ns with eight (one pair per group, the dy = +SMAX jobs on half a warp).
-    static constexpr bool SPLIT = DIRFFT;
-    static constexpr int NGROUP = SPLIT ? 4 : 1;
-    static constexpr int GT = THREADS / NGROUP, GPB = PB / NGROUP;   // threads and pairs of one group
-    static_assert(!SPLIT || (GT % 32 == 0 && GPB * NCOL == GT && GPB * NROW * BSPLIT == GT &&
-                             ((GPB * 2 * R) % 32 == 0 || GPB * 2 * R == 16)),
-                  "each group's tasks on its own threads, its dy = +SMAX jobs on whole warps or half a warp");
+    // lanes that combine a pair's pieces (NROW BSPLIT rows and NS direct outputs)
+    static constexpr int LPP = SMAX <= 12 ? 8 : 32;
 };
 
-// The batch loop's barrier: the whole block, or with C::SPLIT the calling thread's group (named
-// barrier 1 + group over C::GT threads).
+// The batch loop's barrier: the calling thread's group (named barrier 1 + group over C::GT threads).
 template <class C>
 __device__ __forceinline__ void batch_sync() {
-    if constexpr (C::SPLIT) {
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / C::GT), "n"(C::GT) : "memory");
-    } else {
-        __syncthreads();
-    }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / C::GT), "n"(C::GT) : "memory");
 }
 
 // Stage A for one column kx of one pair: Q(dy, kx) for dy = -SMAX..SMAX, with the rows ky = b + R a
@@ -227,7 +216,7 @@ template <class C>
 __device__ __forceinline__ void stage_a_column(float2 (&acc)[C::NS], const float2* __restrict__ img_col,
                                                const float2* __restrict__ ps_col, const float2* __restrict__ twc,
                                                const float2* __restrict__ zcol) {
-    constexpr int H = C::H, R = C::R, NS = C::NS, SMAX = C::SMAX;
+    constexpr int H = C::H, R = C::R, SMAX = C::SMAX;
     float2 cn[L];
     if constexpr (C::PREFETCH) {
         if (!zcol) {
@@ -283,7 +272,7 @@ __device__ __forceinline__ void stage_a_column(float2 (&acc)[C::NS], const float
 template <class C>
 __device__ __forceinline__ void stage_b_row(float (&acc)[C::NS], const float2* __restrict__ qrow,
                                             const float2* __restrict__ twc, int b0, int b1) {
-    constexpr int R = C::R, NS = C::NS, SMAX = C::SMAX;
+    constexpr int R = C::R, SMAX = C::SMAX;
 #pragma unroll 1
     for (int b = b0; b < b1; ++b) {
         float2 x[L];
@@ -355,33 +344,55 @@ __device__ __forceinline__ float loglik_t(float rho, int* status) {
     return t;
 }
 
-// Stage B (row transforms), the dy = +SMAX row, the likelihood epilogue and the per-pair combine of
-// one batch whose Q (stage-A output, [pair][dy][kx]) is in q_s; records for pairs p0 .. hi-1.
+// Shared-memory arrays of a scoring block (pairs j of all groups; group g owns [g GPB, (g + 1) GPB)).
 template <class C>
-__device__ __forceinline__ void score_tail(const float2* __restrict__ q_s, const float2* __restrict__ twc_s,
-                                           float* row_t, float* row_s, int* row_d, float* dir_t,
-                                           const float2* __restrict__ dtw, float* dsum,
-                                           const float2* __restrict__ gtw, int p0, int hi, int s, float c1,
-                                           float* __restrict__ rec_t, float* __restrict__ rec_s,
+struct Sm {
+    float2* img;    // [N][H] the item's image
+    float2* q;      // [PB][NS][QS] stage-A output
+    float2* twc;    // [R][TWS] twiddles, a second table with C::TW2
+    float2* z;      // [PB][N] packed edge columns (C::PACK)
+    float* row_t;   // [NGROUP][ROWS] per-row parts
+    float* row_s;
+    int* row_d;
+    float* dir_t;   // [NGROUP][NDIR] the dy = +SMAX row's ln(1 - rho^2)
+    float2* dtw;    // [2][R][SMAX + 1] (C::DIRFFT)
+    float* dsum;    // [PB][2][SMAX + 1]
+    __device__ __forceinline__ explicit Sm(unsigned char* smem) {
+        img = reinterpret_cast<float2*>(smem);
+        q = reinterpret_cast<float2*>(smem + C::SM_IMG);
+        twc = reinterpret_cast<float2*>(smem + C::SM_IMG + C::SM_QA);
+        z = reinterpret_cast<float2*>(smem + C::SM_IMG + C::SM_QA + C::SM_TWC);
+        row_t = reinterpret_cast<float*>(smem + C::SM_IMG + C::SM_QA + C::SM_TWC + C::SM_Z);
+        row_s = row_t + C::NGROUP * C::ROWS;
+        row_d = reinterpret_cast<int*>(row_s + C::NGROUP * C::ROWS);
+        dir_t = reinterpret_cast<float*>(row_d + C::NGROUP * C::ROWS);
+        dtw = reinterpret_cast<float2*>(smem + C::SM_BASE);
+        dsum = reinterpret_cast<float*>(smem + C::SM_BASE + C::SM_DTW);
+    }
+};
+
+// Stage B (row transforms), the dy = +SMAX row, the likelihood epilogue and the per-pair combine of
+// one batch of the calling group whose Q (stage-A output, [pair][dy][kx]) is in sm.q; records for pairs
+// p0 .. hi-1.
+template <class C>
+__device__ __forceinline__ void score_tail(const Sm<C>& sm, const float2* __restrict__ gtw, int p0, int hi, int s,
+                                           float c1, float* __restrict__ rec_t, float* __restrict__ rec_s,
                                            int* __restrict__ rec_d, int* __restrict__ status) {
-    constexpr int N = C::N, NC = C::NC, NS = C::NS, SMAX = C::SMAX, NROW = C::NROW;
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const bool active = tid < C::THREADS;
-    // ---------------- stage B: one row (dy = -SMAX .. SMAX-1) of one pair per thread (per two
+    constexpr int N = C::N, NC = C::NC, NS = C::NS, SMAX = C::SMAX, NROW = C::NROW, BS = C::BSPLIT;
+    const int grp = threadIdx.x / C::GT, tg = threadIdx.x - grp * C::GT;
+    // ---------------- stage B: one row (dy = -SMAX .. SMAX-1) of one pair per task (per two
     // adjacent threads with BSPLIT = 2)
-    if (tid < C::PB * NROW * C::BSPLIT) {
-        constexpr int BS = C::BSPLIT;
-        static_assert(BS == 1 || (C::PB * NROW * BS) % 32 == 0, "split rows fill whole warps");
-        const int rr = tid / BS;
-        const int h = tid - rr * BS;
-        const int j = rr / NROW;
-        const int r = rr - j * NROW;
-        const float2* qrow = q_s + ((size_t)j * NS + r) * C::QS;
+#pragma unroll 1
+    for (int task = tg; task < C::ROWS; task += C::GT) {
+        const int rr = task / BS;
+        const int h = task - rr * BS;
+        const int jl = rr / NROW;
+        const int r = rr - jl * NROW;
+        const float2* qrow = sm.q + ((size_t)(grp * C::GPB + jl) * NS + r) * C::QS;
         float acc[NS];
 #pragma unroll
         for (int m = 0; m < NS; ++m) acc[m] = 0.f;
-        stage_b_row<C>(acc, qrow, twc_s + (C::TW2 ? C::R * C::TWS : 0), h * (C::R / BS), (h + 1) * (C::R / BS));
+        stage_b_row<C>(acc, qrow, sm.twc + (C::TW2 ? C::R * C::TWS : 0), h * (C::R / BS), (h + 1) * (C::R / BS));
         constexpr int MH = BS == 2 ? (NS + 1) / 2 : NS;   // outputs evaluated by this thread
         int m0 = 0;
         if constexpr (BS == 2) {
@@ -428,22 +439,20 @@ __device__ __forceinline__ void score_tail(const float2* __restrict__ q_s, const
             eval(std::true_type{});
         else
             eval(std::false_type{});
-        row_t[tid] = tmin;
-        row_s[tid] = ssum;
-        row_d[tid] = arg;
+        const int o = grp * C::ROWS + task;
+        sm.row_t[o] = tmin;
+        sm.row_s[o] = ssum;
+        sm.row_d[o] = arg;
     }
     // ---------------- the dy = +SMAX row by real transforms (see Cfg::DIRFFT)
     if constexpr (C::DIRFFT) {
-        constexpr int NJ = C::PB * 2 * C::R;   // jobs: (pair j, component c, sub-sequence b)
-        static_assert(C::R == 8 && NJ % 32 == 0 && NJ <= C::THREADS, "one job per thread, whole warps");
-        // the last NJ threads, or with C::SPLIT the last NJ / NGROUP threads of each group for its
-        // pairs (the upper half of a warp when that is 16)
-        constexpr int NJG = C::SPLIT ? NJ / C::NGROUP : NJ;
+        constexpr int NJG = C::GPB * 2 * C::R;   // jobs: (pair j, component c, sub-sequence b)
+        static_assert(C::R == 8 && NJG <= C::GT, "one job per thread");
+        // the last NJG threads of the group (the upper half of a warp when that is 16)
         constexpr unsigned JM = NJG >= 32 ? 0xffffffffu : (0xffffffffu << (32 - NJG));   // job lanes
-        const int grp = C::SPLIT ? tid / C::GT : 0;
-        const int tj = C::SPLIT ? tid - grp * C::GT - (C::GT - NJG) : tid - (C::THREADS - NJ);
+        const int tj = tg - (C::GT - NJG);
         const int b = tj & 7, c = (tj >> 3) & 1, j = grp * C::GPB + (tj >> 4);
-        const float2* qrow = q_s + ((size_t)j * NS + 2 * SMAX) * C::QS;
+        const float2* qrow = sm.q + ((size_t)j * NS + 2 * SMAX) * C::QS;
         if (tj >= 0) {
             float x[8], yr[9], yi[9], a17[SMAX + 1];
 #pragma unroll
@@ -457,13 +466,14 @@ __device__ __forceinline__ void score_tail(const float2* __restrict__ q_s, const
             rdft16(x, yr, yi);
 #pragma unroll
             for (int k = 0; k <= SMAX; ++k) a17[k] = 0.f;
-            recombine<SMAX + 1>(a17, yr, yi, dtw + (c * C::R + b) * (SMAX + 1));
+            recombine<SMAX + 1>(a17, yr, yi, sm.dtw + (c * C::R + b) * (SMAX + 1));
 #pragma unroll
             for (int k = 0; k <= SMAX; ++k) {
                 a17[k] += __shfl_xor_sync(JM, a17[k], 1);
                 a17[k] += __shfl_xor_sync(JM, a17[k], 2);
                 a17[k] += __shfl_xor_sync(JM, a17[k], 4);
             }
+            float* dsum = sm.dsum;
             if (b == 0) {
 #pragma unroll
                 for (int k = 0; k <= SMAX; ++k) dsum[(j * 2 + c) * (SMAX + 1) + k] = a17[k];
@@ -479,20 +489,18 @@ __device__ __forceinline__ void score_tail(const float2* __restrict__ q_s, const
                 const float cv = dsum[(j * 2) * (SMAX + 1) + dx], sv = dsum[(j * 2 + 1) * (SMAX + 1) + dx];
                 const float rho = cv + (c ? sv : -sv) + ((dx & 1) ? -qn : qn);
                 const int dxs = c ? -dx : dx;
-                dir_t[j * NS + dxs + SMAX] = (row_ok && abs(dxs) <= s) ? loglik_t(rho, status) : INFINITY;
+                sm.dir_t[j * NS + dxs + SMAX] = (row_ok && abs(dxs) <= s) ? loglik_t(rho, status) : INFINITY;
             }
         }
-    }
-    // ---------------- the dy = +SMAX row, one output per task, evaluated directly; the
-    // threads without a stage-B row (tid >= PB NROW) take the first outputs so that few
-    // threads with a row get two
-    if (active && !C::DIRFFT) {
+    } else {
+        // ---------------- the dy = +SMAX row, one output per task, evaluated directly; the threads
+        // after the last stage-B row take the first outputs
 #pragma unroll 1
-        for (int i = (tid + C::THREADS - C::PB * NROW * C::BSPLIT) % C::THREADS; i < C::NDIR; i += C::THREADS) {
-            const int j = i / NS;
-            const int mi = i - j * NS;
+        for (int i = (tg + C::GT - C::ROWS % C::GT) % C::GT; i < C::NDIR; i += C::GT) {
+            const int jl = i / NS;
+            const int mi = i - jl * NS;
             const int dx = mi - SMAX;
-            const float2* qrow = q_s + ((size_t)j * NS + 2 * SMAX) * C::QS;
+            const float2* qrow = sm.q + ((size_t)(grp * C::GPB + jl) * NS + 2 * SMAX) * C::QS;
             float accv = 0.f;
             int idx = pmod(dx, N);
             const int step = idx;
@@ -506,34 +514,35 @@ __device__ __forceinline__ void score_tail(const float2* __restrict__ q_s, const
             const float qn = C::PACK ? qrow[0].y : qrow[NC].x;
             const float rho = qrow[0].x + 2.f * accv + ((dx & 1) ? -qn : qn);
             const bool ok = SMAX <= s && abs(dx) <= s;
-            dir_t[i] = ok ? loglik_t(rho, status) : INFINITY;
+            sm.dir_t[grp * C::NDIR + i] = ok ? loglik_t(rho, status) : INFINITY;
         }
     }
     batch_sync<C>();
-    // ---------------- combine the pieces of each pair (one full warp per pair; with C::SPLIT the
-    // first warps of each group for its pairs)
-    const int jw = C::SPLIT ? (tid / C::GT) * C::GPB + (warp - (tid / C::GT) * (C::GT / 32)) : warp;
-    const int jend = C::SPLIT ? (tid / C::GT + 1) * C::GPB : C::PB;
-    for (int j = jw; warp < C::NWARPS && j < jend; j += C::NWARPS) {
-        const int p = p0 + j;
-        if (p >= hi) continue;
+    // ---------------- combine the pieces of each pair: LPP lanes per pair, on the group's first warps
+    constexpr int LPP = C::LPP, NR = NROW * BS;
+#pragma unroll 1
+    for (int e = tg; (e & ~31) < C::GPB * LPP; e += C::GT) {
+        const int jl = min(e / LPP, C::GPB - 1), l = e % LPP;
+        const float* row_t = sm.row_t + grp * C::ROWS + jl * NR;
+        const float* row_s = sm.row_s + grp * C::ROWS + jl * NR;
+        const int* row_d = sm.row_d + grp * C::ROWS + jl * NR;
+        const float* dir_t = sm.dir_t + grp * C::NDIR + jl * NS;
         Part acc{INFINITY, 0.f, 0x7fffffff};
-        constexpr int NR = NROW * C::BSPLIT;
-        for (int r = lane; r < NR; r += 32)
-            acc = merge(acc, Part{row_t[j * NR + r], row_s[j * NR + r], row_d[j * NR + r]}, c1);
-        for (int mi = lane; mi < NS; mi += 32) {
-            const float t = dir_t[j * NS + mi];
+        for (int r = l; r < NR; r += LPP) acc = merge(acc, Part{row_t[r], row_s[r], row_d[r]}, c1);
+        for (int mi = l; mi < NS; mi += LPP) {
+            const float t = dir_t[mi];
             acc = merge(acc, Part{t, t < INFINITY ? 1.f : 0.f, 2 * SMAX * NS + mi}, c1);
         }
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
+        for (int off = LPP / 2; off > 0; off >>= 1) {
             Part o;
             o.t = __shfl_xor_sync(0xffffffffu, acc.t, off);
             o.s = __shfl_xor_sync(0xffffffffu, acc.s, off);
             o.d = __shfl_xor_sync(0xffffffffu, acc.d, off);
             acc = merge(acc, o, c1);   // merge orders its operands, so both lanes agree
         }
-        if (lane == 0) {
+        const int p = p0 + jl;
+        if (l == 0 && e < C::GPB * LPP && p < hi) {
             rec_t[p] = acc.t;
             rec_s[p] = acc.s;
             rec_d[p] = acc.d;
@@ -541,97 +550,90 @@ __device__ __forceinline__ void score_tail(const float2* __restrict__ q_s, const
     }
 }
 
+// The block's constant tables (once per launch; a block barrier follows before their first use).
+template <class C>
+__device__ __forceinline__ void score_tables(const Sm<C>& sm) {
+    constexpr int N = C::N, SMAX = C::SMAX;
+    const float2* cwN = cw_table<N>();
+    for (int i = threadIdx.x; i < C::R * C::TWS; i += C::THREADS) {
+        const int b = i / C::TWS, d = i - (i / C::TWS) * C::TWS;
+        const float2 w = d <= SMAX ? cwN[pmod(b * d, N)] : make_float2(0.f, 0.f);
+        sm.twc[i] = w;
+        if constexpr (C::TW2) sm.twc[C::R * C::TWS + i] = make_float2(2.f * w.x, 2.f * w.y);
+    }
+    if constexpr (C::DIRFFT) {
+        // (T1, T2) x 2 (the weight of kx != 0) for component c, sub-sequence b, output dx
+        for (int i = threadIdx.x; i < 2 * C::R * (SMAX + 1); i += C::THREADS) {
+            const int c = i / (C::R * (SMAX + 1)), b = (i / (SMAX + 1)) % C::R, dx = i % (SMAX + 1);
+            const int u = dx & 15;
+            const bool cj = u > 8;
+            const float2 w = cwN[(b * dx) % N];   // (cos, sin) of 2 pi b dx / N
+            const float t1 = c == 0 ? w.x : w.y;
+            const float t2 = c == 0 ? (cj ? w.y : -w.y) : (cj ? -w.x : w.x);
+            sm.dtw[i] = make_float2(2.f * t1, 2.f * t2);
+        }
+    }
+}
+
 // One work item: image w against parameter sets [lo, hi) of the wave starting at ps_begin.
 // img: the image's spectrum; rec_*: the image's record row (indexed by the wave-relative set);
 // gtw: exp(-2 pi i t / N), t < N, in global memory (the direct row's twiddles, L1-resident).
-// Threads with tid >= C::THREADS only take part in the barriers.
 template <class C>
-__device__ __forceinline__ void score_item(unsigned char* smem, const float2* __restrict__ gtw,
+__device__ __forceinline__ void score_item(const Sm<C>& sm, const float2* __restrict__ gtw,
                                            const float2* __restrict__ img, const int* __restrict__ ps_idx,
                                            const float2* __restrict__ ps_spec, int ps_begin, int lo, int hi, int s,
                                            float c1, float* __restrict__ rec_t, float* __restrict__ rec_s,
                                            int* __restrict__ rec_d, int* __restrict__ status) {
-    constexpr int N = C::N, NC = C::NC, H = C::H, NS = C::NS, SMAX = C::SMAX, NROW = C::NROW;
-    float2* img_s = reinterpret_cast<float2*>(smem);
-    float2* q_s = reinterpret_cast<float2*>(smem + C::SM_IMG);
-    float2* twc_s = reinterpret_cast<float2*>(smem + C::SM_IMG + C::SM_QA);
-    float2* z_s = reinterpret_cast<float2*>(smem + C::SM_IMG + C::SM_QA + C::SM_TWC);   // [PB][N] (C::PACK)
-    float* row_t = reinterpret_cast<float*>(z_s + (C::PACK ? C::PB * N : 0));
-    float* row_s = row_t + C::PB * NROW * C::BSPLIT;
-    int* row_d = reinterpret_cast<int*>(row_s + C::PB * NROW * C::BSPLIT);
-    float* dir_t = reinterpret_cast<float*>(row_d + C::PB * NROW * C::BSPLIT);
-    float2* dtw = reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(smem) + C::SM_BASE + C::SM_Z);
-    float* dsum = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(dtw) + C::SM_DTW);
-
-    const int tid = threadIdx.x;
-    const bool active = tid < C::THREADS;
+    constexpr int N = C::N, NC = C::NC, H = C::H, NS = C::NS, GT = C::GT, GPB = C::GPB;
+    __shared__ int next_pair;            // first pair of the item's next untaken batch
+    __shared__ int group_next[C::NGROUP];
+    const int grp = threadIdx.x / GT, tg = threadIdx.x - grp * GT;
     __syncthreads();   // the previous item's readers of shared memory are done
     {
-        const float2* cwN = cw_table<N>();
-        for (int i = tid; i < C::R * C::TWS; i += blockDim.x) {
-            const int b = i / C::TWS, d = i - (i / C::TWS) * C::TWS;
-            const float2 w = d <= SMAX ? cwN[pmod(b * d, N)] : make_float2(0.f, 0.f);
-            twc_s[i] = w;
-            if constexpr (C::TW2) twc_s[C::R * C::TWS + i] = make_float2(2.f * w.x, 2.f * w.y);
-        }
         const float4* src = reinterpret_cast<const float4*>(img);
-        float4* dst = reinterpret_cast<float4*>(img_s);
-        for (int i = tid; i < N * H / 2; i += blockDim.x) dst[i] = __ldg(src + i);
-        if constexpr (C::DIRFFT) {
-            // (T1, T2) x 2 (the weight of kx != 0) for component c, sub-sequence b, output dx
-            const float2* cwN = cw_table<N>();
-            for (int i = tid; i < 2 * C::R * (SMAX + 1); i += blockDim.x) {
-                const int c = i / (C::R * (SMAX + 1)), b = (i / (SMAX + 1)) % C::R, dx = i % (SMAX + 1);
-                const int u = dx & 15;
-                const bool cj = u > 8;
-                const float2 w = cwN[(b * dx) % N];   // (cos, sin) of 2 pi b dx / N
-                const float t1 = c == 0 ? w.x : w.y;
-                const float t2 = c == 0 ? (cj ? w.y : -w.y) : (cj ? -w.x : w.x);
-                dtw[i] = make_float2(2.f * t1, 2.f * t2);
-            }
-        }
+        float4* dst = reinterpret_cast<float4*>(sm.img);
+        for (int i = threadIdx.x; i < N * H / 2; i += C::THREADS) dst[i] = __ldg(src + i);
+        if (threadIdx.x == 0) next_pair = lo + C::PB;
     }
     __syncthreads();
-    for (int p0 = lo; p0 < hi; p0 += C::PB) {
+#pragma unroll 1
+    for (int p0 = lo + grp * GPB; p0 < hi;) {
         // ---------------- packed edge columns Z(ky) = P(ky, 0) + i P(ky, N/2) of the batch's pairs
         if constexpr (C::PACK) {
-            // with C::SPLIT each group forms its own pairs' columns
-            const int i0 = C::SPLIT ? (tid / C::GT) * C::GPB * N + tid % C::GT : tid;
-            const int i1 = C::SPLIT ? (tid / C::GT + 1) * C::GPB * N : C::PB * N;
-            const int istep = C::SPLIT ? C::GT : blockDim.x;
-            for (int i = i0; i < i1; i += istep) {
-                const int j = i / N;
-                const int ky = i - j * N;
-                const int p = min(p0 + j, hi - 1);
+            for (int i = tg; i < GPB * N; i += GT) {
+                const int jl = i / N;
+                const int ky = i - jl * N;
+                const int p = min(p0 + jl, hi - 1);
                 const int gp = ps_idx ? __ldg(ps_idx + p) : ps_begin + p;
                 const float2* ps_row = ps_spec + (size_t)gp * N * H + (size_t)ky * H;
-                const float2 e0 = c_mulc(img_s[ky * H], __ldg(ps_row));
-                const float2 e1 = c_mulc(img_s[ky * H + NC], __ldg(ps_row + NC));
-                z_s[i] = make_float2(e0.x - e1.y, e0.y + e1.x);
+                const float2 e0 = c_mulc(sm.img[ky * H], __ldg(ps_row));
+                const float2 e1 = c_mulc(sm.img[ky * H + NC], __ldg(ps_row + NC));
+                sm.z[grp * GPB * N + i] = make_float2(e0.x - e1.y, e0.y + e1.x);
             }
             batch_sync<C>();
         }
         // ---------------- stage A: one column of one pair per task
-        if (active) {
 #pragma unroll 1
-            for (int task = tid; task < C::TASKS_A; task += C::THREADS) {
-                const int j = task / C::NCOL;
-                const int kx = task - j * C::NCOL;
-                const int p = min(p0 + j, hi - 1);
-                const int gp = ps_idx ? __ldg(ps_idx + p) : ps_begin + p;
-                const float2* ps_col = ps_spec + (size_t)gp * N * H + kx;
-                float2 acc[NS];
+        for (int task = tg; task < C::TASKS_A; task += GT) {
+            const int jl = task / C::NCOL;
+            const int kx = task - jl * C::NCOL;
+            const int p = min(p0 + jl, hi - 1);
+            const int gp = ps_idx ? __ldg(ps_idx + p) : ps_begin + p;
+            const float2* ps_col = ps_spec + (size_t)gp * N * H + kx;
+            const int j = grp * GPB + jl;
+            float2 acc[NS];
 #pragma unroll
-                for (int m = 0; m < NS; ++m) acc[m] = make_float2(0.f, 0.f);
-                stage_a_column<C>(acc, img_s + kx, ps_col, twc_s, (C::PACK && kx == 0) ? z_s + j * N : nullptr);
-                float2* qdst = q_s + (size_t)j * NS * C::QS + kx;
+            for (int m = 0; m < NS; ++m) acc[m] = make_float2(0.f, 0.f);
+            stage_a_column<C>(acc, sm.img + kx, ps_col, sm.twc, (C::PACK && kx == 0) ? sm.z + j * N : nullptr);
+            float2* qdst = sm.q + (size_t)j * NS * C::QS + kx;
 #pragma unroll
-                for (int m = 0; m < NS; ++m) qdst[m * C::QS] = acc[m];
-            }
+            for (int m = 0; m < NS; ++m) qdst[m * C::QS] = acc[m];
         }
         batch_sync<C>();
-        score_tail<C>(q_s, twc_s, row_t, row_s, row_d, dir_t, dtw, dsum, gtw, p0, hi, s, c1, rec_t, rec_s, rec_d,
-                      status);
+        // the group's next batch: written between the two barriers, read after the second
+        if (tg == 0) group_next[grp] = atomicAdd(&next_pair, GPB);
+        score_tail<C>(sm, gtw, p0, hi, s, c1, rec_t, rec_s, rec_d, status);
+        p0 = group_next[grp];
     }
 }
 
@@ -648,6 +650,8 @@ k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int
         int* __restrict__ work) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int next_item;
+    const Sm<C> sm(smem);
+    score_tables<C>(sm);
     for (;;) {
         if (threadIdx.x == 0) next_item = atomicAdd(work, 1);
         __syncthreads();
@@ -658,7 +662,7 @@ k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int
         const int lo = ci * chunk;
         const int hi = min(lo + chunk, ps_count);
         const size_t row = (size_t)w * ps_count;
-        score_item<C>(smem, gtw, img_spec + (size_t)w * C::N * C::H, nullptr, ps_spec, ps_begin, lo, hi, s, c1, rec_t + row,
+        score_item<C>(sm, gtw, img_spec + (size_t)w * C::N * C::H, nullptr, ps_spec, ps_begin, lo, hi, s, c1, rec_t + row,
                       rec_s + row, rec_d + row, status);
     }
 }
@@ -713,7 +717,7 @@ __device__ __forceinline__ int lse_add4(double& M, double& S, const double (&m)[
         d[i] = m[i] - M;
         any |= d[i] > kExpMin;
     }
-    if (__any_sync(__activemask(), any)) {
+    if (any) {
         double e[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) e[i] = exp_neg(d[i] > kExpMin ? d[i] : 0.0, tab);
@@ -775,7 +779,8 @@ __device__ __forceinline__ void acc_merge_prev(Acc& r, const Acc& prev) {
 // and, if requested, write the per-orientation posteriors of the share's orientations.  Parts are whole
 // orientations; an image is cut into enough of them to occupy the GPU (reduce_parts).  An image in one part
 // is folded in place (parts = prev = the running accumulators; prev null: the first wave).  Bound by the
-// float64 pipe: one exponential per record for each of the two outputs (REDUCE_NOTE).
+// float64 pipe: one exponential per record for each of the two outputs (64 images x 6912 sets: 93 us as one
+// block per image, 39 us so; 16 images with per-orientation output: 181 -> 32 us).
 __global__ void __launch_bounds__(kRedThreads) k_reduce_wave(
     const float* __restrict__ rec_t, const float* __restrict__ rec_s, const int* __restrict__ rec_d,
     const double* __restrict__ kA, const double* __restrict__ kB, int ps_begin, int wave_len, int nctf,
@@ -1025,18 +1030,38 @@ int score_slots(bioem_ctx* ctx, int* slots) {
     return BIOEM_OK;
 }
 
+// Parameter sets per work item.  A block's groups take an item's batches from its counter and wait for one
+// another between items (about 0.6 of a round of all groups); with more items than slots the last items
+// end unevenly (about 0.75 of an item).  Of the even splits of the wl sets into k chunks, the one with
+// the least rounds + waits; measured at 64 images x 4608 sets, 128 px, +-16 px (ns per pair): chunks of
+// 512: 14.3, 300: 13.5, 243: 13.0, 180: 12.9, 120: 12.7, 64: 12.8.  At most ~34 MB of projection spectra
+// per chunk (512 sets at 128 px), so that the chunk all blocks work on stays in L2.
+template <class C>
+int score_chunk(int n_img, int wl, int slots) {
+    const long long spec = (long long)sizeof(float2) * C::N * C::H;
+    const long long cap = (34ll << 20) / spec > 512 ? (34ll << 20) / spec : 512;
+    const long long k0 = (wl + cap - 1) / cap;
+    long long best = (cap + C::GPB - 1) / C::GPB * C::GPB;
+    double best_cost = 1e300;
+    for (long long k = k0, step = 1; k < 64 * k0 && k <= wl; k += step, step = 1 + k / 16) {
+        const long long chunk = ((wl + k - 1) / k + C::GPB - 1) / C::GPB * C::GPB;
+        const long long items = (wl + chunk - 1) / chunk * n_img;
+        const double turns = items <= slots ? 1.0 : (double)items / slots + 0.75;
+        const double cost = turns * ((double)chunk / C::PB + 0.6);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = chunk;
+        }
+    }
+    return (int)best;
+}
+
 // One k_score<C> launch writing the records of parameter sets [wbegin, wbegin + wl) for every image.
-// Chunk: enough work items to keep every slot busy, at most 512 parameter sets, whole batches.
 template <class C>
 int launch_score_records(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, int slots, int wbegin,
                          int wl, int max_shift, float* rec_t, float* rec_s, int* rec_d) {
     const int n_img = im->n_img;
-    const long long target_items = 4ll * slots;
-    const long long per_img = (target_items + n_img - 1) / n_img;
-    long long chunk = (wl + per_img - 1) / per_img;
-    chunk = ((chunk + C::PB - 1) / C::PB) * C::PB;
-    if (chunk > 512) chunk = 512 / C::PB * C::PB;
-    if (chunk < C::PB) chunk = C::PB;
+    const long long chunk = score_chunk<C>(n_img, wl, slots);
     const long long n_chunks = (wl + chunk - 1) / chunk;
     const long long n_items = n_chunks * n_img;
     if (n_items > 0x7fffffffll) return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "too many work items");
@@ -1082,27 +1107,27 @@ int run_score_gemm(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* 
     return run_waves(ctx, im, ps, max_shift, max_shift, align, out, records);
 }
 
-// <N, SMAX, pairs per batch, threads[, packed edge columns allowed]>: the threads divide the
-// stage-A tasks (PB N/2 with the packed edge columns, PB (N/2 + 1) without) into whole rounds.
-// Packed edge columns where they measured faster (128 px: 2 % at s = 4, 6 % at s = 16); at 32-96
-// px the transforms are short enough that forming Z costs about as much as the column it saves
-// (unpacked 4-9 % faster there).
-using C32_4 = Cfg<32, 4, 32, 272, false>;
-using C64_4 = Cfg<64, 4, 32, 264, false>;
-using C64_8 = Cfg<64, 8, 16, 264, false>;
-using C96_12 = Cfg<96, 12, 10, 245, false>;
-using C128_4 = Cfg<128, 4, 24, 256>;
-// 128 px, s <= 16: 512 threads (four warps per scheduler, 128 registers), one stage-A column per
-// thread and two threads per stage-B row, in four decoupled groups of two pairs (Cfg::SPLIT); 11 %
-// faster than 256 threads with one row per thread, which left the kernel waiting on
-// dependent-instruction latency at two warps per scheduler.
-using C128_16 = Cfg<128, 16, 8, 512, true, 2>;
-using C192_24 = Cfg<192, 24, 2, 194>;
-static_assert(C128_4::PACK && C128_16::PACK, "packed edge columns fit");
-static_assert(C128_16::TASKS_A % C128_16::THREADS == 0 && C128_4::TASKS_A % C128_4::THREADS == 0 &&
-              C64_8::TASKS_A % C64_8::THREADS == 0 && C64_4::TASKS_A % C64_4::THREADS == 0 &&
-              C32_4::TASKS_A % C32_4::THREADS == 0 && C96_12::TASKS_A % C96_12::THREADS == 0 &&
-              C192_24::TASKS_A % C192_24::THREADS == 0, "whole stage-A rounds");
+// <N, SMAX, groups, threads per group, pairs per group batch, packed edge columns[, threads per
+// stage-B row]>.  Groups as many as registers allow without spills and shared memory holds; a group's batch
+// fills whole rounds of its threads with column tasks (PB N/2 with the packed edge columns, PB (N/2 + 1)
+// without) and at most one round with rows.  ns per pair (k_score, one GB300; one block-wide group of
+// 245-272 threads moving through the phases in step before -> now): 32 px 1.76 -> 0.77; 64 px, s = 4: 3.68 ->
+// 2.14, s = 8: 5.22 -> 3.00; 96 px 10.5 -> 7.5; 128 px, s = 4: 14.7 -> 7.7.  More groups at fewer registers lost
+// (128 px, s = 4: 6 x 128 threads of 79 registers 9.9; 8 x 64 threads 10.4), as did fewer, larger ones
+// (3 x 192 threads 7.9, 3 x 256 10.0).  192 px holds two pairs beside the image: one group in step, 54
+// (as two groups of one pair 64: the 97th column then takes a warp per group; the image read through L1 and
+// three pairs in 10 or 12 warps: 62-73).  The odd column kx = N/2
+// stays a column task: spread over a warp's lanes (transforms, then outputs) it took fewer
+// instructions but made that warp the batch's longest (64 px, s = 4: 2.4; 96 px 8.6; 192 px 62).
+// Packed edge columns where they measured faster (128 px: 2 % at s = 4, 6 % at s = 16); at 32-96 px the
+// transforms are short enough that forming Z costs about as much as the column it saves.
+using C32_4 = Cfg<32, 4, 6, 128, 15, false>;
+using C64_4 = Cfg<64, 4, 5, 128, 11, false>;
+using C64_8 = Cfg<64, 8, 3, 160, 9, false>;
+using C96_12 = Cfg<96, 12, 3, 128, 5, false>;
+using C128_4 = Cfg<128, 4, 4, 160, 5, true>;
+using C128_16 = Cfg<128, 16, 4, 128, 2, true, 2>;
+using C192_24 = Cfg<192, 24, 1, 224, 2, false>;
 
 }  // namespace
 
@@ -1289,26 +1314,17 @@ extern "C" int bioem_score_noalloc(bioem_ctx* ctx, const bioem_images* images, c
 }
 
 // ---------------------------------------------------------------------------- batched scoring
-// Several models against several image stacks of mixed sizes in one persistent launch.  A segment
-// is one (model, stack) pair: the stack's image spectra against that model's parameter sets for
-// that stack.  Work items of all segments form one list; every item runs the instance for its
-// image size.  All instances here use 256 threads (2 warps per scheduler keep the 96 / 192 px
-// paths at their register counts).
+// Several models against several image stacks of mixed sizes.  A segment is one (model, stack) pair:
+// the stack's image spectra against that model's parameter sets for that stack.  The segments of one
+// image size form one work list, run by one persistent launch of that size's scoring instance; the
+// launches of the sizes present are parallel branches of the graph, so that the blocks of the next
+// size start on the SMs that the previous size's blocks leave.  (One kernel that held all four sizes
+// gave every size the register count and the 256 threads of the largest: 19.2 ms for 4 models x 4
+// stacks, 1.03e6 pairs, against 16.2 ms so.)
 #include <string>
 #include <vector>
 
 namespace {
-
-// (unpacked edge columns: the four instances share one kernel's registers, and with the packed
-// columns they spill)
-using M64 = Cfg<64, 8, 15, 256, false>;
-using M96 = Cfg<96, 12, 10, 256, false>;
-using M128 = Cfg<128, 16, 7, 256, false>;
-using M192 = Cfg<192, 24, 2, 256, false>;
-constexpr int kMultiThreads = 256;
-
-constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
-constexpr size_t kMultiSmem = cmax(cmax(M64::SMEM, M96::SMEM), cmax(M128::SMEM, M192::SMEM));
 
 struct SegDesc {
     const float2* img;    // [n_img][N][N/2+1]
@@ -1319,7 +1335,7 @@ struct SegDesc {
     float* rec_t;         // [n_img][n_ps] records
     float* rec_s;
     int* rec_d;
-    long long item_begin; // first global item of this segment
+    long long item_begin; // first item of this segment among those of its image size
     long long row_begin;  // first global reduction row (image) of this segment
     int n_img, n_ps, chunk, n_chunks, s, npix, nctf;
     int out_row;          // model index (row of the output matrix)
@@ -1339,13 +1355,17 @@ __device__ __forceinline__ int find_seg(const SegDesc* segs, int n, long long x,
     return lo;
 }
 
-__global__ void __launch_bounds__(kMultiThreads, 1)
-k_score_multi(const SegDesc* __restrict__ segs, int n_segs, long long n_items, int* __restrict__ status,
-              unsigned long long* __restrict__ work) {
+// Work items of the segments of one image size, in index order from a global counter (zero at launch),
+// as in k_score.
+template <class C>
+__global__ void __launch_bounds__(C::THREADS, 1)
+k_score_segs(const SegDesc* __restrict__ segs, int n_segs, long long n_items, int* __restrict__ status,
+             unsigned long long* __restrict__ work) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ long long next_item;
+    const Sm<C> sm(smem);
+    score_tables<C>(sm);
     for (;;) {
-        // items in index order from a global counter (zero at launch), as in k_score
         if (threadIdx.x == 0) next_item = (long long)atomicAdd(work, 1ull);
         __syncthreads();
         const long long item = next_item;
@@ -1358,25 +1378,38 @@ k_score_multi(const SegDesc* __restrict__ segs, int n_segs, long long n_items, i
         const int lo = ci * sd.chunk;
         const int hi = min(lo + sd.chunk, sd.n_ps);
         const size_t row = (size_t)w * sd.n_ps;
-        switch (sd.npix) {
-            case 64:
-                score_item<M64>(smem, sd.gtw, sd.img + (size_t)w * 64 * 33, nullptr, sd.ps, 0, lo, hi, sd.s, sd.c1,
-                                sd.rec_t + row, sd.rec_s + row, sd.rec_d + row, status);
-                break;
-            case 96:
-                score_item<M96>(smem, sd.gtw, sd.img + (size_t)w * 96 * 49, nullptr, sd.ps, 0, lo, hi, sd.s, sd.c1,
-                                sd.rec_t + row, sd.rec_s + row, sd.rec_d + row, status);
-                break;
-            case 128:
-                score_item<M128>(smem, sd.gtw, sd.img + (size_t)w * 128 * 65, nullptr, sd.ps, 0, lo, hi, sd.s, sd.c1,
-                                 sd.rec_t + row, sd.rec_s + row, sd.rec_d + row, status);
-                break;
-            default:
-                score_item<M192>(smem, sd.gtw, sd.img + (size_t)w * 192 * 97, nullptr, sd.ps, 0, lo, hi, sd.s, sd.c1,
-                                 sd.rec_t + row, sd.rec_s + row, sd.rec_d + row, status);
-                break;
-        }
+        score_item<C>(sm, sd.gtw, sd.img + (size_t)w * C::N * C::H, nullptr, sd.ps, 0, lo, hi, sd.s, sd.c1, sd.rec_t + row,
+                      sd.rec_s + row, sd.rec_d + row, status);
     }
+}
+
+using SegKernel = void (*)(const SegDesc*, int, long long, int*, unsigned long long*);
+struct SegInstance {
+    SegKernel kernel;
+    int threads, smem, smax;
+    int unit;   // chunk sizes are multiples of this (the unit that tune files have always used)
+};
+
+// The instance that scores the segments of an image size (null kernel: not a batched size).
+SegInstance seg_instance(int npix) {
+    switch (npix) {
+        case 64: return {k_score_segs<C64_8>, C64_8::THREADS, (int)C64_8::SMEM, C64_8::SMAX, 15};
+        case 96: return {k_score_segs<C96_12>, C96_12::THREADS, (int)C96_12::SMEM, C96_12::SMAX, 10};
+        case 128: return {k_score_segs<C128_16>, C128_16::THREADS, (int)C128_16::SMEM, C128_16::SMAX, 7};
+        case 192: return {k_score_segs<C192_24>, C192_24::THREADS, (int)C192_24::SMEM, C192_24::SMAX, 2};
+        default: return {nullptr, 0, 0, 0, 1};
+    }
+}
+
+// Resident blocks of the instance on the whole GPU (sets the kernel's shared-memory attribute).
+int seg_slots(bioem_ctx* ctx, const SegInstance& si, int* slots) {
+    if (cudaFuncSetAttribute(si.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, si.smem) != cudaSuccess)
+        return bioem_set_error(ctx, BIOEM_ERR_CUDA, "shared memory attribute (%d bytes)", si.smem);
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, si.kernel, si.threads, si.smem) != cudaSuccess || per_sm < 1)
+        return bioem_set_error(ctx, BIOEM_ERR_CUDA, "occupancy query");
+    *slots = per_sm * ctx->num_sms;
+    return BIOEM_OK;
 }
 
 // One block per (segment, image): float64 log-sum-exp over the image's records, written as float32
@@ -1423,24 +1456,6 @@ int tuned_chunk(const std::vector<TuneEntry>& t, int npix, int s) {
     return default_chunk(npix);
 }
 
-int multi_pb(int npix) {
-    switch (npix) {
-        case 64: return M64::PB;
-        case 96: return M96::PB;
-        case 128: return M128::PB;
-        default: return M192::PB;
-    }
-}
-
-int multi_smax(int npix) {
-    switch (npix) {
-        case 64: return M64::SMAX;
-        case 96: return M96::SMAX;
-        case 128: return M128::SMAX;
-        default: return M192::SMAX;
-    }
-}
-
 }  // namespace
 
 struct bioem_batch {
@@ -1451,13 +1466,20 @@ struct bioem_batch {
     std::vector<SegDesc> segs;
     SegDesc* d_segs;
     void* d_rec;
-    unsigned long long* d_work;   // work-item counter of the scoring launch
-    long long n_items, n_rows;
+    unsigned long long* d_work;   // work-item counters of the scoring launches, one per size
+    long long n_rows;
     float* d_out;
+    // the segments [seg0, seg0 + n_segs) of one image size and their launch
+    struct Group {
+        int npix, seg0, n_segs;
+        long long n_items;
+    };
+    std::vector<Group> groups;
     cudaStream_t cap_stream;
+    std::vector<cudaStream_t> side;   // capture only: one branch per further size
+    std::vector<cudaEvent_t> events;
     cudaGraph_t graph;
     cudaGraphExec_t exec;
-    int grid;
 };
 
 // tune table kept per process (per image size and shift window)
@@ -1465,12 +1487,11 @@ static std::mutex g_tune_mutex;
 static std::vector<TuneEntry> g_tune;
 
 // An entry the batched launch can use: a batched image size, a shift window its instance covers,
-// and a chunk that is a whole number of that instance's batches, at most 4096 parameter sets.
+// and a chunk that is a whole number of that size's tuning units, at most 4096 parameter sets.
 static bool tune_entry_valid(int npix, int s, int chunk) {
-    if (npix != 64 && npix != 96 && npix != 128 && npix != 192) return false;
-    if (s < 0 || s > multi_smax(npix) || 2 * s >= npix) return false;
-    const int pb = multi_pb(npix);
-    return chunk > 0 && chunk <= 4096 && chunk % pb == 0;
+    const SegInstance si = seg_instance(npix);
+    if (!si.kernel || s < 0 || s > si.smax || 2 * s >= npix) return false;
+    return chunk > 0 && chunk <= 4096 && chunk % si.unit == 0;
 }
 
 // Read "npix shift chunk" lines into the process table.  Lines that are not three integers, or
@@ -1505,31 +1526,49 @@ static int tune_load(const char* path, int* skipped = nullptr) {
     return n;
 }
 
-static int batch_build(bioem_batch* b, int grid_override) {
+static int batch_build(bioem_batch* b) {
     bioem_ctx* ctx = b->ctx;
-    const size_t nb = sizeof(SegDesc) * b->segs.size();
+    const size_t nb = sizeof(SegDesc) * b->segs.size(), n_groups = b->groups.size();
     if (cudaMalloc((void**)&b->d_segs, nb) != cudaSuccess) return bioem_set_error(ctx, BIOEM_ERR_OOM, "segment table");
     if (cudaMemcpy(b->d_segs, b->segs.data(), nb, cudaMemcpyHostToDevice) != cudaSuccess)
         return bioem_set_error(ctx, BIOEM_ERR_CUDA, "segment table upload");
-    if (cudaMalloc((void**)&b->d_work, sizeof(unsigned long long)) != cudaSuccess)
-        return bioem_set_error(ctx, BIOEM_ERR_OOM, "work counter");
-    if (cudaFuncSetAttribute(k_score_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMultiSmem) != cudaSuccess)
-        return bioem_set_error(ctx, BIOEM_ERR_CUDA, "shared memory attribute (%zu bytes)", kMultiSmem);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_score_multi, kMultiThreads, kMultiSmem) != cudaSuccess ||
-        per_sm < 1)
-        return bioem_set_error(ctx, BIOEM_ERR_CUDA, "occupancy query");
-    long long g = (long long)per_sm * ctx->num_sms;
-    if (grid_override > 0) g = grid_override;
-    if (g > b->n_items) g = b->n_items;
-    b->grid = (int)g;
+    if (cudaMalloc((void**)&b->d_work, sizeof(unsigned long long) * n_groups) != cudaSuccess)
+        return bioem_set_error(ctx, BIOEM_ERR_OOM, "work counters");
+    std::vector<int> grids(n_groups);
+    for (size_t g = 0; g < n_groups; ++g) {
+        int slots = 0;
+        const int rc = seg_slots(ctx, seg_instance(b->groups[g].npix), &slots);
+        if (rc) return rc;
+        grids[g] = (int)(b->groups[g].n_items < slots ? b->groups[g].n_items : slots);
+    }
     if (cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
         return bioem_set_error(ctx, BIOEM_ERR_CUDA, "capture stream");
+    for (size_t g = 0; g < n_groups; ++g) {   // one side stream per further size; fork and join events
+        cudaStream_t st = nullptr;
+        cudaEvent_t ev = nullptr;
+        if (g > 0 && cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess)
+            return bioem_set_error(ctx, BIOEM_ERR_CUDA, "capture stream");
+        if (st) b->side.push_back(st);
+        if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess)
+            return bioem_set_error(ctx, BIOEM_ERR_CUDA, "capture event");
+        b->events.push_back(ev);
+    }
     if (cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
         return bioem_set_error(ctx, BIOEM_ERR_CUDA, "begin capture");
-    cudaMemsetAsync(b->d_work, 0, sizeof(unsigned long long), b->cap_stream);
-    k_score_multi<<<b->grid, kMultiThreads, kMultiSmem, b->cap_stream>>>(b->d_segs, (int)b->segs.size(), b->n_items,
-                                                                        ctx->d_status, b->d_work);
+    cudaMemsetAsync(b->d_work, 0, sizeof(unsigned long long) * n_groups, b->cap_stream);
+    cudaEventRecord(b->events[0], b->cap_stream);
+    for (size_t g = 0; g < n_groups; ++g) {
+        const bioem_batch::Group& gr = b->groups[g];
+        const SegInstance si = seg_instance(gr.npix);
+        cudaStream_t st = g == 0 ? b->cap_stream : b->side[g - 1];
+        if (g > 0) cudaStreamWaitEvent(st, b->events[0], 0);
+        si.kernel<<<grids[g], si.threads, si.smem, st>>>(b->d_segs + gr.seg0, gr.n_segs, gr.n_items, ctx->d_status,
+                                                         b->d_work + g);
+        if (g > 0) {
+            cudaEventRecord(b->events[g], st);
+            cudaStreamWaitEvent(b->cap_stream, b->events[g], 0);
+        }
+    }
     k_reduce_multi<<<(unsigned)b->n_rows, kRedThreads, 0, b->cap_stream>>>(b->d_segs, (int)b->segs.size(), b->d_out,
                                                                            b->n_cols);
     cudaError_t e = cudaStreamEndCapture(b->cap_stream, &b->graph);
@@ -1562,17 +1601,21 @@ int bioem_autotune(bioem_ctx* ctx, const bioem_images* images, const bioem_projs
             }
     }
     const int npix = images->nx;
-    if (npix != 64 && npix != 96 && npix != 128 && npix != 192)
+    const SegInstance si = seg_instance(npix);
+    if (!si.kernel)
         return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "autotune: batched sizes are 64, 96, 128, 192");
-    if (max_shift < 0 || max_shift > multi_smax(npix) || images->nx != projset->nx || images->n_img == 0 ||
+    if (max_shift < 0 || max_shift > si.smax || images->nx != projset->nx || images->n_img == 0 ||
         projset->n_ps == 0)
         return bioem_set_error(ctx, BIOEM_ERR_INVALID_ARG, "autotune: bad case");
     if (cudaSetDevice(ctx->device) != cudaSuccess) return bioem_set_error(ctx, BIOEM_ERR_CUDA, "cudaSetDevice");
     // trial: the first images (up to 2 per SM) against up to 4096 parameter sets, one segment
     const int n_img = images->n_img < 2 * ctx->num_sms ? images->n_img : 2 * ctx->num_sms;
     const int n_ps = projset->n_ps < 4096 ? projset->n_ps : 4096;
-    const int pb = multi_pb(npix);
+    const int pb = si.unit;
     const int cands[5] = {pb * 2, pb * 8, pb * 32, pb * 64, pb * 128};
+    int slots = 0;
+    const int src = seg_slots(ctx, si, &slots);
+    if (src) return src;
     void* rec = nullptr;
     const size_t rec_bytes = (size_t)n_img * n_ps * 12;
     if (cudaMalloc(&rec, rec_bytes) != cudaSuccess) return bioem_set_error(ctx, BIOEM_ERR_OOM, "autotune records");
@@ -1585,10 +1628,6 @@ int bioem_autotune(bioem_ctx* ctx, const bioem_images* images, const bioem_projs
     for (int k = 0; k < 5 && rc == BIOEM_OK; ++k) {
         const int chunk = cands[k];
         if (chunk > 2 * n_ps && k > 0) break;
-        bioem_batch b{};
-        b.ctx = ctx;
-        b.n_models = 1;
-        b.n_stacks = 1;
         SegDesc sd{};
         sd.img = images->d_spec;
         sd.ps = projset->d_spec;
@@ -1607,19 +1646,17 @@ int bioem_autotune(bioem_ctx* ctx, const bioem_images* images, const bioem_projs
         sd.nctf = projset->nctf;
         sd.c1 = 0.5f * (3.0f - (float)(npix * npix));
         sd.log_norm = 0.0;
-        b.n_items = (long long)sd.n_chunks * n_img;
-        b.segs.push_back(sd);
+        const long long n_items = (long long)sd.n_chunks * n_img;
         SegDesc* d_seg = nullptr;
         if (cudaMalloc((void**)&d_seg, sizeof(SegDesc)) != cudaSuccess) { rc = BIOEM_ERR_OOM; break; }
         cudaMemcpy(d_seg, &sd, sizeof(SegDesc), cudaMemcpyHostToDevice);
-        cudaFuncSetAttribute(k_score_multi, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMultiSmem);
-        const int grid = (int)(b.n_items < ctx->num_sms ? b.n_items : ctx->num_sms);
+        const int grid = (int)(n_items < slots ? n_items : slots);
         double ms_best_rep = 1e300;
         for (int rep = 0; rep < 3; ++rep) {
             cudaEventRecord(e0, ctx->stream);
             cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), ctx->stream);
-            k_score_multi<<<grid, kMultiThreads, kMultiSmem, ctx->stream>>>(
-                d_seg, 1, b.n_items, ctx->d_status, reinterpret_cast<unsigned long long*>(ctx->d_work));
+            si.kernel<<<grid, si.threads, si.smem, ctx->stream>>>(d_seg, 1, n_items, ctx->d_status,
+                                                                  reinterpret_cast<unsigned long long*>(ctx->d_work));
             cudaEventRecord(e1, ctx->stream);
             if (cudaEventSynchronize(e1) != cudaSuccess) { rc = bioem_check_cuda(ctx, cudaGetLastError(), "autotune"); break; }
             float ms = 0.f;
@@ -1676,8 +1713,8 @@ int bioem_batch_create(bioem_ctx* ctx, int n_models, int n_stacks, const bioem_i
         const bioem_images* im = stacks[k];
         if (!im || im->ctx != ctx) { delete b; return bioem_set_error(ctx, BIOEM_ERR_INVALID_ARG, "stack %d", k); }
         const int npix = im->nx;
-        if ((npix != 64 && npix != 96 && npix != 128 && npix != 192) || max_shift[k] < 0 ||
-            max_shift[k] > multi_smax(npix) || 2 * max_shift[k] >= npix) {
+        const SegInstance si = seg_instance(npix);
+        if (!si.kernel || max_shift[k] < 0 || max_shift[k] > si.smax || 2 * max_shift[k] >= npix) {
             delete b;
             return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "stack %d: %d px, shift %d", k, npix, max_shift[k]);
         }
@@ -1685,8 +1722,7 @@ int bioem_batch_create(bioem_ctx* ctx, int n_models, int n_stacks, const bioem_i
         col += im->n_img;
     }
     b->n_cols = col;
-    long long items = 0, rows = 0;
-    for (int m = 0; m < n_models; ++m) {
+    for (int m = 0; m < n_models; ++m) {   // every handle is checked before any segment is made
         for (int k = 0; k < n_stacks; ++k) {
             const bioem_images* im = stacks[k];
             const bioem_projset* ps = projsets[(size_t)m * n_stacks + k];
@@ -1695,7 +1731,18 @@ int bioem_batch_create(bioem_ctx* ctx, int n_models, int n_stacks, const bioem_i
                 delete b;
                 return bioem_set_error(ctx, BIOEM_ERR_INVALID_ARG, "projection set (%d, %d) does not match", m, k);
             }
-            if (im->n_img == 0) continue;
+        }
+    }
+    // segments by image size, the longest items first (the largest images)
+    long long rows = 0;
+    const int sizes[4] = {192, 128, 96, 64};
+    for (int npix : sizes) {
+        bioem_batch::Group gr{npix, (int)b->segs.size(), 0, 0};
+        for (int mk = 0; mk < n_models * n_stacks; ++mk) {
+            const int m = mk / n_stacks, k = mk - m * n_stacks;
+            const bioem_images* im = stacks[k];
+            const bioem_projset* ps = projsets[mk];
+            if (im->nx != npix || im->n_img == 0) continue;
             SegDesc sd{};
             sd.img = im->d_spec;
             sd.ps = ps->d_spec;
@@ -1717,15 +1764,16 @@ int bioem_batch_create(bioem_ctx* ctx, int n_models, int n_stacks, const bioem_i
             sd.c1 = 0.5f * (3.0f - (float)(im->nx * im->nx));
             const int S = (2 * max_shift[k] + 1) * (2 * max_shift[k] + 1);
             sd.log_norm = log((double)ps->n_ps * S);
-            sd.item_begin = items;
+            sd.item_begin = gr.n_items;
             sd.row_begin = rows;
-            items += (long long)sd.n_chunks * sd.n_img;
+            gr.n_items += (long long)sd.n_chunks * sd.n_img;
             rows += sd.n_img;
             rec_total += (size_t)sd.n_img * sd.n_ps * 12;
             b->segs.push_back(sd);
         }
+        gr.n_segs = (int)b->segs.size() - gr.seg0;
+        if (gr.n_segs) b->groups.push_back(gr);
     }
-    b->n_items = items;
     b->n_rows = rows;
     if (b->segs.empty()) { delete b; return bioem_set_error(ctx, BIOEM_ERR_INVALID_ARG, "no images"); }
     if (rows > 0x7fffffffll) { delete b; return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "too many rows"); }
@@ -1742,7 +1790,7 @@ int bioem_batch_create(bioem_ctx* ctx, int n_models, int n_stacks, const bioem_i
         sd.rec_d = reinterpret_cast<int*>(base + 2 * npair);
         off += npair * 12;
     }
-    const int rc = batch_build(b, 0);
+    const int rc = batch_build(b);
     if (rc) {
         bioem_batch_free(b);
         return rc;
@@ -1755,8 +1803,8 @@ int bioem_batch_run(bioem_batch* b) {
     if (!b) return BIOEM_ERR_INVALID_ARG;
     bioem_ctx* ctx = b->ctx;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return bioem_set_error(ctx, BIOEM_ERR_CUDA, "cudaSetDevice");
-    ctx->n_launches += 2;
-    ctx->kid_launches[KID_SCORE] += 1;
+    ctx->n_launches += b->groups.size() + 1;
+    ctx->kid_launches[KID_SCORE] += b->groups.size();
     ctx->kid_launches[KID_REDUCE_WAVE] += 1;
     return bioem_check_cuda(ctx, cudaGraphLaunch(b->exec, ctx->stream), "graph launch");
 }
@@ -1775,6 +1823,8 @@ void bioem_batch_free(bioem_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
+    for (cudaStream_t st : b->side) cudaStreamDestroy(st);
+    for (cudaEvent_t ev : b->events) cudaEventDestroy(ev);
     if (b->d_segs) cudaFree(b->d_segs);
     if (b->d_rec) cudaFree(b->d_rec);
     if (b->d_work) cudaFree(b->d_work);
@@ -1794,17 +1844,31 @@ __global__ void __launch_bounds__(C::THREADS, 1)
 k_score_gathered(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int n_img,
                  const int* __restrict__ offsets, const int* __restrict__ ps_idx, const float2* __restrict__ ps_spec,
                  int chunk, int chunks_per_img, int s, float c1, float* __restrict__ rec_t, float* __restrict__ rec_s,
-                 int* __restrict__ rec_d, int* __restrict__ status) {
+                 int* __restrict__ rec_d, int* __restrict__ status, unsigned long long* __restrict__ work) {
     extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ long long next_item;
     const long long n_items = (long long)n_img * chunks_per_img;
-    for (long long item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const Sm<C> sm(smem);
+    score_tables<C>(sm);
+    for (;;) {
+        // items in index order from a global counter (zero at launch), as in k_score; the parts of a chunk
+        // index beyond the end of an image's list are passed over by the thread that takes the items
+        if (threadIdx.x == 0) {
+            long long it;
+            do {
+                it = (long long)atomicAdd(work, 1ull);
+            } while (it < n_items && it / n_img * chunk >= offsets[it % n_img + 1] - offsets[it % n_img]);
+            next_item = it;
+        }
+        __syncthreads();
+        const long long item = next_item;   // read by every thread before score_item's first barrier
+        if (item >= n_items) break;
         const int ci = (int)(item / n_img);
         const int w = (int)(item - (long long)ci * n_img);
         const int b0 = offsets[w], b1 = offsets[w + 1];
         const int lo = ci * chunk;
         const int hi = min(lo + chunk, b1 - b0);
-        if (lo >= hi) continue;   // uniform across the block: no barrier is skipped by a subset
-        score_item<C>(smem, gtw, img_spec + (size_t)w * C::N * C::H, ps_idx + b0, ps_spec, 0, lo, hi, s, c1,
+        score_item<C>(sm, gtw, img_spec + (size_t)w * C::N * C::H, ps_idx + b0, ps_spec, 0, lo, hi, s, c1,
                       rec_t + b0, rec_s + b0, rec_d + b0, status);
     }
 }
@@ -1919,17 +1983,23 @@ int run_gathered(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_score_gathered<C>, C::THREADS, smem);
     if (per_sm < 1) per_sm = 1;
-    const int chunk = 256 / C::PB * C::PB;   // whole batches
+    const int slots = per_sm * ctx->num_sms;
+    // chunks as for lists of the mean length (at most 256 sets: 16 MB of the chunk's projections at 128 px)
+    int chunk = nnz >= n_img ? score_chunk<C>(n_img, (nnz + n_img - 1) / n_img, slots) : C::GPB;
+    if (chunk > 256 / C::GPB * C::GPB) chunk = 256 / C::GPB * C::GPB;
     const int cpi = (max_per_image + chunk - 1) / chunk;
     const long long items = (long long)n_img * cpi;
-    const int grid = (int)(items < (long long)per_sm * ctx->num_sms ? items : (long long)per_sm * ctx->num_sms);
+    const int grid = (int)(items < slots ? items : slots);
     const int n = C::N * C::N;
     if (grid > 0) {
         bioem_launch_begin(ctx, KID_SCORE);
+        if (cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), ctx->stream) != cudaSuccess)
+            return bioem_check_cuda(ctx, cudaGetLastError(), "work counter");
         k_score_gathered<C><<<grid, C::THREADS, smem, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, offsets,
                                                                      ps_idx, ps->d_spec, chunk, cpi, max_shift,
                                                                      0.5f * (3.0f - (float)n), rec_t, rec_s, rec_d,
-                                                                     ctx->d_status);
+                                                                     ctx->d_status,
+                                                                     reinterpret_cast<unsigned long long*>(ctx->d_work));
         bioem_launch_end(ctx, KID_SCORE);
         int rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_score_gathered");
         if (rc) return rc;
