@@ -677,89 +677,124 @@ struct Acc {
 };
 
 constexpr int kRedThreads = 256;
-constexpr int kExpBits = 6;   // table of 2^(j / 64)
-constexpr double kExpMin = -100.0;
+constexpr int kExpBits = 8;   // table of 2^(j / 256)
+__device__ double g_exp2[1 << kExpBits];   // uploaded with the twiddle tables
 
-// exp(x) for x in [kExpMin, 0]: x = (64 q + j) ln2 / 64 + r, |r| <= ln2 / 128, exp(x) = 2^q 2^(j/64) e^r with the Taylor
-// series of e^r to r^5 (truncation below 4e-17), the table-driven scheme of Tang (ACM TOMS 15, 1989).  Ten
-// float64 operations; the reductions below are bound by the float64 pipe (1/70 of the FP32 rate).
+// exp(x) for x in [-100, 0]: x = (256 q + j) ln2 / 256 + r, |r| <= ln2 / 512, exp(x) = 2^q 2^(j/256) e^r with the
+// Taylor series of e^r to r^4 (truncation below 4e-17), the table-driven scheme of Tang (ACM TOMS 15,
+// 1989).  ln2 / 256 as one float64 is 9e-20 off per step of 1 / 256: 5e-16 of the result at x = -16, where the
+// term is 1e-7 of the sum.  Eight float64 operations: the reductions below are bound by the float64 pipe (1/70
+// of the FP32 rate), so what can be an integer operation (comparisons, scaling) is one.
 __device__ __forceinline__ double exp_neg(double x, const double* tab) {
     const double big = 6755399441055744.0;   // 1.5 * 2^52: adding it rounds to an integer in the low word
-    const double kd = fma(x, 92.33248261689366, big);   // 64 / ln 2
+    const double kd = fma(x, 369.32993046757463, big);   // 256 / ln 2
     const int k = __double2loint(kd);
     const double n = kd - big;
-    double r = fma(n, -1.0830424696249145e-2, x);            // ln 2 / 64, leading part and the rest
-    r = fma(n, -3.623510646634843e-19, r);
-    double p = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    p = fma(r, p, 1.0 / 6.0);
+    const double r = fma(n, -0.0027076061740622863, x);   // ln 2 / 256
+    double p = fma(r, 1.0 / 24.0, 1.0 / 6.0);
     p = fma(r, p, 0.5);
     p = fma(r, p, 1.0);
-    const double t = tab[k & 63];
+    const double t = tab[k & ((1 << kExpBits) - 1)];
     const double v = fma(t, r * p, t);
     return __hiloint2double(__double2hiint(v) + (k >> kExpBits) * (1 << 20), __double2loint(v));
 }
 
-// Folds four terms s_i exp(m_i) (m = -inf: none) into (M, S), ln sum = M + ln S; returns the index of the first
-// term that is a new maximum, or -1.  Terms more than 100 below the maximum cannot change S (S >= 1: the
-// maximum's own s is at least 1) and are left out.
-__device__ __forceinline__ int lse_add4(double& M, double& S, const double (&m)[4], const float (&s)[4], const double* tab) {
-    int at = -1;
-    const double mx = fmax(fmax(m[0], m[1]), fmax(m[2], m[3]));
-    if (mx > M) {
-        at = m[0] == mx ? 0 : m[1] == mx ? 1 : m[2] == mx ? 2 : 3;
-        S = M - mx > kExpMin ? S * exp_neg(M - mx, tab) : 0.0;
-        M = mx;
+// Order-preserving integer of a float64 that is not NaN, and back.
+__device__ __forceinline__ long long d_key(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double key_d(long long k) { return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll)); }
+constexpr long long kKeyNone = (long long)0x800fffffffffffffull;   // -inf
+
+// d > -100 for a difference d <= 0 that is not NaN, by its high word
+__device__ __forceinline__ bool in_reach(double d) { return (unsigned)__double2hiint(d) < 0xc0590000u; }
+
+// s exp(d) for d <= 0 that is not NaN; 0 beyond the reach
+__device__ __forceinline__ double scaled_exp(double s, double d, const double* tab) {
+    return in_reach(d) ? s * exp_neg(d, tab) : 0.0;
+}
+
+// Running ln sum = M + ln S; key: of M (kKeyNone: empty).
+struct Lse {
+    double M = -INFINITY, S = 0.0;
+    long long key = kKeyNone;
+};
+
+// Folds four terms s_i exp(m_i) (m = -inf or NaN: none) into a; returns the index of the first term that is a
+// new maximum, or -1.  Terms more than 100 below the maximum cannot change S (S >= 1: the maximum's own
+// s is at least 1) and are left out.
+__device__ __forceinline__ int lse_add4(Lse& a, const double (&m)[4], const float (&s)[4], const double* tab) {
+    long long k[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        k[i] = d_key(m[i]);
+        if ((__double2hiint(m[i]) & 0x7fffffff) >= 0x7ff00000) k[i] = kKeyNone;   // NaN, -inf (+inf does not occur)
     }
-    bool any = false;
+    const long long mx = max(max(k[0], k[1]), max(k[2], k[3]));
+    int at = -1;
+    if (mx > a.key) {
+        at = k[0] == mx ? 0 : k[1] == mx ? 1 : k[2] == mx ? 2 : 3;
+        const double mv = key_d(mx);
+        if (a.key != kKeyNone) a.S = scaled_exp(a.S, a.M - mv, tab);
+        a.M = mv;
+        a.key = mx;
+    }
+    if (a.key == kKeyNone) return at;
+    bool use[4], any = false;
     double d[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        d[i] = m[i] - M;
-        any |= d[i] > kExpMin;
+        d[i] = m[i] - a.M;
+        use[i] = k[i] != kKeyNone && in_reach(d[i]);
+        any |= use[i];
     }
     if (any) {
         double e[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) e[i] = exp_neg(d[i] > kExpMin ? d[i] : 0.0, tab);
+        for (int i = 0; i < 4; ++i) e[i] = exp_neg(use[i] ? d[i] : 0.0, tab);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) S = fma(d[i] > kExpMin ? (double)s[i] : 0.0, e[i], S);
+        for (int i = 0; i < 4; ++i) a.S = fma((double)(use[i] ? s[i] : 0.f), e[i], a.S);
     }
     return at;
 }
 
 __device__ __forceinline__ void exp_table(double* tab) {
-    if (threadIdx.x < (1 << kExpBits)) tab[threadIdx.x] = exp2((double)threadIdx.x / (1 << kExpBits));
+    for (int i = threadIdx.x; i < (1 << kExpBits); i += kRedThreads) tab[i] = g_exp2[i];
 }
 
-// The warp's (M, S, best set) merged into every lane, lanes in a fixed order; bp = the lowest set of the maximum.
-__device__ __forceinline__ void warp_lse(double& M, double& S, int& bp) {
-    double mx = M;
+// The warp's sums and best set merged into every lane, lanes in a fixed order; bp = the lowest set of the maximum.
+__device__ __forceinline__ void warp_lse(Lse& a, int& bp, const double* tab) {
+    long long mx = a.key;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    S = (M > -INFINITY) ? S * exp(M - mx) : 0.0;
-    if (!(M == mx)) bp = 0x7fffffff;
-    M = mx;
+    for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    const double mv = key_d(mx);
+    a.S = a.key != kKeyNone ? scaled_exp(a.S, a.M - mv, tab) : 0.0;
+    if (a.key != mx) bp = 0x7fffffff;
+    a.M = mv;
+    a.key = mx;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
-        S += __shfl_xor_sync(0xffffffffu, S, off);
+        a.S += __shfl_xor_sync(0xffffffffu, a.S, off);
         bp = min(bp, __shfl_xor_sync(0xffffffffu, bp, off));
     }
 }
 
 // The same over a block of kRedThreads, valid in warp 0.
-__device__ __forceinline__ void block_lse(double& M, double& S, int& bp) {
+__device__ __forceinline__ void block_lse(Lse& a, int& bp, const double* tab) {
     constexpr int W = kRedThreads / 32;
     __shared__ double rM[W], rS[W];
+    __shared__ long long rk[W];
     __shared__ int rb[W];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    warp_lse(M, S, bp);
-    if (lane == 0) { rM[warp] = M; rS[warp] = S; rb[warp] = bp; }
+    warp_lse(a, bp, tab);
+    if (lane == 0) { rM[warp] = a.M; rS[warp] = a.S; rk[warp] = a.key; rb[warp] = bp; }
     __syncthreads();
     if (warp == 0) {
-        M = lane < W ? rM[lane] : -INFINITY;
-        S = lane < W ? rS[lane] : 0.0;
-        bp = lane < W ? rb[lane] : 0x7fffffff;
-        warp_lse(M, S, bp);
+        a = Lse{};
+        bp = 0x7fffffff;
+        if (lane < W) { a.M = rM[lane]; a.S = rS[lane]; a.key = rk[lane]; bp = rb[lane]; }
+        warp_lse(a, bp, tab);
     }
 }
 
@@ -779,8 +814,8 @@ __device__ __forceinline__ void acc_merge_prev(Acc& r, const Acc& prev) {
 // and, if requested, write the per-orientation posteriors of the share's orientations.  Parts are whole
 // orientations; an image is cut into enough of them to occupy the GPU (reduce_parts).  An image in one part
 // is folded in place (parts = prev = the running accumulators; prev null: the first wave).  Bound by the
-// float64 pipe: one exponential per record for each of the two outputs (64 images x 6912 sets: 93 us as one
-// block per image, 39 us so; 16 images with per-orientation output: 181 -> 32 us).
+// float64 pipe (13 operations per record; 64 images x 6912 sets: 93 us as one block per image with the
+// library's exponential, 28 us so; 16 images with per-orientation output: 181 -> 15 us).
 __global__ void __launch_bounds__(kRedThreads) k_reduce_wave(
     const float* __restrict__ rec_t, const float* __restrict__ rec_s, const int* __restrict__ rec_d,
     const double* __restrict__ kA, const double* __restrict__ kB, int ps_begin, int wave_len, int nctf,
@@ -794,44 +829,50 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_wave(
     const size_t base = (size_t)w * wave_len;
     exp_table(tab);
     __syncthreads();
-    double M = -INFINITY, S = 0.0;
+    Lse a;
     int bp = 0x7fffffff;
-    const int lo = q0 * nctf, hi = q1 * nctf;
-    for (int p = lo + threadIdx.x; p < hi; p += 4 * kRedThreads) {
-        double m[4];
-        float sv[4];
+    auto term = [&](int p, bool ok, double& m, float& sv) {
+        m = ok ? ka + kB[ps_begin + p] + c1 * (double)rec_t[base + p] : -INFINITY;
+        sv = ok ? rec_s[base + p] : 0.f;
+    };
+    double m[4];
+    float sv[4];
+    if (!logP_orient) {
+        const int lo = q0 * nctf, hi = q1 * nctf;
+        for (int p = lo + threadIdx.x; p < hi; p += 4 * kRedThreads) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int pi = p + i * kRedThreads;
-            m[i] = pi < hi ? ka + kB[ps_begin + pi] + c1 * (double)rec_t[base + pi] : -INFINITY;
-            sv[i] = pi < hi ? rec_s[base + pi] : 0.f;
+            for (int i = 0; i < 4; ++i) term(p + i * kRedThreads, p + i * kRedThreads < hi, m[i], sv[i]);
+            const int at = lse_add4(a, m, sv, tab);
+            if (at >= 0) bp = p + at * kRedThreads;
         }
-        const int at = lse_add4(M, S, m, sv, tab);
-        if (at >= 0) bp = p + at * kRedThreads;
+    } else {
+        // an orientation per thread: its sum over the PSFs is an output and one term of the image's sum
+        for (int ql = q0 + threadIdx.x; ql < q1; ql += kRedThreads) {
+            Lse o;
+            int op = 0x7fffffff;
+            for (int c = 0; c < nctf; c += 4) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) term(ql * nctf + c + i, c + i < nctf, m[i], sv[i]);
+                const int at = lse_add4(o, m, sv, tab);
+                if (at >= 0) op = ql * nctf + c + at;
+            }
+            logP_orient[(size_t)w * nq + ps_begin / nctf + ql] = o.M + log(o.S) - log_norm_orient;
+            if (o.key > a.key) {
+                a.S = a.key != kKeyNone ? o.S + scaled_exp(a.S, a.M - o.M, tab) : o.S;
+                a.M = o.M;
+                a.key = o.key;
+                bp = op;
+            } else if (o.key != kKeyNone) {
+                a.S += scaled_exp(o.S, o.M - a.M, tab);
+            }
+        }
     }
-    block_lse(M, S, bp);
+    block_lse(a, bp, tab);
     if (threadIdx.x == 0) {
         const bool any = bp != 0x7fffffff;
-        Acc r{M, S, any ? M : -INFINITY, any ? ps_begin + bp : 0x7fffffff, any ? rec_d[base + bp] : 0};
+        Acc r{a.M, a.S, any ? a.M : -INFINITY, any ? ps_begin + bp : 0x7fffffff, any ? rec_d[base + bp] : 0};
         if (prev) acc_merge_prev(r, prev[w]);
         parts[blockIdx.x] = r;
-    }
-    if (logP_orient) {
-        for (int ql = q0 + threadIdx.x; ql < q1; ql += kRedThreads) {
-            double Mq = -INFINITY, Sq = 0.0;
-            for (int c = 0; c < nctf; c += 4) {
-                double m[4];
-                float sv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int p = ql * nctf + c + i;
-                    m[i] = c + i < nctf ? ka + kB[ps_begin + p] + c1 * (double)rec_t[base + p] : -INFINITY;
-                    sv[i] = c + i < nctf ? rec_s[base + p] : 0.f;
-                }
-                lse_add4(Mq, Sq, m, sv, tab);
-            }
-            logP_orient[(size_t)w * nq + ps_begin / nctf + ql] = Mq + log(Sq) - log_norm_orient;
-        }
     }
 }
 
@@ -841,19 +882,23 @@ __global__ void __launch_bounds__(kRedThreads) k_finalize(Acc* acc, const Acc* p
                                                           int n_parts, int first, int last, int n_img, double log_norm,
                                                           int nctf, int nsk, int smax, double* logP, int* best_q,
                                                           int* best_ctf, int* best_dx, int* best_dy, double* best_logL) {
+    __shared__ double tab[1 << kExpBits];
     const int w = blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    exp_table(tab);
+    __syncthreads();
     if (w >= n_img) return;
     Acc a{-INFINITY, 0.0, -INFINITY, 0x7fffffff, 0};
     if (lane < n_parts) a = (parts ? parts : acc)[(size_t)w * n_parts + lane];
     Acc prev{-INFINITY, 0.0, -INFINITY, 0x7fffffff, 0};
     if (!first) prev = acc[w];
-    double M = a.M, S = a.S;
+    Lse l;
+    if (a.M > -INFINITY) { l.M = a.M; l.S = a.S; l.key = d_key(a.M); }
     int bp = a.bp;
-    warp_lse(M, S, bp);
+    warp_lse(l, bp, tab);
     const int src = __ffs(__ballot_sync(0xffffffffu, bp != 0x7fffffff && a.bp == bp)) - 1;
     const int bd = __shfl_sync(0xffffffffu, a.bd, src < 0 ? 0 : src);
     if (lane != 0) return;
-    Acc r{M, S, bp != 0x7fffffff ? M : -INFINITY, bp, bd};
+    Acc r{l.M, l.S, bp != 0x7fffffff ? l.M : -INFINITY, bp, bd};
     acc_merge_prev(r, prev);
     acc[w] = r;
     if (!last) return;
@@ -899,11 +944,11 @@ __global__ void k_fold_acc(const Acc* __restrict__ acc, int n_img, double* __res
 }
 
 // ---------------------------------------------------------------------------- host side
-// Parts per image of the wave reduction: about four blocks per SM over all images, each of at least 512
-// records and one orientation, at most 32 (one lane each in k_finalize).
+// Parts per image of the wave reduction: about four blocks per SM over all images, each of at least 1024
+// records (four per thread) and one orientation, at most 32 (one lane each in k_finalize).
 int reduce_parts(const bioem_ctx* ctx, int n_img, long long wave, int nctf) {
     long long n = 4ll * ctx->num_sms / n_img;
-    if (n > wave / 512) n = wave / 512;
+    if (n > wave / (4 * kRedThreads)) n = wave / (4 * kRedThreads);
     if (n > wave / nctf) n = wave / nctf;
     return (int)(n < 1 ? 1 : n > 32 ? 32 : n);
 }
@@ -1194,7 +1239,9 @@ int bioem_upload_score_twiddles(bioem_ctx* ctx) {
         }
         if (e != cudaSuccess) return bioem_check_cuda(ctx, e, "twiddle upload");
     }
-    return BIOEM_OK;
+    double t[1 << kExpBits];
+    for (int j = 0; j < (1 << kExpBits); ++j) t[j] = exp2((double)j / (1 << kExpBits));
+    return bioem_check_cuda(ctx, cudaMemcpyToSymbol(g_exp2, t, sizeof(t)), "exponential table upload");
 }
 
 // ---------------------------------------------------------------------------- allocation-free scoring
@@ -1425,7 +1472,7 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_multi(const SegDesc* __r
     const double c1 = (double)sd.c1;
     exp_table(tab);
     __syncthreads();
-    double M = -INFINITY, S = 0.0;
+    Lse a;
     int bp = 0x7fffffff;
     const size_t base = (size_t)w * sd.n_ps;
     for (int p = threadIdx.x; p < sd.n_ps; p += 4 * kRedThreads) {
@@ -1437,11 +1484,11 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_multi(const SegDesc* __r
             m[i] = pi < sd.n_ps ? ka + sd.kB[pi] + c1 * (double)sd.rec_t[base + pi] : -INFINITY;
             sv[i] = pi < sd.n_ps ? sd.rec_s[base + pi] : 0.f;
         }
-        lse_add4(M, S, m, sv, tab);
+        lse_add4(a, m, sv, tab);
     }
-    block_lse(M, S, bp);
+    block_lse(a, bp, tab);
     if (threadIdx.x == 0)
-        out[(size_t)sd.out_row * out_ld + sd.out_col + w] = (float)(M + log(S) - sd.log_norm);
+        out[(size_t)sd.out_row * out_ld + sd.out_col + w] = (float)(a.M + log(a.S) - sd.log_norm);
 }
 
 struct TuneEntry {
@@ -1885,7 +1932,7 @@ __global__ void __launch_bounds__(kRedThreads) k_fold_gathered(const int* __rest
     const int b0 = offsets[w], b1 = offsets[w + 1];
     exp_table(tab);
     __syncthreads();
-    double M = -INFINITY, S = 0.0;
+    Lse a;
     int bp = 0x7fffffff;
     for (int i0 = b0 + threadIdx.x; i0 < b1; i0 += 4 * kRedThreads) {
         double m[4];
@@ -1896,11 +1943,11 @@ __global__ void __launch_bounds__(kRedThreads) k_fold_gathered(const int* __rest
             m[k] = i < b1 ? kA[w] + kB[ps_idx[i]] + c1 * (double)rec_t[i] : -INFINITY;
             sv[k] = i < b1 ? rec_s[i] : 0.f;
         }
-        lse_add4(M, S, m, sv, tab);
+        lse_add4(a, m, sv, tab);
     }
-    block_lse(M, S, bp);
+    block_lse(a, bp, tab);
     if (threadIdx.x == 0) {
-        Acc r{M, S, -INFINITY, 0, 0};
+        Acc r{a.M, a.S, -INFINITY, 0, 0};
         if (!first) acc_merge_prev(r, Acc{acc[2 * w], acc[2 * w + 1], -INFINITY, 0, 0});
         acc[2 * w] = r.M;
         acc[2 * w + 1] = r.S;
