@@ -31,7 +31,7 @@ namespace {
 
 constexpr int kLayers = 6;
 constexpr int kT = 256;
-constexpr int kFeatSplits = 4;   // k splits of the feature gradient (its parts need F kFeatSplits <= C S^2 = 64 F)
+constexpr int kFeatSplits = 16;   // most k splits of the feature gradient (its parts need F kFeatSplits <= C S^2 = 64 F)
 
 struct Layer {
     int cin, cout, stride, hin, hout;
@@ -40,41 +40,59 @@ struct Layer {
 };
 
 // ------------------------------------------------------------------ input preparation
-// out[b][y][x] = standardised 2x2 average of img[b]; per image: zero mean, unit variance over S^2.
+// out[b][y][x] = standardised down x down average of img[b]; per image: zero mean, unit variance over S^2
+// (float64 sums per thread, then over lanes and warps in order).  Bound by float64 arithmetic, so few threads
+// with many pixels each: a sum over more lanes costs more float64 additions than the pixels.
 __global__ void __launch_bounds__(kT) k_downsample_norm(const float* __restrict__ img, int n_in, int down,
                                                         float* __restrict__ out) {
     const int b = blockIdx.x;
     const int S = n_in / down;
     const float* src = img + (size_t)b * n_in * n_in;
     float* dst = out + (size_t)b * S * S;
-    __shared__ double r1[kT], r2[kT];
+    __shared__ double r1[kT / 32], r2[kT / 32];
     double s1 = 0.0, s2 = 0.0;
-    for (int i = threadIdx.x; i < S * S; i += blockDim.x) {
-        const int y = i / S, x = i - (i / S) * S;
+#pragma unroll 4
+    for (int i = threadIdx.x; i < S * S; i += kT) {
+        const int y = i / S, x = i - y * S;
         float v = 0.f;
-        for (int dy = 0; dy < down; ++dy)
-            for (int dx = 0; dx < down; ++dx) v += src[(y * down + dy) * n_in + x * down + dx];
+        if (down == 2) {
+            const float* p = src + (size_t)(2 * y) * n_in + 2 * x;
+            v = v + __ldg(p) + __ldg(p + 1) + __ldg(p + n_in) + __ldg(p + n_in + 1);
+        } else {
+            for (int dy = 0; dy < down; ++dy)
+                for (int dx = 0; dx < down; ++dx) v += src[(size_t)(y * down + dy) * n_in + x * down + dx];
+        }
         v *= 1.0f / (float)(down * down);
         dst[i] = v;
-        s1 += v;
-        s2 += (double)v * v;
+        const double d = v;
+        s1 += d;
+        s2 = fma(d, d, s2);
     }
-    r1[threadIdx.x] = s1;
-    r2[threadIdx.x] = s2;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+        s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        r1[threadIdx.x >> 5] = s1;
+        r2[threadIdx.x >> 5] = s2;
+    }
+    __shared__ float stat[2];
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) {
-            r1[threadIdx.x] += r1[threadIdx.x + st];
-            r2[threadIdx.x] += r2[threadIdx.x + st];
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kT / 32; ++w) {
+            s1 += r1[w];
+            s2 += r2[w];
         }
-        __syncthreads();
+        const double n = (double)S * S;
+        const double mean = s1 / n;
+        const double var = s2 / n - mean * mean;
+        stat[0] = (float)mean;
+        stat[1] = var > 0.0 ? (float)(1.0 / sqrt(var)) : 0.f;
     }
-    const double n = (double)S * S;
-    const double mean = r1[0] / n;
-    const double var = r2[0] / n - mean * mean;
-    const float inv = var > 0.0 ? (float)(1.0 / sqrt(var)) : 0.f;
-    const float m = (float)mean;
-    for (int i = threadIdx.x; i < S * S; i += blockDim.x) dst[i] = (dst[i] - m) * inv;
+    __syncthreads();
+    const float m = stat[0], inv = stat[1];
+    for (int i = threadIdx.x; i < S * S; i += kT) dst[i] = (dst[i] - m) * inv;
 }
 
 // ------------------------------------------------------------------ convolution
@@ -84,8 +102,9 @@ __global__ void __launch_bounds__(kT) k_downsample_norm(const float* __restrict_
 // loaded once serves 3 CO products per value and a weight serves XT; the products of two channels go
 // out as one packed FP32 pair.  Every output is still summed in the order (ci, ky, kx) starting from
 // the bias, with the taps outside the image left out, so the activations do not depend on the tiling.
-// Bound by the FP32 pipe.  CO = 16 has the fewest loads per product; fewer channels per thread are
-// taken where that would leave too few blocks (conv_co).  VEC: rows read as float4 with the edge
+// Bound by the FP32 pipe (42 of 73 TFLOP/s at 32 x 32 px, 256 samples: 12-16 warps per SM).  CO = 16 has the
+// fewest loads per product; fewer channels per thread are taken where that would leave too few
+// blocks (conv_co).  Loading the next channel's rows ahead gained nothing (registers for warps).  VEC: rows read as float4 with the edge
 // values from the neighbouring lanes (needs output rows of whole groups of four).
 constexpr int XT = 4;
 constexpr int kConvT = 128;
@@ -95,7 +114,7 @@ constexpr int kConvT = 128;
 // (cin, cout are then the layer's output and input channels); no bias, and the ReLU that produced the
 // layer's input (mask = that input) is applied to the result instead of in a pass of its own.
 template <int CO, int STRIDE, bool VEC, bool BWD>
-__global__ void __launch_bounds__(kConvT) k_conv(const float* __restrict__ in, const __half* __restrict__ W,
+__global__ void __launch_bounds__(kConvT, 4) k_conv(const float* __restrict__ in, const __half* __restrict__ W,
                                                  const __half* __restrict__ bias, const float* __restrict__ mask,
                                                  int cin, int cout, int hin, int hout, int groups, long long n_tasks,
                                                  float* __restrict__ out) {
@@ -310,34 +329,38 @@ __global__ void __launch_bounds__(kConvT) k_conv_bwd_data2(const float* __restri
 // Weight gradients gW[co][ci][ky][kx] = sum_{b,y,x} gout[b][co][y][x] in[b][ci][y s + ky - 1][x s + kx - 1] and bias
 // gradients gb[co] = sum_{b,y,x} gout[b][co][y][x], as partial sums per block (k_conv_wgrad_sum adds them in
 // block order: deterministic).  A block holds 32 x 32 channels x 9 taps, 2 x 2 x 9 sums per thread, and
-// walks over tiles of WR output rows x at most kWgX columns of one sample staged in shared memory
-// (inputs with a border of zeros), four columns at a time: 144 products per 14 (stride 1) or 20 (stride 2) shared reads, against
-// one read per product when each (co, ci) pair was a block of its own.  Bound by the FP32 pipe.
-// Channel strides are 4 x odd floats, so the 16-byte reads of 8 neighbouring channels do not conflict.
+// walks over tiles of WR output rows x GW columns of one sample staged in shared memory (outside values
+// zero), four columns at a time: 144 products per 14-16 shared reads, against one read per product when
+// each (co, ci) pair was a block of its own.  Bound by the FP32 pipe.  All of a tile's loads are in flight
+// together (row by row, each waited for, they took longer than the products: 281 us for the 32 x 32 px stride-1
+// layer of 256 samples against 115).  Channel strides are 4 x odd floats, so the 16-byte reads of 8
+// neighbouring channels do not conflict.
 constexpr int kWgT = 256, kWgC = 32, kWgX = 64;
 
-__host__ __device__ constexpr int wg_rows(int stride) { return stride == 1 ? 4 : 2; }   // output rows per strip
-__host__ __device__ constexpr int odd4(int n) { return ((n + 3) / 4 | 1) * 4; }          // >= n, 4 x odd
-__host__ __device__ inline int wg_gw(int hout) { return hout < kWgX ? (hout + 3) / 4 * 4 : kWgX; }   // staged gout row
-__host__ __device__ inline int wg_iw(int hout, int stride) { return (wg_gw(hout) * stride + 2 + 3) / 4 * 4; }
-__host__ __device__ inline int wg_gch(int hout, int stride) { return odd4(wg_rows(stride) * wg_gw(hout)); }
-__host__ __device__ inline int wg_ich(int hout, int stride) {
-    return odd4(((wg_rows(stride) - 1) * stride + 3) * wg_iw(hout, stride));
-}
+__host__ __device__ constexpr int odd4(int n) { return ((n + 3) / 4 | 1) * 4; }   // >= n, 4 x odd
 
-template <int STRIDE>
+template <int STRIDE, int GW>
+struct WgTile {
+    static constexpr int WR = STRIDE == 1 ? (GW == 8 ? 8 : 128 / GW) : 64 / GW;   // output rows
+    static constexpr int IR = (WR - 1) * STRIDE + 3;                                // input rows
+    static constexpr int IW = STRIDE == 1 ? GW + 8 : 2 * GW + 4;   // staged input row: column ix at ix + 4
+    static constexpr int GCH = odd4(WR * GW), ICH = odd4(IR * IW);   // channel strides
+    static constexpr size_t SMEM = (size_t)kWgC * (GCH + ICH) * sizeof(float);
+};
+
+// VEC: rows of whole groups of four (16-byte loads).
+template <int STRIDE, int GW, bool VEC>
 __global__ void __launch_bounds__(kWgT, 2) k_conv_wgrad(const float* __restrict__ gout, const float* __restrict__ in,
                                                         int B, int cin, int cout, int hin, int hout,
                                                         float* __restrict__ part) {
-    constexpr int WR = wg_rows(STRIDE), IR = (WR - 1) * STRIDE + 3;
+    using W = WgTile<STRIDE, GW>;
+    constexpr int WR = W::WR, IR = W::IR, IW = W::IW, GCH = W::GCH, ICH = W::ICH;
     extern __shared__ __align__(16) float sm[];
-    const int gw = wg_gw(hout), iw = wg_iw(hout, STRIDE), gch = wg_gch(hout, STRIDE), ich = wg_ich(hout, STRIDE);
-    float* gs = sm;                   // [32 co][WR][gw]
-    float* is = sm + kWgC * gch;      // [32 ci][IR][iw], column ix + 1
+    float* gs = sm;                   // [32 co][WR][GW]
+    float* is = sm + kWgC * GCH;      // [32 ci][IR][IW]
     const int nci = (cin + kWgC - 1) / kWgC;
     const int co0 = (int)blockIdx.y / nci * kWgC, ci0 = (int)blockIdx.y % nci * kWgC;
     const int tc = threadIdx.x & 15, to = threadIdx.x >> 4;   // ci = ci0 + tc + 16 j, co = co0 + to + 16 i
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     float acc[2][2][9], sb[2] = {0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < 2; ++i)
@@ -345,57 +368,99 @@ __global__ void __launch_bounds__(kWgT, 2) k_conv_wgrad(const float* __restrict_
         for (int j = 0; j < 2; ++j)
 #pragma unroll
             for (int k = 0; k < 9; ++k) acc[i][j][k] = 0.f;
-    const int tiles_x = (hout + gw - 1) / gw, tiles = (hout + WR - 1) / WR * tiles_x;
+    // four values of a row from column x (all of them inside or outside the row with VEC)
+    auto load4 = [](const float* row, int x, int n, bool ok) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (VEC) {
+            if (ok && x < n) v = __ldg(reinterpret_cast<const float4*>(row + x));
+        } else if (ok) {
+            if (x < n) v.x = __ldg(row + x);
+            if (x + 1 < n) v.y = __ldg(row + x + 1);
+            if (x + 2 < n) v.z = __ldg(row + x + 2);
+            if (x + 3 < n) v.w = __ldg(row + x + 3);
+        }
+        return v;
+    };
+    const int tiles_x = (hout + GW - 1) / GW, tiles = (hout + WR - 1) / WR * tiles_x;
     const long long units = (long long)B * tiles;
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
         const int b = (int)(u / tiles), t = (int)(u - (long long)b * tiles);
-        const int y0 = t / tiles_x * WR, xs = t % tiles_x * gw;
-        __syncthreads();   // the previous tile has been read
-        for (int r = warp; r < kWgC * WR; r += kWgT / 32) {
-            const int c = r / WR, y = r - c * WR;
-            const float* src = gout + (((size_t)b * cout + co0 + c) * hout + y0 + y) * hout + xs;
-            const bool ok = co0 + c < cout && y0 + y < hout;
-            for (int x = lane; x < gw; x += 32) gs[c * gch + y * gw + x] = ok && xs + x < hout ? __ldg(src + x) : 0.f;
+        const int y0 = t / tiles_x * WR, xs = t % tiles_x * GW;
+        constexpr int NG = kWgC * WR * (GW / 4), NI = kWgC * IR * (GW * STRIDE / 4), NE = kWgC * IR * 2;
+        constexpr int PG = (NG + kWgT - 1) / kWgT, PI = (NI + kWgT - 1) / kWgT, PE = (NE + kWgT - 1) / kWgT;
+        float4 vg[PG], vi[PI];
+        float ve[PE];
+#pragma unroll
+        for (int k = 0; k < PG; ++k) {
+            const int e = threadIdx.x + k * kWgT, x = e % (GW / 4) * 4, y = e / (GW / 4) % WR, c = e / (GW / 4 * WR);
+            const bool ok = e < NG && co0 + c < cout && y0 + y < hout;
+            vg[k] = load4(gout + (((size_t)b * cout + co0 + c) * hout + y0 + y) * hout, xs + x, hout, ok);
         }
-        for (int r = warp; r < kWgC * IR; r += kWgT / 32) {
-            const int c = r / IR, y = r - c * IR;
+#pragma unroll
+        for (int k = 0; k < PI; ++k) {
+            constexpr int Q = GW * STRIDE / 4;
+            const int e = threadIdx.x + k * kWgT, x = e % Q * 4, y = e / Q % IR, c = e / (Q * IR);
             const int iy = y0 * STRIDE + y - 1;
-            const float* src = in + (((size_t)b * cin + ci0 + c) * hin + iy) * hin;
-            const bool ok = ci0 + c < cin && iy >= 0 && iy < hin;
-            for (int x = lane; x < iw; x += 32) {
-                const int ix = xs * STRIDE + x - 1;
-                is[c * ich + y * iw + x] = ok && ix >= 0 && ix < hin ? __ldg(src + ix) : 0.f;
-            }
+            const bool ok = e < NI && ci0 + c < cin && iy >= 0 && iy < hin;
+            vi[k] = load4(in + (((size_t)b * cin + ci0 + c) * hin + iy) * hin, xs * STRIDE + x, hin, ok);
+        }
+#pragma unroll
+        for (int k = 0; k < PE; ++k) {   // the columns left and right of the tile
+            const int e = threadIdx.x + k * kWgT, y = e / 2 % IR, c = e / (2 * IR);
+            const int iy = y0 * STRIDE + y - 1, ix = e & 1 ? (xs + GW) * STRIDE : xs * STRIDE - 1;
+            const bool ok = e < NE && ci0 + c < cin && iy >= 0 && iy < hin && ix >= 0 && ix < hin;
+            ve[k] = ok ? __ldg(in + (((size_t)b * cin + ci0 + c) * hin + iy) * hin + ix) : 0.f;
+        }
+        __syncthreads();   // the previous tile has been read
+#pragma unroll
+        for (int k = 0; k < PG; ++k) {
+            const int e = threadIdx.x + k * kWgT, x = e % (GW / 4) * 4, y = e / (GW / 4) % WR, c = e / (GW / 4 * WR);
+            if (e < NG) *reinterpret_cast<float4*>(gs + c * GCH + y * GW + x) = vg[k];
+        }
+#pragma unroll
+        for (int k = 0; k < PI; ++k) {
+            constexpr int Q = GW * STRIDE / 4;
+            const int e = threadIdx.x + k * kWgT, x = e % Q * 4, y = e / Q % IR, c = e / (Q * IR);
+            if (e < NI) *reinterpret_cast<float4*>(is + c * ICH + y * IW + 4 + x) = vi[k];
+        }
+#pragma unroll
+        for (int k = 0; k < PE; ++k) {
+            const int e = threadIdx.x + k * kWgT, y = e / 2 % IR, c = e / (2 * IR);
+            if (e < NE && !(STRIDE == 2 && (e & 1))) is[c * ICH + y * IW + (e & 1 ? 4 + GW * STRIDE : 3)] = ve[k];
         }
         __syncthreads();
 #pragma unroll 1
         for (int y = 0; y < WR; ++y) {
-#pragma unroll 1
-            for (int x0 = 0; x0 < gw; x0 += 4) {
+            const float* gp = gs + to * GCH + y * GW;
+            const float* ip = is + tc * ICH + y * STRIDE * IW + 4;
+            float left[2][3];   // the value before the next group of columns
+#pragma unroll
+            for (int j = 0; j < 2; ++j)
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) left[j][ky] = ip[16 * j * ICH + ky * IW - 1];
+#pragma unroll 2
+            for (int x0 = 0; x0 < GW; x0 += 4) {
                 float g[2][4];
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                    const float4 t = *reinterpret_cast<const float4*>(gs + (to + 16 * i) * gch + y * gw + x0);
-                    g[i][0] = t.x; g[i][1] = t.y; g[i][2] = t.z; g[i][3] = t.w;
-                    sb[i] += (t.x + t.y) + (t.z + t.w);
+                    const float4 v = *reinterpret_cast<const float4*>(gp + 16 * i * GCH + x0);
+                    g[i][0] = v.x; g[i][1] = v.y; g[i][2] = v.z; g[i][3] = v.w;
+                    sb[i] += (v.x + v.y) + (v.z + v.w);
                 }
 #pragma unroll
                 for (int j = 0; j < 2; ++j)
 #pragma unroll
                     for (int ky = 0; ky < 3; ++ky) {
-                        const float* row = is + (tc + 16 * j) * ich + (y * STRIDE + ky) * iw + x0 * STRIDE;
-                        float v[3 * STRIDE + 3];
+                        const float* row = ip + 16 * j * ICH + ky * IW + x0 * STRIDE;
+                        float v[4 * STRIDE + 2];
+                        v[0] = left[j][ky];
 #pragma unroll
                         for (int q = 0; q < STRIDE; ++q) {
-                            const float4 t = *reinterpret_cast<const float4*>(row + 4 * q);
-                            v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
+                            const float4 w = *reinterpret_cast<const float4*>(row + 4 * q);
+                            v[4 * q + 1] = w.x; v[4 * q + 2] = w.y; v[4 * q + 3] = w.z; v[4 * q + 4] = w.w;
                         }
-                        if constexpr (STRIDE == 1) {
-                            const float2 t = *reinterpret_cast<const float2*>(row + 4);
-                            v[4] = t.x; v[5] = t.y;
-                        } else {
-                            v[8] = row[8];
-                        }
+                        left[j][ky] = v[4 * STRIDE];
+                        v[4 * STRIDE + 1] = STRIDE == 1 ? row[4] : 0.f;   // stride 2 ends inside the group
 #pragma unroll
                         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -423,16 +488,15 @@ __global__ void __launch_bounds__(kWgT, 2) k_conv_wgrad(const float* __restrict_
     }
 }
 
-// The same for the first layer (one input channel, stride 1): a warp per output channel (four of a
-// block's 32 in turn), its lanes over groups of four columns of a tile of 16 rows.  Bound by reading
-// gout once.
-constexpr int kW1Rows = 16;
+// The same for the first layer (one input channel, stride 1): two output channels per warp, 16 per block, its
+// lanes over groups of four columns of a tile of 16 rows.  Bound by reading gout once.
+constexpr int kW1Rows = 16, kW1C = 16;
 __global__ void __launch_bounds__(kWgT) k_conv_wgrad1(const float* __restrict__ gout, const float* __restrict__ in,
                                                       int B, int cout, int h, float* __restrict__ part) {
     extern __shared__ __align__(16) float is[];   // [kW1Rows + 2][iw], column ix + 1
-    const int gw = wg_gw(h), iw = gw + 4, q4 = gw / 4;
+    const int gw = h < kWgX ? (h + 3) / 4 * 4 : kWgX, iw = gw + 4, q4 = gw / 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int CW = kWgC / (kWgT / 32);   // output channels per warp
+    constexpr int CW = kW1C / (kWgT / 32);   // output channels per warp
     float acc[CW][10];
 #pragma unroll
     for (int c = 0; c < CW; ++c)
@@ -441,6 +505,7 @@ __global__ void __launch_bounds__(kWgT) k_conv_wgrad1(const float* __restrict__ 
     const int tiles_x = (h + gw - 1) / gw, tiles = (h + kW1Rows - 1) / kW1Rows * tiles_x;
     const long long units = (long long)B * tiles;
     const bool vec = h % 4 == 0;
+    const int cw = blockIdx.y * kW1C + warp * CW;
     for (long long u = blockIdx.x; u < units; u += gridDim.x) {
         const int b = (int)(u / tiles), t = (int)(u - (long long)b * tiles);
         const int y0 = t / tiles_x * kW1Rows, xs = t % tiles_x * gw;
@@ -452,43 +517,44 @@ __global__ void __launch_bounds__(kWgT) k_conv_wgrad1(const float* __restrict__ 
         }
         __syncthreads();
         const int rows = min(kW1Rows, h - y0);
+#pragma unroll 2
         for (int e = lane; e < rows * q4; e += 32) {
             const int y = e / q4, x0 = (e - y * q4) * 4;
             if (xs + x0 >= h) continue;
+            float g[CW][4];
+#pragma unroll
+            for (int c = 0; c < CW; ++c) {
+                const float* gp = gout + (((size_t)b * cout + min(cw + c, cout - 1)) * h + y0 + y) * h + xs + x0;
+                if (vec) {
+                    const float4 v = __ldg(reinterpret_cast<const float4*>(gp));
+                    g[c][0] = v.x; g[c][1] = v.y; g[c][2] = v.z; g[c][3] = v.w;
+                } else {
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) g[c][x] = xs + x0 + x < h ? __ldg(gp + x) : 0.f;
+                }
+            }
             float v[3][6];
 #pragma unroll
             for (int ky = 0; ky < 3; ++ky) {
                 const float* row = is + (y + ky) * iw + x0;
-                const float4 t = *reinterpret_cast<const float4*>(row);
-                const float2 t2 = *reinterpret_cast<const float2*>(row + 4);
-                v[ky][0] = t.x; v[ky][1] = t.y; v[ky][2] = t.z; v[ky][3] = t.w; v[ky][4] = t2.x; v[ky][5] = t2.y;
+                const float4 w = *reinterpret_cast<const float4*>(row);
+                const float2 w2 = *reinterpret_cast<const float2*>(row + 4);
+                v[ky][0] = w.x; v[ky][1] = w.y; v[ky][2] = w.z; v[ky][3] = w.w; v[ky][4] = w2.x; v[ky][5] = w2.y;
             }
 #pragma unroll
-            for (int c = 0; c < CW; ++c) {
-                const int co = blockIdx.y * kWgC + warp * CW + c;
-                if (co >= cout) break;
-                const float* gp = gout + (((size_t)b * cout + co) * h + y0 + y) * h + xs + x0;
-                float g[4];
-                if (vec) {
-                    const float4 t = __ldg(reinterpret_cast<const float4*>(gp));
-                    g[0] = t.x; g[1] = t.y; g[2] = t.z; g[3] = t.w;
-                } else {
-#pragma unroll
-                    for (int x = 0; x < 4; ++x) g[x] = xs + x0 + x < h ? __ldg(gp + x) : 0.f;
-                }
+            for (int c = 0; c < CW; ++c)
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) acc[c][k] = fmaf(g[x], v[k / 3][x + k % 3], acc[c][k]);
-                    acc[c][9] += g[x];
+                    for (int k = 0; k < 9; ++k) acc[c][k] = fmaf(g[c][x], v[k / 3][x + k % 3], acc[c][k]);
+                    acc[c][9] += g[c][x];
                 }
-            }
         }
     }
     float* o = part + (size_t)blockIdx.x * ((size_t)cout * 9 + cout);
 #pragma unroll
     for (int c = 0; c < CW; ++c) {
-        const int co = blockIdx.y * kWgC + warp * CW + c;
+        const int co = cw + c;
 #pragma unroll
         for (int k = 0; k < 10; ++k) {
             float s = acc[c][k];
@@ -521,18 +587,46 @@ __global__ void __launch_bounds__(kT) k_conv_wgrad_sum(const float* __restrict__
 // ------------------------------------------------------------------ dense layers (tiled GEMM)
 // C(m, n) = sum_k A(m, k) B(n, k), k ascending in one FP32 accumulator per output.  128 threads, a
 // TM x TN tile, MT x NT outputs per thread (rows in packed FP32 pairs), KT of k per step in two shared
-// buffers, the next step's operands held in registers meanwhile.  Bound by the FP32 pipe: the first
-// form (4 x 4 outputs per thread, one buffer, a thread's loads a row of A apart) spent its time on
-// shared-memory reads and uncoalesced loads.  The operands come from functors so that the two heads
-// form one product (their columns, rows or k ranges follow one another):
-//   op.a(m, k), op.b(n, k)  the operands (0 outside the product)     op.store(m, n, v)
-//   OP::AK / OP::BK         true: consecutive k are adjacent in memory (else consecutive m / n)
-constexpr int kGemmT = 128, KT = 16;
+// buffers, the next step's operands held in registers meanwhile.  Bound by the FP32 pipe; each thread's
+// share of an operand lies on a few rows whose addresses are formed once (per element they
+// took half as many instructions as the products) and whose values stay as loaded until they are stored
+// (converting float16 weights at the load waited for it): 163 -> 128 us for the logits of 256 samples, 353 -> 110
+// for their feature gradients.
+// The two heads form one product (their columns or rows follow one another).
+constexpr int kGemmT = 128, KT = 32;
+
+// One operand of a tile: ROWS rows (m or n), KT of k.  ADJ: consecutive k are adjacent in memory; a warp then
+// takes 8 k x 4 rows per load (full 32-byte sectors, conflict-free transposed stores), else a run of rows.
+template <int ROWS, bool ADJ, class T>
+struct Operand {
+    static constexpr int PER = ROWS * KT / kGemmT, NP = ADJ ? ROWS / 16 : 1;
+    const T* p[NP];
+    bool ok[NP];
+    long long ld;   // step of k when not ADJ
+    T v[PER];       // as loaded: converting here would wait for the load
+    static __device__ __forceinline__ int row(int i) {
+        return ADJ ? ((int)threadIdx.x >> 3) + 16 * (i % NP) : (int)threadIdx.x % ROWS;
+    }
+    static __device__ __forceinline__ int k(int i) {
+        return ADJ ? ((int)threadIdx.x & 7) + 8 * (i / NP) : (int)threadIdx.x / ROWS + i * (kGemmT / ROWS);
+    }
+    __device__ __forceinline__ void fetch(int k0, int ke) {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int kk = k0 + k(i);
+            v[i] = ok[i % NP] && kk < ke ? p[i % NP][ADJ ? (long long)kk : kk * ld] : T(0.f);
+        }
+    }
+    template <int LD>
+    __device__ __forceinline__ void stage(float (&S)[KT][LD]) const {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) S[k(i)][row(i)] = (float)v[i];
+    }
+};
 
 template <int TM, int TN, int MT, int NT, class OP>
 __global__ void __launch_bounds__(kGemmT) k_gemm(const OP op, int k_per_split, int K) {
     static_assert(TM / MT * (TN / NT) == kGemmT && MT % 4 == 0 && NT % 4 == 0, "one MT x NT block per thread");
-    constexpr int PA = TM * KT / kGemmT, PB = TN * KT / kGemmT;
     __shared__ __align__(16) float As[2][KT][TM + 4], Bs[2][KT][TN + 4];
     const int tn = threadIdx.x % (TN / NT), tm = threadIdx.x / (TN / NT);
     const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
@@ -542,54 +636,24 @@ __global__ void __launch_bounds__(kGemmT) k_gemm(const OP op, int k_per_split, i
     for (int i = 0; i < MT / 2; ++i)
 #pragma unroll
         for (int j = 0; j < NT; ++j) acc[i][j] = make_float2(0.f, 0.f);
-    float ra[PA], rb[PB];
-    // element i of a thread's share: k-adjacent operands take 8 k x 16 rows per pass (full 32-byte
-    // sectors, conflict-free transposed stores), the others a run of rows at one k
-    auto at = [](bool adj, int rows, int i, int& r, int& k) {
-        const int e = threadIdx.x + i * kGemmT;
-        if (adj) {
-            k = (e & 7) + ((e / (8 * rows)) << 3);
-            r = (e >> 3) % rows;
-        } else {
-            r = e % rows;
-            k = e / rows;
-        }
-    };
-    auto fetch = [&](int k0) {
+    Operand<TM, OP::AK, typename OP::TA> A;
+    Operand<TN, OP::BK, typename OP::TB> B;
 #pragma unroll
-        for (int i = 0; i < PA; ++i) {
-            int r, k;
-            at(OP::AK, TM, i, r, k);
-            ra[i] = k0 + k < ke ? op.a(m0 + r, k0 + k) : 0.f;
-        }
+    for (int i = 0; i < A.NP; ++i) A.ok[i] = op.a(m0 + A.row(i), A.p[i], A.ld);
 #pragma unroll
-        for (int i = 0; i < PB; ++i) {
-            int r, k;
-            at(OP::BK, TN, i, r, k);
-            rb[i] = k0 + k < ke ? op.b(n0 + r, k0 + k) : 0.f;
-        }
-    };
-    auto stage = [&](int buf) {
-#pragma unroll
-        for (int i = 0; i < PA; ++i) {
-            int r, k;
-            at(OP::AK, TM, i, r, k);
-            As[buf][k][r] = ra[i];
-        }
-#pragma unroll
-        for (int i = 0; i < PB; ++i) {
-            int r, k;
-            at(OP::BK, TN, i, r, k);
-            Bs[buf][k][r] = rb[i];
-        }
-    };
-    fetch(kb);
-    stage(0);
+    for (int i = 0; i < B.NP; ++i) B.ok[i] = op.b(n0 + B.row(i), B.p[i], B.ld);
+    A.fetch(kb, ke);
+    B.fetch(kb, ke);
+    A.stage(As[0]);
+    B.stage(Bs[0]);
     __syncthreads();
     int buf = 0;
     for (int k0 = kb; k0 < ke; k0 += KT, buf ^= 1) {
         const bool more = k0 + KT < ke;
-        if (more) fetch(k0 + KT);
+        if (more) {
+            A.fetch(k0 + KT, ke);
+            B.fetch(k0 + KT, ke);
+        }
 #pragma unroll
         for (int kk = 0; kk < KT; ++kk) {
             float2 a[MT / 2];
@@ -611,7 +675,10 @@ __global__ void __launch_bounds__(kGemmT) k_gemm(const OP op, int k_per_split, i
 #pragma unroll
                 for (int i = 0; i < MT / 2; ++i) acc[i][j] = __ffma2_rn(a[i], make_float2(bv[j], bv[j]), acc[i][j]);
         }
-        if (more) stage(buf ^ 1);
+        if (more) {
+            A.stage(As[buf ^ 1]);
+            B.stage(Bs[buf ^ 1]);
+        }
         __syncthreads();
     }
 #pragma unroll
@@ -622,17 +689,25 @@ __global__ void __launch_bounds__(kGemmT) k_gemm(const OP op, int k_per_split, i
                      (i & 1) ? acc[i / 2][j].y : acc[i / 2][j].x);
 }
 
+// The products.  op.a(m, p, ld) / op.b(n, p, ld): the row's address at k = 0 and (not ADJ) the step of k; false
+// outside the product.
+
 // Both heads' logits: m = sample, n = orientation bins then defocus bins, k = feature.
 struct HeadFwd {
     static constexpr bool AK = true, BK = true;
+    using TA = float;
+    using TB = __half;
     const float* feat;
     const __half *wq, *bq, *wd, *bd;
     float *lq, *ld;
     int B, nq, nd, F;
-    __device__ __forceinline__ float a(int m, int k) const { return m < B ? __ldg(feat + (size_t)m * F + k) : 0.f; }
-    __device__ __forceinline__ float b(int n, int k) const {
-        const __half* w = n < nq ? wq + (size_t)n * F : wd + (size_t)(n - nq) * F;
-        return n < nq + nd ? __half2float(w[k]) : 0.f;
+    __device__ __forceinline__ bool a(int m, const float*& p, long long&) const {
+        p = feat + (size_t)min(m, B - 1) * F;
+        return m < B;
+    }
+    __device__ __forceinline__ bool b(int n, const __half*& p, long long&) const {
+        p = n < nq ? wq + (size_t)n * F : wd + (size_t)min(n - nq, nd - 1) * F;
+        return n < nq + nd;
     }
     __device__ __forceinline__ void store(int m, int n, int, float v) const {
         if (m >= B || n >= nq + nd) return;
@@ -644,14 +719,21 @@ struct HeadFwd {
 // Both heads' weight gradients: m = bin, n = feature, k = sample.
 struct HeadGradW {
     static constexpr bool AK = false, BK = false;
+    using TA = float;
+    using TB = float;
     const float *glq, *gld, *feat;
     float *gwq, *gwd;
     int B, nq, nd, F;
-    __device__ __forceinline__ float a(int m, int k) const {
-        if (m >= nq + nd) return 0.f;
-        return m < nq ? __ldg(glq + (size_t)k * nq + m) : __ldg(gld + (size_t)k * nd + m - nq);
+    __device__ __forceinline__ bool a(int m, const float*& p, long long& ld) const {
+        p = m < nq ? glq + m : gld + min(m - nq, nd - 1);
+        ld = m < nq ? nq : nd;
+        return m < nq + nd;
     }
-    __device__ __forceinline__ float b(int n, int k) const { return n < F ? __ldg(feat + (size_t)k * F + n) : 0.f; }
+    __device__ __forceinline__ bool b(int n, const float*& p, long long& ld) const {
+        p = feat + min(n, F - 1);
+        ld = F;
+        return n < F;
+    }
     __device__ __forceinline__ void store(int m, int n, int, float v) const {
         if (m >= nq + nd || n >= F) return;
         if (m < nq) gwq[(size_t)m * F + n] = v;
@@ -659,33 +741,40 @@ struct HeadGradW {
     }
 };
 
-// Feature gradients, split over k: m = sample, n = feature, k = orientation bins then defocus bins;
+// Feature gradients from the orientation head, split over k: m = sample, n = feature, k = orientation bin;
 // part[split][m][n], summed by k_feat_grad.
 struct HeadGradX {
     static constexpr bool AK = true, BK = false;
-    const float *glq, *gld;
-    const __half *wq, *wd;
+    using TA = float;
+    using TB = __half;
+    const float* glq;
+    const __half* wq;
     float* part;
-    int B, nq, nd, F;
-    __device__ __forceinline__ float a(int m, int k) const {
-        if (m >= B) return 0.f;
-        return k < nq ? __ldg(glq + (size_t)m * nq + k) : __ldg(gld + (size_t)m * nd + k - nq);
+    int B, nq, F;
+    __device__ __forceinline__ bool a(int m, const float*& p, long long&) const {
+        p = glq + (size_t)min(m, B - 1) * nq;
+        return m < B;
     }
-    __device__ __forceinline__ float b(int n, int k) const {
-        const __half* w = k < nq ? wq + (size_t)k * F : wd + (size_t)(k - nq) * F;
-        return n < F ? __half2float(w[n]) : 0.f;
+    __device__ __forceinline__ bool b(int n, const __half*& p, long long& ld) const {
+        p = wq + min(n, F - 1);
+        ld = F;
+        return n < F;
     }
     __device__ __forceinline__ void store(int m, int n, int z, float v) const {
         if (m < B && n < F) part[((size_t)z * B + m) * F + n] = v;
     }
 };
 
-// gfeat = the sum of the k splits, back through the ReLU whose output is feat.
-__global__ void __launch_bounds__(kT) k_feat_grad(const float* __restrict__ part, int splits, size_t n,
+// gfeat = the sum of the k splits plus the defocus head's share, back through the ReLU whose output is feat.
+__global__ void __launch_bounds__(kT) k_feat_grad(const float* __restrict__ part, int splits, int B, int F,
+                                                  const float* __restrict__ gld, const __half* __restrict__ wd, int nd,
                                                   const float* __restrict__ feat, float* __restrict__ gfeat) {
+    const size_t n = (size_t)B * F;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const int b = (int)(i / F), f = (int)(i - (size_t)b * F);
         float s = 0.f;
         for (int z = 0; z < splits; ++z) s += part[(size_t)z * n + i];
+        for (int d = 0; d < nd; ++d) s = fmaf(gld[(size_t)b * nd + d], __half2float(wd[(size_t)d * F + f]), s);
         gfeat[i] = feat[i] > 0.f ? s : 0.f;
     }
 }
@@ -1104,10 +1193,10 @@ int prepare_input(bioem_cnn* n, const float* d_images, int B) {
     return check(n->ctx, "cnn input");
 }
 
-// Output channels per thread: 16 while that leaves at least four blocks per SM, else 8, else 4.
+// Output channels per thread: 16 while that leaves at least three blocks per SM, else 8, else 4.
 int conv_co(const bioem_ctx* ctx, long long n_tasks, int channels) {
     int co = 16;
-    while (co > 4 && (n_tasks + kConvT - 1) / kConvT * ((channels + co - 1) / co) < 4ll * ctx->num_sms) co /= 2;
+    while (co > 4 && (n_tasks + kConvT - 1) / kConvT * ((channels + co - 1) / co) < 3ll * ctx->num_sms) co /= 2;
     return co;
 }
 
@@ -1160,30 +1249,44 @@ void launch_conv_bwd_data(bioem_cnn* n, const Layer& Ly, const float* gout, cons
     n->ctx->n_launches++;
 }
 
-// Weight-gradient blocks: two per SM over all channel blocks, at most one per tile.
+// Weight-gradient blocks per channel block: two per SM over all of them, at most one per tile.
 int wgrad_blocks(const bioem_ctx* ctx, long long units, int channel_blocks) {
     const long long most = 2ll * ctx->num_sms / channel_blocks > 0 ? 2ll * ctx->num_sms / channel_blocks : 1;
     return (int)(units < most ? units : most);
 }
 
+template <int STRIDE, int GW>
+int conv_wgrad_launch(bioem_ctx* ctx, const Layer& Ly, const float* gout, const float* in, int B, int channel_blocks,
+                      float* part, int* blocks) {
+    using W = WgTile<STRIDE, GW>;
+    const long long tiles = (long long)((Ly.hout + W::WR - 1) / W::WR) * ((Ly.hout + GW - 1) / GW);
+    *blocks = wgrad_blocks(ctx, B * tiles, channel_blocks);
+    auto kern = Ly.hout % 4 == 0 ? k_conv_wgrad<STRIDE, GW, true> : k_conv_wgrad<STRIDE, GW, false>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W::SMEM) != cudaSuccess)
+        return bioem_check_cuda(ctx, cudaGetLastError(), "cnn shared memory");
+    kern<<<dim3(*blocks, channel_blocks), kWgT, W::SMEM, ctx->stream>>>(gout, in, B, Ly.cin, Ly.cout, Ly.hin, Ly.hout, part);
+    return BIOEM_OK;
+}
+
 int launch_conv_wgrad(bioem_cnn* n, const Layer& Ly, const float* gout, const float* in, int B, float* g) {
     bioem_ctx* ctx = n->ctx;
-    const int nco = (Ly.cout + kWgC - 1) / kWgC, nci = (Ly.cin + kWgC - 1) / kWgC;
-    const int gw = wg_gw(Ly.hout), tiles_x = (Ly.hout + gw - 1) / gw;
-    int blocks;
+    int blocks = 0, rc = BIOEM_OK;
     if (Ly.cin == 1 && Ly.stride == 1) {
-        blocks = wgrad_blocks(ctx, (long long)B * ((Ly.hout + kW1Rows - 1) / kW1Rows) * tiles_x, nco);
+        const int gw = Ly.hout < kWgX ? (Ly.hout + 3) / 4 * 4 : kWgX;
+        const long long tiles = (long long)((Ly.hout + kW1Rows - 1) / kW1Rows) * ((Ly.hout + gw - 1) / gw);
+        blocks = wgrad_blocks(ctx, B * tiles, 1);
         const size_t sm = sizeof(float) * (kW1Rows + 2) * (gw + 4);
-        k_conv_wgrad1<<<dim3(blocks, nco), kWgT, sm, ctx->stream>>>(gout, in, B, Ly.cout, Ly.hout, n->d_part);
+        k_conv_wgrad1<<<dim3(blocks, (Ly.cout + kW1C - 1) / kW1C), kWgT, sm, ctx->stream>>>(gout, in, B, Ly.cout, Ly.hout,
+                                                                                        n->d_part);
     } else {
-        const int wr = wg_rows(Ly.stride);
-        blocks = wgrad_blocks(ctx, (long long)B * ((Ly.hout + wr - 1) / wr) * tiles_x, nco * nci);
-        const size_t sm = sizeof(float) * kWgC * (size_t)(wg_gch(Ly.hout, Ly.stride) + wg_ich(Ly.hout, Ly.stride));
-        auto kern = Ly.stride == 1 ? k_conv_wgrad<1> : k_conv_wgrad<2>;
-        if (sm > 48 * 1024 &&
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
-            return bioem_check_cuda(ctx, cudaGetLastError(), "cnn shared memory");
-        kern<<<dim3(blocks, nco * nci), kWgT, sm, ctx->stream>>>(gout, in, B, Ly.cin, Ly.cout, Ly.hin, Ly.hout, n->d_part);
+        const int cb = ((Ly.cout + kWgC - 1) / kWgC) * ((Ly.cin + kWgC - 1) / kWgC);
+        // the narrowest tile that holds an output row, at most kWgX columns
+#define WG(S, W) conv_wgrad_launch<S, W>(ctx, Ly, gout, in, B, cb, n->d_part, &blocks)
+#define WG_S(S) (Ly.hout <= 8 ? WG(S, 8) : Ly.hout <= 16 ? WG(S, 16) : Ly.hout <= 32 ? WG(S, 32) : WG(S, kWgX))
+        rc = Ly.stride == 1 ? WG_S(1) : WG_S(2);
+#undef WG_S
+#undef WG
+        if (rc) return rc;
     }
     const int n_w = Ly.cout * Ly.cin * 9, total = n_w + Ly.cout;
     k_conv_wgrad_sum<<<(total + 31) / 32, kT, 0, ctx->stream>>>(n->d_part, blocks, n_w, total, g + Ly.w_off,
@@ -1223,19 +1326,22 @@ int backward(bioem_cnn* n, const int* d_yq, const int* d_yd, int B, float* g) {
     const int F = (int)n->F;
     // head weights gW[o][f] = sum_b glogit[b][o] feat[b][f]; biases: column sums
     const HeadGradW gw{n->d_lq, n->d_ld, feat, g + h.wq, g + h.wd, B, n->n_q, n->n_d, F};
-    k_gemm<128, 64, 8, 8><<<dim3((F + 63) / 64, (n->n_q + n->n_d + 127) / 128), kGemmT, 0, st>>>(gw, B, B);
+    k_gemm<64, 64, 8, 4><<<dim3((F + 63) / 64, (n->n_q + n->n_d + 63) / 64), kGemmT, 0, st>>>(gw, B, B);
     k_colsum<<<(n->n_q + 31) / 32 + (n->n_d + 31) / 32, kT, 0, st>>>(n->d_lq, n->n_q, n->d_ld, n->n_d, B, g + h.bq,
                                                                    g + h.bd);
-    // feature gradient gfeat[b][f] = sum_o glq[b][o] Wq[o][f] + sum_o gld[b][o] Wd[o][f]: a short product
-    // (few tiles, long k), so k is split; the parts lie where the first layer's output gradient is
+    // feature gradient gfeat[b][f] = sum_o glq[b][o] Wq[o][f] + sum_o gld[b][o] Wd[o][f]: few tiles and a long k,
+    // so k is split into about six tiles per SM; the parts lie where the first layer's output gradient is
     // written later (C S^2 B floats, at least kFeatSplits F B)
     float* gfeat = n->d_gact + last.out_off * B;
-    const HeadGradX gx{n->d_lq, n->d_ld, n->d_p16 + h.wq, n->d_p16 + h.wd, n->d_gact + n->layers[0].out_off * B,
-                       B, n->n_q, n->n_d, F};
-    const int K = n->n_q + n->n_d, kps = ((K + kFeatSplits - 1) / kFeatSplits + KT - 1) / KT * KT;
-    const int splits = (K + kps - 1) / kps;
-    k_gemm<64, 64, 8, 4><<<dim3((F + 63) / 64, (B + 63) / 64, splits), kGemmT, 0, st>>>(gx, kps, K);
-    k_feat_grad<<<grid_for((size_t)B * F), kT, 0, st>>>(gx.part, splits, (size_t)B * F, feat, gfeat);
+    const HeadGradX gx{n->d_lq, n->d_p16 + h.wq, n->d_gact + n->layers[0].out_off * B, B, n->n_q, F};
+    const dim3 tiles((F + 63) / 64, (B + 63) / 64);
+    long long splits = 6ll * ctx->num_sms / ((long long)tiles.x * tiles.y);
+    splits = splits < 1 ? 1 : splits > kFeatSplits ? kFeatSplits : splits;
+    const int kps = (int)(((n->n_q + splits - 1) / splits + KT - 1) / KT * KT);
+    splits = (n->n_q + kps - 1) / kps;
+    k_gemm<64, 64, 8, 4><<<dim3(tiles.x, tiles.y, (unsigned)splits), kGemmT, 0, st>>>(gx, kps, n->n_q);
+    k_feat_grad<<<grid_for((size_t)B * F), kT, 0, st>>>(gx.part, (int)splits, B, F, n->d_ld, n->d_p16 + h.wd, n->n_d, feat,
+                                                        gfeat);
     ctx->n_launches += 5;
     // conv layers, last to first
     for (int l = kLayers - 1; l >= 0; --l) {
