@@ -356,15 +356,16 @@ constexpr float kErfcZero = 11.f, kWindow = 10.5f;
 // tile and chunk) and accumulates w_a gy gx as packed FP32 pairs.  Every pixel sums its atoms in index
 // order; left out are exact zeros only.  A chunk's positions are formed (float64, one warp, lane = atom) two
 // chunks ahead of its sums and its tables one chunk ahead: one barrier per chunk.
-// Bound by issue: ~150 warp instructions per atom for the tables, ~170 for the sums.  The first form
-// tabulated every boundary of the image for every atom and summed whole rows: 7.0 us per orientation (128
-// px, 5000 atoms, sigma 1.5 A).
+// Bound by issue (0.6 per cycle and scheduler) and the latency of erfc: ~220 warp instructions per atom for
+// the tables, ~170 for the sums.  128 px, 5000 atoms, sigma 1.5 A, us per orientation: 7.1 when every boundary
+// of the image was tabulated for every atom and whole rows were summed, 3.4 with 8 warps of 4 tiles, 3.1
+// with 16 warps of 2.
 template <int N>
 struct ProjCfg {
     static constexpr int LR = N == 32 ? 2 : 4, LC = LR;
     static constexpr int TR = 4 * LR, TC = 8 * LC;                 // tile
     static constexpr int TCOLS = N / TC, TROWS = N / TR;
-    static constexpr int NW = N == 96 ? 9 : N == 192 ? 18 : 8;     // warps
+    static constexpr int NW = N == 96 ? 18 : N == 128 ? 16 : N == 192 ? 24 : 8;   // warps
     static constexpr int BAND = NW / TCOLS, TPW = TROWS / BAND;    // tile rows per band, tiles per warp
     static_assert(TCOLS * TC == N && TROWS * TR == N && BAND * TCOLS == NW && TPW * BAND == TROWS, "tiles cover the image");
     static constexpr int T = 32 * NW;
@@ -385,7 +386,7 @@ __device__ __forceinline__ void load_vec(const float* src, float (&v)[V]) {
 }
 
 template <int N>
-__global__ void __launch_bounds__(ProjCfg<N>::T) k_project(const float4* __restrict__ atoms, int n_atoms,
+__global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1) k_project(const float4* __restrict__ atoms, int n_atoms,
                                                            const float4* __restrict__ quats, double sigma,
                                                            double pixel, float* __restrict__ out) {
     using C = ProjCfg<N>;
