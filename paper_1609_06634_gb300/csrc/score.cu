@@ -637,15 +637,22 @@ __device__ __forceinline__ void score_item(const Sm<C>& sm, const float2* __rest
     }
 }
 
+// Parameter sets of the short chunks that end a launch: a quarter of the others, whole group batches.
+template <class C>
+__host__ __device__ constexpr int short_chunk(int chunk) {
+    return (chunk / 4 + C::GPB - 1) / C::GPB * C::GPB;
+}
+
 // Work items (chunk ci, image w), item = ci n_img + w, are taken in index order from a global counter
 // (zero at launch): the items in flight stay within one or two chunks of parameter sets, so a chunk
 // is read from DRAM about once (a fixed item-per-block assignment let the blocks drift apart over
 // thousands of items until several chunks competed for the L2; visiting two chunks per image before
-// the next image, to reuse each image, made the two chunks compete the same way).
+// the next image, to reuse each image, made the two chunks compete the same way).  The first n_long chunks
+// hold `chunk` sets, the rest a quarter of that, so that the blocks end closer together.
 template <class C>
 __global__ void __launch_bounds__(C::THREADS, 1)
 k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int n_img,
-        const float2* __restrict__ ps_spec, int ps_begin, int ps_count, int chunk, int n_items, int s, float c1,
+        const float2* __restrict__ ps_spec, int ps_begin, int ps_count, int chunk, int n_long, int n_items, int s, float c1,
         float* __restrict__ rec_t, float* __restrict__ rec_s, int* __restrict__ rec_d, int* __restrict__ status,
         int* __restrict__ work) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -659,8 +666,9 @@ k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int
         if (item >= n_items) break;
         const int ci = item / n_img;
         const int w = item - ci * n_img;
-        const int lo = ci * chunk;
-        const int hi = min(lo + chunk, ps_count);
+        const int tail = short_chunk<C>(chunk);
+        const int lo = ci < n_long ? ci * chunk : n_long * chunk + (ci - n_long) * tail;
+        const int hi = min(lo + (ci < n_long ? chunk : tail), ps_count);
         const size_t row = (size_t)w * ps_count;
         score_item<C>(sm, gtw, img_spec + (size_t)w * C::N * C::H, nullptr, ps_spec, ps_begin, lo, hi, s, c1, rec_t + row,
                       rec_s + row, rec_d + row, status);
@@ -1107,7 +1115,16 @@ int launch_score_records(bioem_ctx* ctx, const bioem_images* im, const bioem_pro
                          int wl, int max_shift, float* rec_t, float* rec_s, int* rec_d) {
     const int n_img = im->n_img;
     const long long chunk = score_chunk<C>(n_img, wl, slots);
-    const long long n_chunks = (wl + chunk - 1) / chunk;
+    // with more items than slots, about the last item of each slot goes out in short chunks: ns per pair
+    // without -> with: 128 px, s = 4: 7.74 -> 7.37; 96 px 7.66 -> 7.43; 64 px, s = 4: 2.25 -> 2.19 (two or three
+    // items' worth gained no more)
+    long long n_chunks = (wl + chunk - 1) / chunk, n_long = n_chunks;
+    if (n_chunks * n_img > slots && chunk >= 4 * C::GPB) {
+        n_long = wl / chunk - ((long long)slots + n_img - 1) / n_img;
+        if (n_long < 0) n_long = 0;
+        const int tail = short_chunk<C>((int)chunk);
+        n_chunks = n_long + (wl - n_long * chunk + tail - 1) / tail;
+    }
     const long long n_items = n_chunks * n_img;
     if (n_items > 0x7fffffffll) return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "too many work items");
     const int grid = (int)(n_items < slots ? n_items : slots);
@@ -1116,7 +1133,7 @@ int launch_score_records(bioem_ctx* ctx, const bioem_images* im, const bioem_pro
     if (cudaMemsetAsync(ctx->d_work, 0, sizeof(int), ctx->stream) != cudaSuccess)
         return bioem_check_cuda(ctx, cudaGetLastError(), "work counter");
     k_score<C><<<grid, C::THREADS, C::SMEM, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, ps->d_spec,
-                                                            wbegin, wl, (int)chunk, (int)n_items, max_shift, c1f,
+                                                            wbegin, wl, (int)chunk, (int)n_long, (int)n_items, max_shift, c1f,
                                                             rec_t, rec_s, rec_d, ctx->d_status, ctx->d_work);
     bioem_launch_end(ctx, KID_SCORE);
     return bioem_check_cuda(ctx, cudaGetLastError(), "k_score");
@@ -1156,8 +1173,8 @@ int run_score_gemm(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* 
 // stage-B row]>.  Groups as many as registers allow without spills and shared memory holds; a group's batch
 // fills whole rounds of its threads with column tasks (PB N/2 with the packed edge columns, PB (N/2 + 1)
 // without) and at most one round with rows.  ns per pair (k_score, one GB300; one block-wide group of
-// 245-272 threads moving through the phases in step before -> now): 32 px 1.76 -> 0.77; 64 px, s = 4: 3.68 ->
-// 2.14, s = 8: 5.22 -> 3.00; 96 px 10.5 -> 7.5; 128 px, s = 4: 14.7 -> 7.7.  More groups at fewer registers lost
+// 245-272 threads moving through the phases in step before -> now): 32 px 1.76 -> 0.85; 64 px, s = 4: 3.68 ->
+// 2.19, s = 8: 5.22 -> 3.1; 96 px 10.5 -> 7.4; 128 px, s = 4: 14.7 -> 7.4.  More groups at fewer registers lost
 // (128 px, s = 4: 6 x 128 threads of 79 registers 9.9; 8 x 64 threads 10.4), as did fewer, larger ones
 // (3 x 192 threads 7.9, 3 x 256 10.0).  192 px holds two pairs beside the image: one group in step, 54
 // (as two groups of one pair 64: the 97th column then takes a warp per group; the image read through L1 and
