@@ -527,7 +527,8 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
 }
 
 // T[c][ky][kx] = CTF(s) Env(s) for PSF c on the half-spectrum grid, evaluated in float64.
-// coef[3c..3c+2] = (a, A, b); s = 2 pi (kx~, ky~) / (N pixel) with signed frequency indices.  The value depends on kx~^2 + ky~^2 only, so each unordered pair {|kx~|, |ky~|} is
+// coef[4c..4c+3] = (a, A, b, sqrt(1 - A^2)); s = 2 pi (kx~, ky~) / (N pixel) with signed frequency
+// indices.  The value depends on kx~^2 + ky~^2 only, so each unordered pair {|kx~|, |ky~|} is
 // evaluated once and written to its (up to four) places: bound by float64 arithmetic, a quarter of
 // evaluating every coefficient (1.20 ms for 1024 PSFs at 128 px before).
 __global__ void k_ctf_table(const double* __restrict__ coef, int nctf, int N, double pixel,
@@ -544,8 +545,10 @@ __global__ void k_ctf_table(const double* __restrict__ coef, int nctf, int N, do
         while (hi * (hi + 1) / 2 > r) --hi;
         const int lo = r - hi * (hi + 1) / 2;
         const double s2 = f * f * ((double)lo * lo + (double)hi * hi);
-        const double a = coef[3 * c], A = coef[3 * c + 1], b = coef[3 * c + 2];
-        const double ctf = -A * cos(0.5 * a * s2) - sqrt(1.0 - A * A) * sin(0.5 * a * s2);
+        const double a = coef[4 * c], A = coef[4 * c + 1], b = coef[4 * c + 2];
+        double sn, cs;
+        sincos(0.5 * a * s2, &sn, &cs);
+        const double ctf = -A * cs - coef[4 * c + 3] * sn;
         const float v = (float)(ctf * exp(-0.5 * b * s2));
         auto put = [&](int ky, int kx) { T[(size_t)c * N * H + (size_t)ky * H + kx] = v; };
         put(lo, hi);
@@ -740,21 +743,22 @@ int set_smem(const void* fn, size_t bytes) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess ? 0 : -1;
 }
 
-void ctf_coefficients(const bioem_ctf& c, double* out3) {
+void ctf_coefficients(const bioem_ctf& c, double* out4) {
     const double v = c.voltage_kV * 1.0e3;
     const double lam = 12.2643 / sqrt(v * (1.0 + 0.97845e-6 * v));
-    out3[0] = lam * c.defocus_A / (2.0 * 3.14159265358979323846);
-    out3[1] = c.amp_contrast;
-    out3[2] = c.bfactor_A2 / (8.0 * 3.14159265358979323846 * 3.14159265358979323846);
+    out4[0] = lam * c.defocus_A / (2.0 * 3.14159265358979323846);
+    out4[1] = c.amp_contrast;
+    out4[2] = c.bfactor_A2 / (8.0 * 3.14159265358979323846 * 3.14159265358979323846);
+    out4[3] = sqrt(1.0 - c.amp_contrast * c.amp_contrast);
 }
 
 // Build the CTF table for nctf PSFs into *d_T (allocated here; caller frees).
 int build_ctf_table(bioem_ctx* ctx, const bioem_ctf* ctfs, int nctf, int npix, double pixel_A, float** d_T) {
-    double* h = (double*)malloc(sizeof(double) * 3 * nctf);
+    double* h = (double*)malloc(sizeof(double) * 4 * nctf);
     if (!h) return bioem_set_error(ctx, BIOEM_ERR_OOM, "host allocation failed");
-    for (int c = 0; c < nctf; ++c) ctf_coefficients(ctfs[c], h + 3 * c);
+    for (int c = 0; c < nctf; ++c) ctf_coefficients(ctfs[c], h + 4 * c);
     double* d_coef = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&d_coef, sizeof(double) * 3 * nctf, ctx->stream);
+    cudaError_t e = cudaMallocAsync((void**)&d_coef, sizeof(double) * 4 * nctf, ctx->stream);
     if (e != cudaSuccess) { free(h); return bioem_set_error(ctx, BIOEM_ERR_OOM, "cudaMallocAsync(ctf coef)"); }
     const size_t tsize = (size_t)nctf * npix * (npix / 2 + 1);
     e = cudaMallocAsync((void**)d_T, sizeof(float) * tsize, ctx->stream);
@@ -763,7 +767,7 @@ int build_ctf_table(bioem_ctx* ctx, const bioem_ctf* ctfs, int nctf, int npix, d
         free(h);
         return bioem_set_error(ctx, BIOEM_ERR_OOM, "cudaMallocAsync(ctf table)");
     }
-    e = cudaMemcpyAsync(d_coef, h, sizeof(double) * 3 * nctf, cudaMemcpyHostToDevice, ctx->stream);
+    e = cudaMemcpyAsync(d_coef, h, sizeof(double) * 4 * nctf, cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) {
         const size_t work = (tsize / 4 + 255) / 256 + 1;
         const int blocks = (int)(work < 4096 ? work : 4096);
