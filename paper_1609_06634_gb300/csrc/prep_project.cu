@@ -356,10 +356,10 @@ constexpr float kErfcZero = 11.f, kWindow = 10.5f;
 // tile and chunk) and accumulates w_a gy gx as packed FP32 pairs.  Every pixel sums its atoms in index
 // order; left out are exact zeros only.  A chunk's positions are formed (float64, one warp, lane = atom) two
 // chunks ahead of its sums and its tables one chunk ahead: one barrier per chunk.
-// Bound by issue (0.6 per cycle and scheduler) and the latency of erfc: ~220 warp instructions per atom for
-// the tables, ~170 for the sums.  128 px, 5000 atoms, sigma 1.5 A, us per orientation: 7.1 when every boundary
+// Bound by issue (0.7 per cycle and scheduler) and the latency of erfc: ~540 warp instructions per atom at 128 px
+// (1.1 A), most of them for the tables' three passes and for 6.7 tiles' sums.  128 px, 5000 atoms, sigma 1.5 A, us per orientation: 7.1 when every boundary
 // of the image was tabulated for every atom and whole rows were summed, 3.4 with 8 warps of 4 tiles, 3.1
-// with 16 warps of 2.
+// with 16 warps of 2, 2.9 with atoms taken by the warps that are free.
 template <int N>
 struct ProjCfg {
     static constexpr int LR = N == 32 ? 2 : 4, LC = LR;
@@ -369,6 +369,10 @@ struct ProjCfg {
     static constexpr int BAND = NW / TCOLS, TPW = TROWS / BAND;    // tile rows per band, tiles per warp
     static_assert(TCOLS * TC == N && TROWS * TR == N && BAND * TCOLS == NW && TPW * BAND == TROWS, "tiles cover the image");
     static constexpr int T = 32 * NW;
+    // Warps take the atoms they tabulate one by one, after their sums, so that those with sparse tiles tabulate
+    // more: 1024 maps at 128 px 4.79 -> 4.56 ms, 500 at 192 px 7.66 -> 5.18 ms.  At 96 px (two passes per
+    // atom) and below equal shares are as good or better: 2.35 against 2.48 ms for 1000 maps at 64 px.
+    static constexpr bool TAKE = N >= 128;
     static constexpr int CH = 32;                                  // atoms per chunk: one per lane of a ballot
     static constexpr size_t SM_TAB = (size_t)CH * 2 * N * sizeof(float);   // gx, gy rows of a chunk
     static constexpr size_t SMEM = 2 * SM_TAB;
@@ -399,6 +403,7 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
     struct Axis { float h, l; int lo, hi; };
     __shared__ Axis pos[3][CH][2];
     __shared__ float wgt[3][CH];
+    __shared__ int taken[2];   // atoms of table 0 / 1's chunk that warps have taken
 
     const int q = blockIdx.x;
     if (threadIdx.x == 0) {
@@ -440,9 +445,14 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
         pos[buf][lane][1] = ay;
         wgt[buf][lane] = w;
     };
-    auto tables = [&](int pb, int buf) {   // every warp: its atoms of the chunk in pos[pb], into table buf
+    auto tables = [&](int pb, int buf) {   // every warp: its share of the chunk in pos[pb], into table buf
         const int axis = lane >> 4, l = lane & 15;
-        for (int a = warp; a < CH; a += NW) {
+        auto take = [&]() {
+            int a = 0;
+            if (lane == 0) a = atomicAdd(&taken[buf], 1);
+            return __shfl_sync(0xffffffffu, a, 0);
+        };
+        for (int a = C::TAKE ? take() : warp; a < CH; a = C::TAKE ? take() : a + NW) {
             const Axis v = pos[pb][a][axis];
             const Axis o = pos[pb][a][axis ^ 1];
             if (v.hi < v.lo || o.hi < o.lo) continue;   // off the image on an axis (the same in both half warps)
@@ -475,6 +485,7 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
             for (int j = 0; j < LC; ++j) acc[t][i][j] = make_float2(0.f, 0.f);
     const int lr = (lane >> 3) * LR, lc = (lane & 7) * LC;
 
+    if (threadIdx.x < 2) taken[threadIdx.x] = 0;
     if (warp == 0) positions(0, 0);
     if (warp == NW - 1) positions(CH, 1);
     __syncthreads();
@@ -486,7 +497,7 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
         const Axis px = pos[pb][lane][0], py = pos[pb][lane][1];
         const bool some = px.lo <= px.hi && py.lo <= py.hi;
         if (warp == c % NW && a0 + 2 * CH < n_atoms) positions(a0 + 2 * CH, p2);
-        if (a0 + CH < n_atoms) tables(p1, buf ^ 1);
+        if (!C::TAKE && a0 + CH < n_atoms) tables(p1, buf ^ 1);
         const float* base = tab + (size_t)buf * CH * 2 * N;
 #pragma unroll
         for (int t = 0; t < C::TPW; ++t) {
@@ -507,6 +518,8 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
                         acc[t][i][j] = __ffma2_rn(make_float2(vy[2 * i], vy[2 * i + 1]), make_float2(vx[j], vx[j]), acc[t][i][j]);
             }
         }
+        if (C::TAKE && a0 + CH < n_atoms) tables(p1, buf ^ 1);
+        if (threadIdx.x == 0) taken[buf] = 0;   // next taken from after the barrier
         pb = p1;
         __syncthreads();
     }
@@ -673,31 +686,250 @@ __global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(con
     }
 }
 
-// Synthetic map for pair i: I1 = Re F^-1[F(I0_i) T_i] with F^-1 normalised by 1/N^2.
+// ---- transforms by factors, for the maps
+// cos(2 pi j / n), by the Taylor series of cos or sin about 0 after reduction to an eighth of a turn.
+constexpr double cos_turn(int j, int n) {
+    double x = (double)(((j % n) + n) % n) / n;
+    if (x > 0.5) x = 1.0 - x;
+    double sign = 1.0;
+    if (x > 0.25) {
+        x = 0.5 - x;
+        sign = -1.0;
+    }
+    const bool use_sin = x > 0.125;
+    const double t = 2.0 * 3.14159265358979323846 * (use_sin ? 0.25 - x : x);
+    double term = use_sin ? t : 1.0, sum = 0.0;
+    for (int k = use_sin ? 2 : 1; k < 30; k += 2) {
+        sum += term;
+        term *= -t * t / (k * (k + 1));
+    }
+    return sign * sum;
+}
+// w.x, w.y[j] = cos, sin of 2 pi j / R
+template <int R>
+struct Roots {
+    float c[R] = {}, s[R] = {};
+    constexpr Roots() {
+        for (int j = 0; j < R; ++j) {
+            c[j] = (float)cos_turn(j, R);
+            s[j] = (float)cos_turn(4 * j - R, 4 * R);
+        }
+    }
+};
+// v exp(-+ 2 pi i j / R) (upper sign forward), 0 <= j < R known at compile time
+template <int R, bool INV>
+__device__ __forceinline__ float2 turn(float2 v, int j) {
+    constexpr Roots<R> w{};
+    if (j == 0) return v;
+    if (4 * j == R) return INV ? make_float2(-v.y, v.x) : make_float2(v.y, -v.x);
+    if (2 * j == R) return make_float2(-v.x, -v.y);
+    return INV ? c_mul(v, make_float2(w.c[j], w.s[j])) : c_mul(v, make_float2(w.c[j], -w.s[j]));
+}
+// In-register transform of R = 2^a or 3 2^a values, natural order in and out.
+template <int R, bool INV>
+__device__ __forceinline__ void dft(float2 (&x)[R]) {
+    if constexpr (R == 2) {
+        const float2 a = x[0];
+        x[0] = c_add(a, x[1]);
+        x[1] = c_sub(a, x[1]);
+    } else if constexpr (R == 3) {
+        const float2 t = c_add(x[1], x[2]), d = c_sub(x[1], x[2]);
+        const float2 m = make_float2(fmaf(-0.5f, t.x, x[0].x), fmaf(-0.5f, t.y, x[0].y));
+        constexpr float s = INV ? 0.8660254037844386f : -0.8660254037844386f;
+        x[0] = c_add(x[0], t);
+        x[1] = make_float2(fmaf(-s, d.y, m.x), fmaf(s, d.x, m.y));
+        x[2] = make_float2(fmaf(s, d.y, m.x), fmaf(-s, d.x, m.y));
+    } else if constexpr (R == 4) {
+        const float2 a = c_add(x[0], x[2]), b = c_sub(x[0], x[2]), c = c_add(x[1], x[3]);
+        const float2 d = turn<4, INV>(c_sub(x[1], x[3]), 1);
+        x[0] = c_add(a, c);
+        x[1] = c_add(b, d);
+        x[2] = c_sub(a, c);
+        x[3] = c_sub(b, d);
+    } else {
+        constexpr int P = R % 4 == 0 ? 4 : 2, Q = R / P;
+        float2 y[Q][P];
+#pragma unroll
+        for (int b = 0; b < Q; ++b) {
+#pragma unroll
+            for (int a = 0; a < P; ++a) y[b][a] = x[Q * a + b];
+            dft<P, INV>(y[b]);
+#pragma unroll
+            for (int k = 0; k < P; ++k) y[b][k] = turn<R, INV>(y[b][k], b * k);
+        }
+#pragma unroll
+        for (int k = 0; k < P; ++k) {
+            float2 t[Q];
+#pragma unroll
+            for (int b = 0; b < Q; ++b) t[b] = y[b][k];
+            dft<Q, INV>(t);
+#pragma unroll
+            for (int k2 = 0; k2 < Q; ++k2) x[k + P * k2] = t[k2];
+        }
+    }
+}
+
+// N = 16 R: with n = R a + b and k = k1 + 16 k2, a length-N transform is R transforms of 16 values (over a),
+// a turn by b k1 / N and 16 transforms of R values (over b).
 template <int N>
-__global__ void __launch_bounds__(Dft<N>::T) k_psf_real(const float* __restrict__ img0,
-                                                        const float2* __restrict__ g_tw,
-                                                        const float* __restrict__ T,
-                                                        float* __restrict__ out) {
-    constexpr int H = Dft<N>::H, TH = Dft<N>::T;
+struct Fft {
+    static constexpr int R = N / 16, H = N / 2 + 1;
+    static constexpr int T = N == 32 ? 64 : N == 64 ? 128 : N == 192 ? 512 : 256;
+    static constexpr int MINB = N <= 64 ? 8 : N == 192 ? 1 : 3;
+    // Rows 2p and 2p + 1 of the spectrum hold the packed transform of a pair of image rows meanwhile, R runs
+    // of 16 with one place between them; with this pitch neither the runs nor the pairs conflict.
+    static constexpr int P = 17 * R / 2;
+    static_assert(R % 2 == 0 && P >= H, "a packed transform fits two rows");
+    static constexpr size_t SMEM = (size_t)(N * P + N) * sizeof(float2);
+};
+
+// Synthetic map for pair i: I1 = Re F^-1[F(I0_i) T_i] with F^-1 normalised by 1/N^2.  A block per map, every pass in
+// place in shared memory: rows two by two as one complex transform (a warp takes four pairs and needs no
+// block barrier), columns with the PSF and the first half of the inverse applied while a column's R
+// frequencies are in registers.  Bound by shared memory and the latency of its passes.  1024 maps at 128 px: 2174 us by
+// dense sums over shared memory, 721 us by dense sums in register tiles (N multiply-adds per
+// coefficient and pass), 65 us so.  The spectra that are scored keep the dense sums (k_psf_spectra): another
+// rounding moves their FP32 scale.
+template <int N>
+__global__ void __launch_bounds__(Fft<N>::T, Fft<N>::MINB) k_psf_real(const float* __restrict__ img0,
+                                                                   const float2* __restrict__ g_tw,
+                                                                   const float* __restrict__ T,
+                                                                   float* __restrict__ out) {
+    using C = Fft<N>;
+    constexpr int R = C::R, H = C::H, P = C::P, TH = C::T, NW = TH / 32;
     extern __shared__ __align__(16) unsigned char smem[];
-    const DftSm<N> sm(smem);
-    const int i = blockIdx.x;
-    sm.twiddles(g_tw, false);
+    float2* const F = reinterpret_cast<float2*>(smem);
+    float2* const tw = F + N * P;   // exp(-2 pi i t / N)
+    const size_t map = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < N; i += TH) tw[i] = g_tw[i];
     __syncthreads();
-    r2c_rows<N>(img0 + (size_t)i * N * N, 0.f, sm);
+    // rows: C = row 2p + i row 2p + 1 transformed, then taken apart into the halves 2 F (the factor
+    // is taken back at the end)
+    const float* img = img0 + map * N * N;
+    const int j = lane & 7, kA = j, kB = j ? 16 - j : 8;   // a lane's two residues k1, partners under k -> N - k
+    for (int g = warp; g < N / 8; g += NW) {
+        for (int t = lane; t < 4 * R; t += 32) {
+            const int p = 4 * g + t / R, b = t % R;
+            const float* row = img + (size_t)2 * p * N + b;
+            float2 x[16];
+#pragma unroll
+            for (int a = 0; a < 16; ++a) x[a] = make_float2(__ldg(row + R * a), __ldg(row + N + R * a));
+            dft<16, false>(x);
+            float2* buf = F + (size_t)2 * p * P + 17 * b;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) buf[k] = k ? c_mul(x[k], tw[b * k]) : x[k];
+        }
+        __syncwarp();
+        float2* const buf = F + (size_t)2 * (4 * g + (lane >> 3)) * P;
+        float2 u[R], v[R];
+#pragma unroll
+        for (int b = 0; b < R; ++b) {
+            u[b] = buf[17 * b + kA];
+            v[b] = buf[17 * b + kB];
+        }
+        dft<R, false>(u);
+        dft<R, false>(v);
+        __syncwarp();
+        auto apart = [&](int k, float2 c, float2 d) {   // d = C(N - k)
+            buf[k] = make_float2(c.x + d.x, c.y - d.y);
+            buf[P + k] = make_float2(c.y + d.y, d.x - c.x);
+        };
+#pragma unroll
+        for (int k2 = 0; k2 < R / 2; ++k2) {
+            apart(kA + 16 * k2, u[k2], j ? v[R - 1 - k2] : u[(R - k2) % R]);
+            apart(kB + 16 * k2, v[k2], j ? u[R - 1 - k2] : v[R - 1 - k2]);
+        }
+        if (j == 0) apart(N / 2, u[R / 2], u[R / 2]);
+    }
     __syncthreads();
-    c2c_columns_inplace<N>(sm);
-    const float* Ti = T + (size_t)i * N * H;
-    for (int o = threadIdx.x; o < N * H; o += TH) sm.F[o] = c_scale(sm.F[o], __ldg(Ti + o));
-    sm.twiddles(g_tw, true);
+    // columns
+    for (int e = threadIdx.x; e < H * R; e += TH) {
+        const int kx = e % H, b = e / H;
+        float2* col = F + b * P + kx;
+        float2 x[16];
+#pragma unroll
+        for (int a = 0; a < 16; ++a) x[a] = col[R * a * P];
+        dft<16, false>(x);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) col[R * k * P] = k ? c_mul(x[k], tw[b * k]) : x[k];
+    }
     __syncthreads();
-    c2c_columns_inplace<N>(sm);
-    sm.twiddles(g_tw, false);
+    const float* Ti = T + map * N * H;
+    for (int e = threadIdx.x; e < H * 16; e += TH) {
+        const int kx = e % H, k1 = e / H;
+        float2* col = F + R * k1 * P + kx;
+        float2 v[R];
+#pragma unroll
+        for (int b = 0; b < R; ++b) v[b] = col[b * P];
+        dft<R, false>(v);
+#pragma unroll
+        for (int k2 = 0; k2 < R; ++k2) v[k2] = c_scale(v[k2], __ldg(Ti + (k1 + 16 * k2) * H + kx));
+        dft<R, true>(v);
+#pragma unroll
+        for (int b = 0; b < R; ++b) col[b * P] = b ? c_mulc(tw[b * k1], v[b]) : v[b];
+    }
     __syncthreads();
-    float* o = out + (size_t)i * N * N;
-    const float inv = 1.0f / ((float)N * N);
-    c2r_rows<N>(sm, [&](int y, int x, float v) { o[y * N + x] = v * inv; });
+    for (int e = threadIdx.x; e < H * R; e += TH) {
+        const int kx = e % H, b = e / H;
+        float2* col = F + b * P + kx;
+        float2 x[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) x[k] = col[R * k * P];
+        dft<16, true>(x);
+#pragma unroll
+        for (int a = 0; a < 16; ++a) col[R * a * P] = x[a];
+    }
+    __syncthreads();
+    // rows: C(k) = G_2p(k) + i G_2p+1(k) of the Hermitian rows G (the imaginary parts at k = 0 and N/2 do not
+    // count), transformed back: its real and imaginary parts are the two rows of the map
+    constexpr float inv = 0.5f / ((float)N * N);
+    float* o = out + map * N * N;
+    for (int g = warp; g < N / 8; g += NW) {
+        float2* const buf = F + (size_t)2 * (4 * g + (lane >> 3)) * P;
+        float2 u[R], v[R], dA[R / 2], dB[R / 2];
+        auto join = [&](int k, float2& c, float2& d) {
+            const float2 g0 = buf[k], g1 = buf[P + k];
+            c = make_float2(g0.x - g1.y, g0.y + g1.x);
+            d = make_float2(g0.x + g1.y, g1.x - g0.y);   // C(N - k)
+        };
+#pragma unroll
+        for (int k2 = 0; k2 < R / 2; ++k2) {
+            join(kA + 16 * k2, u[k2], dA[k2]);
+            join(kB + 16 * k2, v[k2], dB[k2]);
+        }
+        const float2 mid = make_float2(buf[N / 2].x, buf[P + N / 2].x);
+        if (j == 0) u[0] = make_float2(buf[0].x, buf[P].x);
+#pragma unroll
+        for (int i = R / 2; i < R; ++i) {
+            u[i] = j ? dB[R - 1 - i] : i == R / 2 ? mid : dA[(R - i) % (R / 2)];
+            v[i] = j ? dA[R - 1 - i] : dB[R - 1 - i];
+        }
+        dft<R, true>(u);
+        dft<R, true>(v);
+        __syncwarp();
+#pragma unroll
+        for (int b = 0; b < R; ++b) {
+            buf[17 * b + kA] = c_mulc(tw[b * kA], u[b]);
+            buf[17 * b + kB] = c_mulc(tw[b * kB], v[b]);
+        }
+        __syncwarp();
+        for (int t = lane; t < 4 * R; t += 32) {
+            const int p = 4 * g + t / R, b = t % R;
+            const float2* run = F + (size_t)2 * p * P + 17 * b;
+            float2 x[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) x[k] = run[k];
+            dft<16, true>(x);
+            float* row = o + (size_t)2 * p * N + b;
+#pragma unroll
+            for (int a = 0; a < 16; ++a) {
+                row[R * a] = x[a].x * inv;
+                row[N + R * a] = x[a].y * inv;
+            }
+        }
+        __syncwarp();
+    }
 }
 
 // Real-space image of a stored unit-norm half spectrum S (Eq. 3, inverse transform):
