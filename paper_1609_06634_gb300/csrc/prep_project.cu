@@ -14,7 +14,7 @@
 // conjugate of Eq. 2's transform; the scoring kernel applies the matching inverse phase, so the
 // correlation it evaluates is C_co(d) = sum_r o(r) I1(r + d) with d as in Eq. 7.  These
 // transforms run once per image and once per orientation, so they are plain dense DFT sums over
-// shared memory; the hot loop is the scoring kernel.
+// shared memory, but for the maps', which go by factors; the hot loop is the scoring kernel.
 #include <math.h>
 #include <stdarg.h>
 #include <stdio.h>
@@ -1091,11 +1091,10 @@ int launch_synthetic_n(bioem_ctx* ctx, const float* d_atoms, int n_atoms, double
                                                    reinterpret_cast<const float4*>(d_quats), sigma_A, pixel_A, d_I0);
     bioem_launch_end(ctx, KID_PROJECT);
     rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_project");
-    const size_t sm = DftSm<N>::bytes();
-    if (!rc && set_smem<N>((const void*)k_psf_real<N>, sm)) rc = bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");
+    if (!rc && set_smem<N>((const void*)k_psf_real<N>, Fft<N>::SMEM)) rc = bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");
     if (!rc) {
         bioem_launch_begin(ctx, KID_PSF_REAL);
-        k_psf_real<N><<<n, Dft<N>::T, sm, ctx->stream>>>(d_I0, bioem_twiddles(ctx, N), d_T, d_out);
+        k_psf_real<N><<<n, Fft<N>::T, Fft<N>::SMEM, ctx->stream>>>(d_I0, bioem_twiddles(ctx, N), d_T, d_out);
         bioem_launch_end(ctx, KID_PSF_REAL);
         rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_psf_real");
     }
