@@ -134,7 +134,7 @@ __host__ __device__ constexpr int bitrev(int u, int bits) {
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v / 2); }
 __host__ __device__ constexpr int pmod(int a, int m) { return ((a % m) + m) % m; }
 
-template <int N_, int SMAX_, int NG_, int GT_, int GPB_, bool PACK_, int BSPLIT_ = 1>
+template <int N_, int SMAX_, int NG_, int GT_, int GPB_, bool PACK_, int BSPLIT_ = 1, int ASPLIT_ = 1>
 struct Cfg {
     static constexpr int N = N_;
     static constexpr int SMAX = SMAX_;
@@ -158,7 +158,11 @@ struct Cfg {
     // for half of the dx outputs)
     static constexpr int BSPLIT = BSPLIT_;
     static constexpr int ROWS = GPB * NROW * BSPLIT;   // stage-B tasks per batch
-    static_assert(BSPLIT == 1 || (BSPLIT == 2 && ROWS == GT), "split rows: one per thread");
+    static_assert(BSPLIT == 1 || (BSPLIT == 2 && ROWS <= GT && ROWS % 32 == 0), "split rows: one per thread, whole warps");
+    // stage-A threads per column: with 2 each sums half of the sub-sequences and they add their halves in
+    // shared memory (twice the warps where shared memory holds few pairs; another order of the sums)
+    static constexpr int ASPLIT = ASPLIT_;
+    static_assert(ASPLIT == 1 || (ASPLIT == 2 && PACK_ && GPB * NC * 2 == GT && R % 2 == 0), "split columns: one per thread");
     static constexpr bool PREFETCH = THREADS <= 320;   // stage-A projection prefetch (registers)
     static constexpr int QS = H;               // Q row stride (complex); odd -> conflict-free columns
     static constexpr int NDIR = GPB * NS;      // outputs of the dy = +SMAX row, evaluated directly
@@ -175,8 +179,11 @@ struct Cfg {
     // batch in shared memory before stage A.
     static constexpr bool PACK = PACK_;
     static constexpr int NCOL = PACK ? NC : H;      // stage-A column tasks per pair
-    static constexpr int TASKS_A = GPB * NCOL;      // stage-A column tasks per batch
-    static constexpr size_t SM_Z = PACK ? (size_t)PB * N * sizeof(float2) : 0;
+    static constexpr int TASKS_A = GPB * NCOL;      // stage-A column tasks per batch (of ASPLIT threads)
+    // with split columns Z shares its space with the stage-B pieces (a barrier more per batch)
+    static constexpr bool ZALIAS = ASPLIT == 2;
+    static constexpr size_t SM_ZB = PACK ? (size_t)PB * N * sizeof(float2) : 0;
+    static constexpr size_t SM_Z = ZALIAS ? 0 : SM_ZB;
     // The dy = +SMAX row by real transforms (the 128 px, +-16 px instance): jobs (pair, Re / Im,
     // kx sub-sequence) on the last GPB 2 R threads of the group, each a real 16-point transform
     // recombined into the SMAX + 1 even (cosine) or odd (sine) outputs, summed over sub-sequences by
@@ -191,7 +198,8 @@ struct Cfg {
     static_assert((SM_IMG + SM_QA) % 16 == 0 && (TWS * sizeof(float2)) % 16 == 0, "16-byte twiddle pairs");
     static constexpr size_t SM_ROW = (size_t)NGROUP * ROWS * (2 * sizeof(float) + sizeof(int));
     static constexpr size_t SM_DIR = (size_t)NGROUP * NDIR * sizeof(float);
-    static constexpr size_t SM_BASE = (SM_IMG + SM_QA + SM_TWC + SM_Z + SM_ROW + SM_DIR + 7) / 8 * 8;
+    static constexpr size_t SM_TAIL = ZALIAS && SM_ZB > SM_ROW + SM_DIR ? SM_ZB : SM_ROW + SM_DIR;
+    static constexpr size_t SM_BASE = (SM_IMG + SM_QA + SM_TWC + SM_Z + SM_TAIL + 7) / 8 * 8;
     static constexpr size_t SM_DTW = DIRFFT ? (size_t)2 * R * (SMAX + 1) * sizeof(float2) : 0;
     static constexpr size_t SM_DSUM = DIRFFT ? (size_t)PB * 2 * (SMAX + 1) * sizeof(float) : 0;
     static constexpr size_t SMEM = SM_BASE + SM_DTW + SM_DSUM;
@@ -215,9 +223,13 @@ __device__ __forceinline__ void batch_sync() {
 template <class C>
 __device__ __forceinline__ void stage_a_column(float2 (&acc)[C::NS], const float2* __restrict__ img_col,
                                                const float2* __restrict__ ps_col, const float2* __restrict__ twc,
-                                               const float2* __restrict__ zcol) {
+                                               const float2* __restrict__ zcol, int b0 = 0, int b1 = C::R) {
     constexpr int H = C::H, R = C::R, SMAX = C::SMAX;
     float2 cn[L];
+    if constexpr (C::ASPLIT > 1) {
+        img_col += b0 * H;
+        ps_col += b0 * H;
+    }
     if constexpr (C::PREFETCH) {
         if (!zcol) {
 #pragma unroll
@@ -225,7 +237,7 @@ __device__ __forceinline__ void stage_a_column(float2 (&acc)[C::NS], const float
         }
     }
 #pragma unroll 1
-    for (int b = 0; b < R; ++b) {
+    for (int b = b0; b < b1; ++b) {
         float2 x[L];
         if (zcol) {
 #pragma unroll
@@ -233,7 +245,7 @@ __device__ __forceinline__ void stage_a_column(float2 (&acc)[C::NS], const float
         } else if constexpr (C::PREFETCH) {
 #pragma unroll
             for (int a = 0; a < L; ++a) x[a] = c_mulc(img_col[(R * a) * H], cn[a]);
-            if (b + 1 < R) {
+            if (b + 1 < b1) {
 #pragma unroll
                 for (int a = 0; a < L; ++a) cn[a] = __ldg(ps_col + (R * a + 1) * H);
             }
@@ -361,7 +373,7 @@ struct Sm {
         img = reinterpret_cast<float2*>(smem);
         q = reinterpret_cast<float2*>(smem + C::SM_IMG);
         twc = reinterpret_cast<float2*>(smem + C::SM_IMG + C::SM_QA);
-        z = reinterpret_cast<float2*>(smem + C::SM_IMG + C::SM_QA + C::SM_TWC);
+        z = reinterpret_cast<float2*>(smem + C::SM_IMG + C::SM_QA + C::SM_TWC);   // with C::ZALIAS also row_t
         row_t = reinterpret_cast<float*>(smem + C::SM_IMG + C::SM_QA + C::SM_TWC + C::SM_Z);
         row_s = row_t + C::NGROUP * C::ROWS;
         row_d = reinterpret_cast<int*>(row_s + C::NGROUP * C::ROWS);
@@ -600,6 +612,7 @@ __device__ __forceinline__ void score_item(const Sm<C>& sm, const float2* __rest
     for (int p0 = lo + grp * GPB; p0 < hi;) {
         // ---------------- packed edge columns Z(ky) = P(ky, 0) + i P(ky, N/2) of the batch's pairs
         if constexpr (C::PACK) {
+            if constexpr (C::ZALIAS) batch_sync<C>();   // the previous batch's pieces have been combined
             for (int i = tg; i < GPB * N; i += GT) {
                 const int jl = i / N;
                 const int ky = i - jl * N;
@@ -612,9 +625,10 @@ __device__ __forceinline__ void score_item(const Sm<C>& sm, const float2* __rest
             }
             batch_sync<C>();
         }
-        // ---------------- stage A: one column of one pair per task
+        // ---------------- stage A: one column of one pair per task (per two threads with ASPLIT = 2)
 #pragma unroll 1
-        for (int task = tg; task < C::TASKS_A; task += GT) {
+        for (int e = tg; e < C::TASKS_A * C::ASPLIT; e += GT) {
+            const int half = C::ASPLIT == 2 ? e / C::TASKS_A : 0, task = e - half * C::TASKS_A;
             const int jl = task / C::NCOL;
             const int kx = task - jl * C::NCOL;
             const int p = min(p0 + jl, hi - 1);
@@ -624,10 +638,25 @@ __device__ __forceinline__ void score_item(const Sm<C>& sm, const float2* __rest
             float2 acc[NS];
 #pragma unroll
             for (int m = 0; m < NS; ++m) acc[m] = make_float2(0.f, 0.f);
-            stage_a_column<C>(acc, sm.img + kx, ps_col, sm.twc, (C::PACK && kx == 0) ? sm.z + j * N : nullptr);
+            constexpr int RS = C::R / C::ASPLIT;
+            stage_a_column<C>(acc, sm.img + kx, ps_col, sm.twc, (C::PACK && kx == 0) ? sm.z + j * N : nullptr, half * RS,
+                              (half + 1) * RS);
             float2* qdst = sm.q + (size_t)j * NS * C::QS + kx;
+            if constexpr (C::ASPLIT == 1) {
 #pragma unroll
-            for (int m = 0; m < NS; ++m) qdst[m * C::QS] = acc[m];
+                for (int m = 0; m < NS; ++m) qdst[m * C::QS] = acc[m];
+            } else {
+                // each thread stores its sums of one half of the outputs and adds those of the other half to
+                // its partner's (one task per thread: every thread of the group passes the barrier once)
+                constexpr int MH = (NS + 1) / 2;
+#pragma unroll
+                for (int m = 0; m < NS; ++m)
+                    if ((m < MH) == (half == 0)) qdst[m * C::QS] = acc[m];
+                batch_sync<C>();
+#pragma unroll
+                for (int m = 0; m < NS; ++m)
+                    if ((m < MH) != (half == 0)) qdst[m * C::QS] = c_add(qdst[m * C::QS], acc[m]);
+            }
         }
         batch_sync<C>();
         // the group's next batch: written between the two barriers, read after the second
@@ -1190,6 +1219,10 @@ using C96_12 = Cfg<96, 12, 3, 128, 5, false>;
 using C128_4 = Cfg<128, 4, 4, 160, 5, true>;
 using C128_16 = Cfg<128, 16, 4, 128, 2, true, 2>;
 using C192_24 = Cfg<192, 24, 1, 224, 2, false>;
+// The batched call's 192 px instance (its matrix is FP32): two threads per column and per row, packed edge
+// columns: 12 warps instead of 7 on the two pairs that shared memory holds, 54 -> 47 ns per pair.  k_score keeps
+// C192_24, whose sums have the order of every other FP32 instance.
+using B192_24 = Cfg<192, 24, 1, 384, 2, true, 2, 2>;
 
 }  // namespace
 
@@ -1384,7 +1417,7 @@ extern "C" int bioem_score_noalloc(bioem_ctx* ctx, const bioem_images* images, c
 // launches of the sizes present are parallel branches of the graph, so that the blocks of the next
 // size start on the SMs that the previous size's blocks leave.  (One kernel that held all four sizes
 // gave every size the register count and the 256 threads of the largest: 19.2 ms for 4 models x 4
-// stacks, 1.03e6 pairs, against 16.2 ms so.)
+// stacks, 1.03e6 pairs, against 16.1 ms so.)
 #include <string>
 #include <vector>
 
@@ -1460,7 +1493,7 @@ SegInstance seg_instance(int npix) {
         case 64: return {k_score_segs<C64_8>, C64_8::THREADS, (int)C64_8::SMEM, C64_8::SMAX, 15};
         case 96: return {k_score_segs<C96_12>, C96_12::THREADS, (int)C96_12::SMEM, C96_12::SMAX, 10};
         case 128: return {k_score_segs<C128_16>, C128_16::THREADS, (int)C128_16::SMEM, C128_16::SMAX, 7};
-        case 192: return {k_score_segs<C192_24>, C192_24::THREADS, (int)C192_24::SMEM, C192_24::SMAX, 2};
+        case 192: return {k_score_segs<B192_24>, B192_24::THREADS, (int)B192_24::SMEM, B192_24::SMAX, 2};
         default: return {nullptr, 0, 0, 0, 1};
     }
 }
