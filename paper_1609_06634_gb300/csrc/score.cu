@@ -208,6 +208,12 @@ struct Cfg {
     static constexpr size_t SM_GTW = GTW ? (size_t)N * sizeof(float2) : 0;
     static constexpr size_t SMEM = SM_BASE + SM_DTW + SM_DSUM + SM_GTW;
     static_assert(SMEM <= kScoreSmemLimit, "dynamic shared memory per block");
+    // Work by phases (k_score_phases) or by chunks from a counter (k_score).  Phases have fewer waits and end
+    // evenly, but spread the blocks over all of a phase's spectra, which the instances with two pairs per group
+    // feel: they read the most per second with the fewest warps.  ns per pair, chunks -> phases: 32 px 0.85 ->
+    // 0.78; 64 px, s = 4: 2.16 -> 2.07, s = 8: 3.05 -> 2.90; 96 px 6.94 -> 6.85; 128 px, s = 4: 7.3 -> 6.87; but 128 px,
+    // s = 16: 12.1 -> 12.4 (512 images: 11.59 -> 12.0); 192 px 49.2 -> 49.6 to 50.3.
+    static constexpr bool PHASES = GPB > 2;
     // lanes that combine a pair's pieces (NROW BSPLIT rows and NS direct outputs)
     static constexpr int LPP = SMAX <= 12 ? 8 : 32;
 };
@@ -752,6 +758,39 @@ k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int
     }
 }
 
+// The wave's sets go by in phases of phase_sets, whose spectra stay in the L2.  Within a phase the (image, batch)
+// pairs, image by image, are split evenly over the blocks, counting a new image as kImageUnits batches
+// of a group (its load and the wait of the groups for one another): a block meets one image, or the end of one
+// and the start of the next, and every block ends a phase at the same time.
+template <class C>
+__global__ void __launch_bounds__(C::THREADS, 1)
+k_score_phases(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int n_img,
+        const float2* __restrict__ ps_spec, int ps_begin, int ps_count, int phase_sets, int s, float c1,
+        float* __restrict__ rec_t, float* __restrict__ rec_s, int* __restrict__ rec_d, int* __restrict__ status) {
+    constexpr int kImageUnits = (6 * C::NGROUP + 5) / 10 > 0 ? (6 * C::NGROUP + 5) / 10 : 1;   // about 0.6 of a round
+    extern __shared__ __align__(16) unsigned char smem[];
+    const Sm<C> sm(smem);
+    score_tables<C>(sm, gtw);
+    for (int f0 = 0; f0 < ps_count; f0 += phase_sets) {
+        const int f1 = min(f0 + phase_sets, ps_count);
+        const int units = (f1 - f0 + C::GPB - 1) / C::GPB, stride = units + kImageUnits;
+        const long long all = (long long)n_img * stride;
+        // (the blocks' parts shift from phase to phase, so that none always gets two images)
+        const int part = (int)((blockIdx.x + 61ll * (f0 / phase_sets)) % gridDim.x);
+        const long long x0 = all * part / gridDim.x, x1 = all * (part + 1) / gridDim.x;
+        for (int w = (int)(x0 / stride); w < n_img; ++w) {
+            const long long at = (long long)w * stride + kImageUnits;   // of the image's first batch
+            if (at >= x1) break;
+            const int u0 = (int)max(x0 - at, 0ll), u1 = (int)min(x1 - at, (long long)units);
+            if (u0 >= u1) continue;
+            const size_t row = (size_t)w * ps_count;
+            score_item<C>(sm, Job{gtw, img_spec + (size_t)w * C::N * C::H, nullptr, ps_spec, ps_begin, s, c1, rec_t + row,
+                                  rec_s + row, rec_d + row},
+                          f0 + u0 * C::GPB, min(f0 + u1 * C::GPB, f1), status);
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------- reductions (float64)
 struct Acc {
     double M;    // running max
@@ -1151,10 +1190,13 @@ int run_waves(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, i
 template <class C>
 int score_slots(bioem_ctx* ctx, int* slots) {
     const size_t smem = C::SMEM;
-    if (cudaFuncSetAttribute(k_score<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    const void* kernel;
+    if constexpr (C::PHASES) kernel = (const void*)k_score_phases<C>;
+    else kernel = (const void*)k_score<C>;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return bioem_set_error(ctx, BIOEM_ERR_CUDA, "shared memory attribute (%zu bytes)", smem);
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_score<C>, C::THREADS, smem) != cudaSuccess || per_sm < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, C::THREADS, smem) != cudaSuccess || per_sm < 1)
         return bioem_set_error(ctx, BIOEM_ERR_CUDA, "occupancy query");
     *slots = per_sm * ctx->num_sms;
     return BIOEM_OK;
@@ -1191,33 +1233,56 @@ int score_chunk(int n_img, int wl, int slots) {
     return (int)best;
 }
 
+// Parameter sets of a phase: 48 MB of spectra, which the L2 keeps (it is two halves, and what one reads from the
+// other's memory it holds too: 128 px, s = 4, ns per pair: 24 MB 7.07, 32: 7.04, 48: 6.92, 64: 7.26, 96: 7.71),
+// but at least eight rounds of every block.
+template <class C>
+int phase_sets(int n_img, int wl, int slots) {
+    constexpr long long spec = (long long)sizeof(float2) * C::N * C::H;
+    long long fit = (48ll << 20) / spec;
+    const long long least = (8ll * C::PB * slots + n_img - 1) / n_img;
+    if (fit < least) fit = least;
+    const long long phases = (wl + fit - 1) / fit;
+    return (int)(((wl + phases - 1) / phases + C::GPB - 1) / C::GPB * C::GPB);
+}
+
 // One k_score<C> launch writing the records of parameter sets [wbegin, wbegin + wl) for every image.
 template <class C>
 int launch_score_records(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, int slots, int wbegin,
                          int wl, int max_shift, float* rec_t, float* rec_s, int* rec_d) {
     const int n_img = im->n_img;
-    const long long chunk = score_chunk<C>(n_img, wl, slots);
-    // with more items than slots, about the last item of each slot goes out in short chunks: ns per pair
-    // without -> with: 128 px, s = 4: 7.74 -> 7.37; 96 px 7.66 -> 7.43; 64 px, s = 4: 2.25 -> 2.19 (two or three
-    // items' worth gained no more)
-    long long n_chunks = (wl + chunk - 1) / chunk, n_long = n_chunks;
-    if (n_chunks * n_img > slots && chunk >= 4 * C::GPB) {
-        n_long = wl / chunk - ((long long)slots + n_img - 1) / n_img;
-        if (n_long < 0) n_long = 0;
-        const int tail = short_chunk<C>((int)chunk);
-        n_chunks = n_long + (wl - n_long * chunk + tail - 1) / tail;
-    }
-    const long long n_items = n_chunks * n_img;
-    if (n_items > 0x7fffffffll) return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "too many work items");
-    const int grid = (int)(n_items < slots ? n_items : slots);
     const float c1f = 0.5f * (3.0f - (float)(C::N * C::N));
-    bioem_launch_begin(ctx, KID_SCORE);
-    if (cudaMemsetAsync(ctx->d_work, 0, sizeof(int), ctx->stream) != cudaSuccess)
-        return bioem_check_cuda(ctx, cudaGetLastError(), "work counter");
-    k_score<C><<<grid, C::THREADS, C::SMEM, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, ps->d_spec,
-                                                            wbegin, wl, (int)chunk, (int)n_long, (int)n_items, max_shift, c1f,
-                                                            rec_t, rec_s, rec_d, ctx->d_status, ctx->d_work);
-    bioem_launch_end(ctx, KID_SCORE);
+    if constexpr (C::PHASES) {
+        const int phase = phase_sets<C>(n_img, wl, slots);
+        const long long units = (long long)n_img * ((phase + C::GPB - 1) / C::GPB);
+        const int grid = (int)(units < slots ? units : slots);
+        bioem_launch_begin(ctx, KID_SCORE);
+        k_score_phases<C><<<grid, C::THREADS, C::SMEM, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, ps->d_spec,
+                                                                wbegin, wl, phase, max_shift, c1f, rec_t, rec_s, rec_d,
+                                                                ctx->d_status);
+        bioem_launch_end(ctx, KID_SCORE);
+    } else {
+        const long long chunk = score_chunk<C>(n_img, wl, slots);
+        // with more items than slots, about the last item of each slot goes out in short chunks: 13.19 -> 12.94 ns
+        // per pair at 128 px, +-16 px, 64 images (two or three items' worth gained no more)
+        long long n_chunks = (wl + chunk - 1) / chunk, n_long = n_chunks;
+        if (n_chunks * n_img > slots && chunk >= 4 * C::GPB) {
+            n_long = wl / chunk - ((long long)slots + n_img - 1) / n_img;
+            if (n_long < 0) n_long = 0;
+            const int tail = short_chunk<C>((int)chunk);
+            n_chunks = n_long + (wl - n_long * chunk + tail - 1) / tail;
+        }
+        const long long n_items = n_chunks * n_img;
+        if (n_items > 0x7fffffffll) return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "too many work items");
+        const int grid = (int)(n_items < slots ? n_items : slots);
+        bioem_launch_begin(ctx, KID_SCORE);
+        if (cudaMemsetAsync(ctx->d_work, 0, sizeof(int), ctx->stream) != cudaSuccess)
+            return bioem_check_cuda(ctx, cudaGetLastError(), "work counter");
+        k_score<C><<<grid, C::THREADS, C::SMEM, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, ps->d_spec,
+                                                                wbegin, wl, (int)chunk, (int)n_long, (int)n_items, max_shift, c1f,
+                                                                rec_t, rec_s, rec_d, ctx->d_status, ctx->d_work);
+        bioem_launch_end(ctx, KID_SCORE);
+    }
     return bioem_check_cuda(ctx, cudaGetLastError(), "k_score");
 }
 
@@ -1255,10 +1320,10 @@ int run_score_gemm(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* 
 // stage-B row]>.  Groups as many as registers allow without spills and shared memory holds; a group's batch
 // fills whole rounds of its threads with column tasks (PB N/2 with the packed edge columns, PB (N/2 + 1)
 // without) and at most one round with rows.  ns per pair (k_score, one GB300; one block-wide group of
-// 245-272 threads moving through the phases in step before -> now): 32 px 1.76 -> 0.85; 64 px, s = 4: 3.68 ->
-// 2.19, s = 8: 5.22 -> 3.1; 96 px 10.5 -> 7.4; 128 px, s = 4: 14.7 -> 7.4.  More groups at fewer registers lost
+// 245-272 threads moving through the phases in step before -> now): 32 px 1.76 -> 0.78; 64 px, s = 4: 3.68 ->
+// 2.07, s = 8: 5.22 -> 2.90; 96 px 10.5 -> 6.85; 128 px, s = 4: 14.7 -> 6.87.  More groups at fewer registers lost
 // (128 px, s = 4: 6 x 128 threads of 79 registers 9.9; 8 x 64 threads 10.4), as did fewer, larger ones
-// (3 x 192 threads 7.9, 3 x 256 10.0).  192 px holds two pairs beside the image: one group in step, 54
+// (3 x 192 threads 7.9, 3 x 256 10.0).  192 px holds two pairs beside the image: one group in step, 49
 // (as two groups of one pair 64: the 97th column then takes a warp per group; the image read through L1 and
 // three pairs in 10 or 12 warps: 62-73).  The odd column kx = N/2
 // stays a column task: spread over a warp's lanes (transforms, then outputs) it took fewer

@@ -86,3 +86,24 @@ def test_reduction_parts_and_waves(env, n_img, n_defocus, bfactors):
     np.testing.assert_allclose(one["logP"].cpu().numpy()[:3], ref["logP"], rtol=0, atol=TOL)
     np.testing.assert_allclose(one["logP_orient"].cpu().numpy()[:3], ref["logP_orient"], rtol=0, atol=TOL)
     np.testing.assert_allclose(one["best_logL"].cpu().numpy()[:3], [b[4] for b in ref["best"]], rtol=0, atol=TOL)
+
+
+# more spectra than one phase (or several chunks, at the +-16 px window), images fewer than, near and above the
+# number of SMs, so that blocks get parts of one image, two images, or several
+@pytest.mark.parametrize("npix,shift,n_img,n_orient", [
+    (32, 4, 37, 1500), (64, 4, 41, 420), (64, 8, 153, 420), (96, 12, 29, 331), (128, 4, 37, 201), (128, 4, 1, 201),
+    (128, 4, 307, 13), (128, 16, 37, 201)])
+def test_whole_range_equals_its_parts(env, npix, shift, n_img, n_orient):
+    """Per-pair values of a long range are, bit for bit, those of short ranges of the same sets."""
+    bioem, ctx = env
+    cfg, wl, _ = _case(npix, shift, 1, n_orient, 4, (0.0, 50.0))
+    imgs = np.random.default_rng(npix + n_img).standard_normal((n_img, npix, npix)).astype(np.float32)
+    im = bioem.prepare_images(ctx, _dev(imgs), cfg.pixel_A)
+    ps = bioem.project_model(ctx, _dev(wl["atoms"]), cfg.sigma_A, _dev(wl["quats"]), wl["ctfs"], npix, cfg.pixel_A)
+    n_ps = n_orient * 8
+    pmax, plse = bioem.score_pairs(ctx, im, ps, shift)
+    for begin in range(0, n_ps, 333):
+        count = min(333, n_ps - begin)
+        a, b = bioem.score_pairs(ctx, im, ps, shift, begin, count)
+        assert (a == pmax[:, begin:begin + count]).all() and (b == plse[:, begin:begin + count]).all(), begin
+    assert bool((pmax == pmax).all()) and ctx.status() == 0
