@@ -2079,38 +2079,59 @@ void bioem_batch_free(bioem_batch* b) {
 // projection set), folded into running per-image float64 (max, sum) accumulators.
 namespace {
 
+// The lists, end to end, are split evenly over the blocks, counting an image as kImageSets more sets (its load
+// and the wait of the groups for one another, 0.6 of a round); parts end on whole group batches of their
+// image's list.  k_score us, items of one image from a counter -> so: 64 images of 512 sets, 128 px, s = 4: 320 ->
+// 260; 300 images of 173 sets, 64 px: 214 -> 176; 1024 images of 225 sets, 128 px, s = 16: 2.95 ms either way.
 template <class C>
 __global__ void __launch_bounds__(C::THREADS, 1)
 k_score_gathered(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int n_img,
-                 const int* __restrict__ offsets, const int* __restrict__ ps_idx, const float2* __restrict__ ps_spec,
-                 int chunk, int chunks_per_img, int s, float c1, float* __restrict__ rec_t, float* __restrict__ rec_s,
-                 int* __restrict__ rec_d, int* __restrict__ status, unsigned long long* __restrict__ work) {
+                 const int* __restrict__ offsets, const int* __restrict__ ps_idx, const float2* __restrict__ ps_spec, int s,
+                 float c1, float* __restrict__ rec_t, float* __restrict__ rec_s, int* __restrict__ rec_d,
+                 int* __restrict__ status) {
+    constexpr int kImageSets = (6 * C::PB + 5) / 10, GPB = C::GPB;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ long long next_item;
-    const long long n_items = (long long)n_img * chunks_per_img;
+    __shared__ Job job;
+    __shared__ long long x0, x1;   // the block's part
+    __shared__ int next_w, part_lo, part_hi;
     const Sm<C> sm(smem);
     score_tables<C>(sm, gtw);
+    auto start = [&](int w) { return (long long)(offsets[w] - offsets[0]) + (long long)w * kImageSets; };
+    if (threadIdx.x == 0) {
+        const long long all = start(n_img);
+        x0 = all * blockIdx.x / gridDim.x;
+        x1 = all * (blockIdx.x + 1) / gridDim.x;
+        int w = 0;   // the last image that starts at or before x0
+        for (int hi = n_img - 1; w < hi;) {
+            const int mid = (w + hi + 1) >> 1;
+            if (start(mid) <= x0) w = mid;
+            else hi = mid - 1;
+        }
+        next_w = w;
+    }
     for (;;) {
-        // items in index order from a global counter (zero at launch), as in k_score; the parts of a chunk
-        // index beyond the end of an image's list are passed over by the thread that takes the items
+        __syncthreads();   // the previous image's readers of the job are done
         if (threadIdx.x == 0) {
-            long long it;
-            do {
-                it = (long long)atomicAdd(work, 1ull);
-            } while (it < n_items && it / n_img * chunk >= offsets[it % n_img + 1] - offsets[it % n_img]);
-            next_item = it;
+            part_lo = part_hi = 0;
+            for (int w = next_w; w < n_img; ++w) {
+                const long long at = start(w) + kImageSets;   // of the image's first set
+                if (at >= x1) break;
+                const int b0 = offsets[w], len = offsets[w + 1] - b0;
+                const int lo = (int)((max(x0 - at, 0ll) + GPB - 1) / GPB) * GPB;
+                const int hi = min(len, (int)((min(x1 - at, (long long)len) + GPB - 1) / GPB) * GPB);
+                if (lo >= hi) continue;
+                job = Job{gtw, img_spec + (size_t)w * C::N * C::H, ps_idx + b0, ps_spec, 0, s, c1, rec_t + b0, rec_s + b0,
+                          rec_d + b0};
+                part_lo = lo;
+                part_hi = hi;
+                next_w = w + 1;
+                break;
+            }
         }
         __syncthreads();
-        const long long item = next_item;   // read by every thread before score_item's first barrier
-        if (item >= n_items) break;
-        const int ci = (int)(item / n_img);
-        const int w = (int)(item - (long long)ci * n_img);
-        const int b0 = offsets[w], b1 = offsets[w + 1];
-        const int lo = ci * chunk;
-        const int hi = min(lo + chunk, b1 - b0);
-        score_item<C>(sm, Job{gtw, img_spec + (size_t)w * C::N * C::H, ps_idx + b0, ps_spec, 0, s, c1, rec_t + b0, rec_s + b0,
-                              rec_d + b0},
-                      lo, hi, status);
+        const int lo = part_lo, hi = part_hi;
+        if (lo >= hi) break;
+        score_item<C>(sm, job, lo, hi, status);
     }
 }
 
@@ -2225,22 +2246,15 @@ int run_gathered(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_score_gathered<C>, C::THREADS, smem);
     if (per_sm < 1) per_sm = 1;
     const int slots = per_sm * ctx->num_sms;
-    // chunks as for lists of the mean length (at most 256 sets: 16 MB of the chunk's projections at 128 px)
-    int chunk = nnz >= n_img ? score_chunk<C>(n_img, (nnz + n_img - 1) / n_img, slots) : C::GPB;
-    if (chunk > 256 / C::GPB * C::GPB) chunk = 256 / C::GPB * C::GPB;
-    const int cpi = (max_per_image + chunk - 1) / chunk;
-    const long long items = (long long)n_img * cpi;
-    const int grid = (int)(items < slots ? items : slots);
+    const long long batches = (long long)n_img + nnz / C::GPB;   // at least as many as there are
+    const int grid = nnz > 0 ? (int)(batches < slots ? batches : slots) : 0;
     const int n = C::N * C::N;
     if (grid > 0) {
         bioem_launch_begin(ctx, KID_SCORE);
-        if (cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), ctx->stream) != cudaSuccess)
-            return bioem_check_cuda(ctx, cudaGetLastError(), "work counter");
         k_score_gathered<C><<<grid, C::THREADS, smem, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, offsets,
-                                                                     ps_idx, ps->d_spec, chunk, cpi, max_shift,
+                                                                     ps_idx, ps->d_spec, max_shift,
                                                                      0.5f * (3.0f - (float)n), rec_t, rec_s, rec_d,
-                                                                     ctx->d_status,
-                                                                     reinterpret_cast<unsigned long long*>(ctx->d_work));
+                                                                     ctx->d_status);
         bioem_launch_end(ctx, KID_SCORE);
         int rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_score_gathered");
         if (rc) return rc;
@@ -2313,9 +2327,9 @@ int bioem_group_logsumexp(bioem_ctx* ctx, const double* d_values, long long n_gr
     if (!ctx || n_groups < 0 || group_len < 1 || (n_groups > 0 && (!d_values || !d_out))) return BIOEM_ERR_INVALID_ARG;
     if (n_groups == 0) return BIOEM_OK;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return bioem_set_error(ctx, BIOEM_ERR_CUDA, "cudaSetDevice");
-    const long long blocks = (n_groups + 255) / 256;
+    const long long blocks = (n_groups + 63) / 64;   // few groups: over every SM's float64 pipe
     bioem_launch_begin(ctx, KID_LSE_MERGE);
-    k_group_lse<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, ctx->stream>>>(d_values, n_groups, group_len, d_out);
+    k_group_lse<<<(unsigned)(blocks < 4096 ? blocks : 4096), 64, 0, ctx->stream>>>(d_values, n_groups, group_len, d_out);
     bioem_launch_end(ctx, KID_LSE_MERGE);
     return bioem_check_cuda(ctx, cudaGetLastError(), "k_group_lse");
 }

@@ -107,3 +107,26 @@ def test_whole_range_equals_its_parts(env, npix, shift, n_img, n_orient):
         a, b = bioem.score_pairs(ctx, im, ps, shift, begin, count)
         assert (a == pmax[:, begin:begin + count]).all() and (b == plse[:, begin:begin + count]).all(), begin
     assert bool((pmax == pmax).all()) and ctx.status() == 0
+
+
+# empty lists first, last and between; one image alone; lists far longer than the others; fewer sets than blocks
+@pytest.mark.parametrize("npix,shift,lengths", [
+    (32, 4, [0, 0, 700, 1, 0, 3, 0]), (64, 8, [2100]), (96, 12, [1, 0, 1]), (128, 4, [5, 900, 0, 40, 1, 1, 260] * 9),
+    (128, 16, [0, 33, 2, 1000, 0, 7] * 30)])
+def test_gathered_lists_of_any_length(env, npix, shift, lengths):
+    """Each image against its own list: the values of the whole range's pairs, bit for bit."""
+    import torch
+    bioem, ctx = env
+    cfg, wl, _ = _case(npix, shift, 1, 150)
+    n_img = len(lengths)
+    rng = np.random.default_rng(npix)
+    im = bioem.prepare_images(ctx, _dev(rng.standard_normal((n_img, npix, npix)).astype(np.float32)), cfg.pixel_A)
+    ps = bioem.project_model(ctx, _dev(wl["atoms"]), cfg.sigma_A, _dev(wl["quats"]), wl["ctfs"], npix, cfg.pixel_A)
+    off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    idx = rng.integers(0, 150, off[-1]).astype(np.int32)
+    got = bioem.score_gathered_pairs(ctx, im, ps, shift, _dev(off), _dev(idx), max(lengths))
+    _, plse = bioem.score_pairs(ctx, im, ps, shift)
+    rows = torch.from_numpy(np.repeat(np.arange(n_img), lengths)).to(plse.device)
+    want = plse[rows, _dev(idx).long()]
+    # the pair sums of the two calls round ln L in a different order: float64, values below 1e5
+    assert float((got - want).abs().max()) < 1e-9 and ctx.status() == 0
