@@ -191,6 +191,12 @@ struct Cfg {
     static constexpr bool DIRFFT = PACK && N == 128 && SMAX == 16;
     static_assert(!DIRFFT || (GPB * NCOL == GT && BSPLIT == 2 && ((GPB * 2 * R) % 32 == 0 || GPB * 2 * R == 16)),
                   "each group's tasks on its own threads, its dy = +SMAX jobs on whole warps or half a warp");
+    // The next batch's edge columns are formed while the rows of this one are transformed, by the threads without
+    // a dy = +SMAX job (DIRFFT) or without a row or direct output.  As a step of their own before stage A, with a
+    // barrier more, 128 px took 12.09 instead of 11.84 ns per pair at s = 16 and 6.87 instead of 6.55 at s = 4; by
+    // all threads 11.92 and 6.72.
+    static constexpr int ZFIRST = DIRFFT ? 0 : (ROWS + NDIR + 31) / 32 * 32 < GT ? (ROWS + NDIR + 31) / 32 * 32 : 0;
+    static constexpr int ZCOUNT = DIRFFT ? GT - (GPB * 2 * R + 31) / 32 * 32 : GT - ZFIRST;
     // that instance keeps a second table 2 W_N^(b d) for stage B (the weight 2 of kx != 0 rides on the
     // twiddles, exact, instead of scaling every input)
     static constexpr bool TW2 = DIRFFT;
@@ -414,8 +420,10 @@ struct Job {
 // Stage B (row transforms), the dy = +SMAX row, the likelihood epilogue and the per-pair combine of
 // one batch of the calling group whose Q (stage-A output, [pair][dy][kx]) is in sm.q; records for pairs
 // p0 .. hi-1.
-template <class C>
-__device__ __forceinline__ void score_tail(const Sm<C>& sm, const Job& job, int p0, int hi, int* __restrict__ status) {
+// between: what the threads do before the pieces are combined.
+template <class C, class F>
+__device__ __forceinline__ void score_tail(const Sm<C>& sm, const Job& job, int p0, int hi, int* __restrict__ status,
+                                           F&& between) {
     const int s = job.s;
     const float c1 = job.c1;
     constexpr int N = C::N, NC = C::NC, NS = C::NS, SMAX = C::SMAX, NROW = C::NROW, BS = C::BSPLIT;
@@ -557,6 +565,7 @@ __device__ __forceinline__ void score_tail(const Sm<C>& sm, const Job& job, int 
             sm.dir_t[grp * C::NDIR + i] = ok ? loglik_t(rho, status) : INFINITY;
         }
     }
+    between();
     batch_sync<C>();
     // ---------------- combine the pieces of each pair: LPP lanes per pair, on the group's first warps
     constexpr int LPP = C::LPP, NR = NROW * BS;
@@ -632,21 +641,32 @@ __device__ __forceinline__ void score_item(const Sm<C>& sm, const Job& job, int 
         if (threadIdx.x == 0) next_pair = lo + C::PB;
     }
     __syncthreads();
+    // packed edge columns Z(ky) = P(ky, 0) + i P(ky, N/2) of the batch at p0, by the group's threads
+    // first .. first + count - 1
+    auto edge_columns = [&](int p0, int first, int count) {
+        if (tg < first || tg >= first + count) return;
+        for (int i = tg - first; i < GPB * N; i += count) {
+            const int jl = i / N;
+            const int ky = i - jl * N;
+            const int p = min(p0 + jl, hi - 1);
+            const int gp = job.ps_idx ? __ldg(job.ps_idx + p) : job.ps_begin + p;
+            const float2* ps_row = job.ps + (size_t)gp * N * H + (size_t)ky * H;
+            const float2 e0 = c_mulc(sm.img[ky * H], __ldg(ps_row));
+            const float2 e1 = c_mulc(sm.img[ky * H + NC], __ldg(ps_row + NC));
+            sm.z[grp * GPB * N + i] = make_float2(e0.x - e1.y, e0.y + e1.x);
+        }
+    };
+    if constexpr (C::PACK && !C::ZALIAS) {
+        if (lo + grp * GPB < hi) {
+            edge_columns(lo + grp * GPB, 0, GT);
+            batch_sync<C>();
+        }
+    }
 #pragma unroll 1
     for (int p0 = lo + grp * GPB; p0 < hi;) {
-        // ---------------- packed edge columns Z(ky) = P(ky, 0) + i P(ky, N/2) of the batch's pairs
-        if constexpr (C::PACK) {
-            if constexpr (C::ZALIAS) batch_sync<C>();   // the previous batch's pieces have been combined
-            for (int i = tg; i < GPB * N; i += GT) {
-                const int jl = i / N;
-                const int ky = i - jl * N;
-                const int p = min(p0 + jl, hi - 1);
-                const int gp = job.ps_idx ? __ldg(job.ps_idx + p) : job.ps_begin + p;
-                const float2* ps_row = job.ps + (size_t)gp * N * H + (size_t)ky * H;
-                const float2 e0 = c_mulc(sm.img[ky * H], __ldg(ps_row));
-                const float2 e1 = c_mulc(sm.img[ky * H + NC], __ldg(ps_row + NC));
-                sm.z[grp * GPB * N + i] = make_float2(e0.x - e1.y, e0.y + e1.x);
-            }
+        if constexpr (C::ZALIAS) {
+            batch_sync<C>();   // the previous batch's pieces have been combined
+            edge_columns(p0, 0, GT);
             batch_sync<C>();
         }
         // ---------------- stage A: one column of one pair per task (per two threads with ASPLIT = 2)
@@ -682,11 +702,16 @@ __device__ __forceinline__ void score_item(const Sm<C>& sm, const Job& job, int 
                     if ((m < MH) != (half == 0)) qdst[m * C::QS] = c_add(qdst[m * C::QS], acc[m]);
             }
         }
-        batch_sync<C>();
-        // the group's next batch: written between the two barriers, read after the second
+        // the group's next batch: written before the barrier, read between it and the next one
         if (tg == 0) group_next[grp] = atomicAdd(&next_pair, GPB);
-        score_tail<C>(sm, job, p0, hi, status);
-        p0 = group_next[grp];
+        batch_sync<C>();
+        const int pn = group_next[grp];
+        score_tail<C>(sm, job, p0, hi, status, [&]() {
+            // the next batch's edge columns by the threads that are free first (Cfg::ZFIRST)
+            if constexpr (C::PACK && !C::ZALIAS)
+                if (pn < hi) edge_columns(pn, C::ZFIRST, C::ZCOUNT);
+        });
+        p0 = pn;
     }
 }
 
@@ -1321,7 +1346,7 @@ int run_score_gemm(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* 
 // fills whole rounds of its threads with column tasks (PB N/2 with the packed edge columns, PB (N/2 + 1)
 // without) and at most one round with rows.  ns per pair (k_score, one GB300; one block-wide group of
 // 245-272 threads moving through the phases in step before -> now): 32 px 1.76 -> 0.78; 64 px, s = 4: 3.68 ->
-// 2.07, s = 8: 5.22 -> 2.90; 96 px 10.5 -> 6.85; 128 px, s = 4: 14.7 -> 6.87.  More groups at fewer registers lost
+// 2.07, s = 8: 5.22 -> 2.90; 96 px 10.5 -> 6.85; 128 px, s = 4: 14.7 -> 6.55.  More groups at fewer registers lost
 // (128 px, s = 4: 6 x 128 threads of 79 registers 9.9; 8 x 64 threads 10.4), as did fewer, larger ones
 // (3 x 192 threads 7.9, 3 x 256 10.0).  192 px holds two pairs beside the image: one group in step, 49
 // (as two groups of one pair 64: the 97th column then takes a warp per group; the image read through L1 and
