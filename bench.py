@@ -88,7 +88,7 @@ def kernel_source_sha(kernel: str) -> str:
 #   k_score: per evaluated pair, from one launch of 2048 images x 4608 sets (above L2), scaled by
 #            pairs to the bench's launches (profiles/k_score_throughput.md).
 #   k_score_gemm: per launch of the precision workloads (64 images x 6912 sets, +-4 px).
-K_SCORE_TRAFFIC = {"source_sha256": "f1d1c96b7a9aaf909575e174927254a9a99fd620c601fec5e301c2ca40fd73c8", "bytes_per_pair": (1553334016 + 118952960) / (2048 * 4608)}
+K_SCORE_TRAFFIC = {"source_sha256": "67f77ea988b4d2ce701dc6cf4863691b2f57eb4d524e737f2c8d0bca9126f5c0", "bytes_per_pair": (2361264640 + 117821696) / (2048 * 4608)}
 K_SCORE_GEMM_TRAFFIC = {"source_sha256": "083bf58cd6cd1f4630508bfac27c7d80488b5d30f742979416b2b4b648b51731", "bytes_per_launch": {
     '128/bf16x2': 3528212224, '128/fp16x2': 3795020800, '128/bf16x2_real': 3479105792, '128/fp16x2_real': 4123705344,
     '64/bf16x2': 895100672, '64/fp16x2': 895214592, '64/bf16x2_real': 868046336, '64/fp16x2_real': 867884544}}

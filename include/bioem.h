@@ -231,8 +231,8 @@ int bioem_score_noalloc(bioem_ctx* ctx, const bioem_images* images, const bioem_
  * 64, 96, 128 or 192 px) against projsets[m * n_stacks + k] (model m projected for stack k's size,
  * pixel and grid) with |d| <= max_shift[k] (at most N/8).  bioem_batch_create builds the work list
  * of all segments, allocates the per-pair records (12 bytes per pair of every segment) and captures
- * one persistent scoring launch plus one reduction launch in a CUDA graph; bioem_batch_run replays
- * the graph on the context's stream.  Output: d_logP_matrix [n_models][sum_k n_img_k] float32,
+ * one persistent scoring launch per image size plus one reduction launch in a CUDA graph;
+ * bioem_batch_run replays the graph on the context's stream.  Output: d_logP_matrix [n_models][sum_k n_img_k] float32,
  * ln P(image | model) as bioem_score computes it, images of stack k in columns
  * [sum_{k'<k} n_img_k', ...).  Handles must outlive the batch.  Work items use the chunk size
  * chosen by bioem_autotune for their (size, shift window), or a default.
@@ -253,7 +253,7 @@ int bioem_autotune(bioem_ctx* ctx, const bioem_images* images, const bioem_projs
 
 /* Load an autotune cache file into this process's table without tuning (no device work).  Only
  * lines "npix shift chunk" with npix in {64, 96, 128, 192}, 0 <= shift <= npix/8 and chunk a
- * positive multiple of the batched instance's pairs per batch, at most 4096, are taken; any other
+ * positive multiple of the size's tuning unit (15, 10, 7, 2 sets), at most 4096, are taken; any other
  * non-blank line is skipped (bioem_autotune then tunes that case afresh and rewrites the file with
  * valid lines only).  *n_taken / *n_skipped (either may be NULL) receive the counts.
  * Errors: INVALID_ARG (NULL path, or the file cannot be opened). */
