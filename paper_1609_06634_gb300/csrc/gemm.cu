@@ -287,19 +287,23 @@ __device__ __forceinline__ void part_add(Part& st, float& r2max, float v, float 
 
 __device__ __forceinline__ bool warp_all(bool ok) { return __all_sync(0xffffffffu, ok) != 0; }
 
-// OR of `flag` over the 256 epilogue threads (named barrier 1; every epilogue thread must arrive).  The
-// forms without .aligned: per-lane stores precede both barriers.
+// OR of `flag` over the 256 epilogue threads (named barrier 1; every epilogue thread must arrive).
+// Per-lane stores precede both barriers, which are the .aligned forms: the lanes are brought together first.
 __device__ __forceinline__ bool epilogue_any(bool flag) {
     uint32_t r;
+    __syncwarp();
     asm volatile(
-        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
         : "=r"(r)
         : "r"((uint32_t)flag), "r"(EPI_THREADS)
         : "memory");
     return r != 0;
 }
 
-__device__ __forceinline__ void epilogue_sync() { asm volatile("barrier.sync 1, %0;" ::"r"(EPI_THREADS) : "memory"); }
+__device__ __forceinline__ void epilogue_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, %0;" ::"r"(EPI_THREADS) : "memory");
+}
 
 __global__ void __launch_bounds__(GEMM_THREADS, 1) k_score_gemm(const GemmArgs g) {
     extern __shared__ __align__(1024) unsigned char smem[];

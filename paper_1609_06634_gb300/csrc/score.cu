@@ -225,11 +225,13 @@ struct Cfg {
 };
 
 // The batch loop's barrier: the calling thread's group (named barrier 1 + group over C::GT threads).
-// barrier.sync, not bar.sync: the latter is the .aligned form, undefined for a warp whose lanes are apart, and
-// code whose trip counts differ from lane to lane (rows, direct outputs, large rho^2) runs up to this barrier.
+// bar.sync is the .aligned form, undefined for a warp whose lanes are apart, and code whose trip counts differ from
+// lane to lane (rows, direct outputs, large rho^2) runs up to it: the lanes are brought together first.
+// (barrier.sync, which needs no convergence, took 53.67 instead of 53.28 ms for 512 images x 9216 sets.)
 template <class C>
 __device__ __forceinline__ void batch_sync() {
-    asm volatile("barrier.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / C::GT), "n"(C::GT) : "memory");
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / C::GT), "n"(C::GT) : "memory");
 }
 
 // Stage A for one column kx of one pair: Q(dy, kx) for dy = -SMAX..SMAX, with the rows ky = b + R a
