@@ -1518,7 +1518,9 @@ int bioem_propose(bioem_cnn* n, const float* d_images, int n_img, int k, int* d_
     int n2 = 64;   // entries of the sorting network: a power of two, at least a warp's 64
     while (sorted && n2 < k) n2 *= 2;
     const size_t sm = (size_t)n2 * 6;
-    if (sorted && cudaFuncSetAttribute(k_topk_joint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+    // the limit belongs to the function on this device, not to this call: the same value from every caller, so
+    // that one on another thread cannot lower it before the launch
+    if (sorted && cudaFuncSetAttribute(k_topk_joint, cudaFuncAttributeMaxDynamicSharedMemorySize, 6 * kTopMaxK) != cudaSuccess)
         return bioem_check_cuda(n->ctx, cudaGetLastError(), "top-k shared memory");
     for (int b0 = 0; b0 < n_img; b0 += n->max_batch) {
         const int B = n_img - b0 < n->max_batch ? n_img - b0 : n->max_batch;
