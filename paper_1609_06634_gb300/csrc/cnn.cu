@@ -335,6 +335,10 @@ __global__ void __launch_bounds__(kConvT) k_conv_bwd_data2(const float* __restri
 // together (row by row, each waited for, they took longer than the products: 281 us for the 32 x 32 px stride-1
 // layer of 256 samples against 115).  Channel strides are 4 x odd floats, so the 16-byte reads of 8
 // neighbouring channels do not conflict.
+// Only products of a gradient that is not 0 with a value inside the image count: a value that is not finite
+// behind a ReLU that stopped it (an image of NaN gives an input of NaN, and first activations of 0) must not
+// reach the sums.  The fast path forms 0 x value everywhere, the same sum while all values are finite; a tile
+// that holds another value takes the slow one.
 constexpr int kWgT = 256, kWgC = 32, kWgX = 64;
 
 __host__ __device__ constexpr int odd4(int n) { return ((n + 3) / 4 | 1) * 4; }   // >= n, 4 x odd
@@ -347,6 +351,11 @@ struct WgTile {
     static constexpr int GCH = odd4(WR * GW), ICH = odd4(IR * IW);   // channel strides
     static constexpr size_t SMEM = (size_t)kWgC * (GCH + ICH) * sizeof(float);
 };
+
+// chk + 0 v: NaN if chk or a value of v is not finite, else chk
+__device__ __forceinline__ float not_finite(float4 v, float chk) {
+    return fmaf(v.w, 0.f, fmaf(v.z, 0.f, fmaf(v.y, 0.f, fmaf(v.x, 0.f, chk))));
+}
 
 // VEC: rows of whole groups of four (16-byte loads).
 template <int STRIDE, int GW, bool VEC>
@@ -412,23 +421,54 @@ __global__ void __launch_bounds__(kWgT, 2) k_conv_wgrad(const float* __restrict_
             ve[k] = ok ? __ldg(in + (((size_t)b * cin + ci0 + c) * hin + iy) * hin + ix) : 0.f;
         }
         __syncthreads();   // the previous tile has been read
+        float chk = 0.f;   // NaN once a staged value is not finite
 #pragma unroll
         for (int k = 0; k < PG; ++k) {
             const int e = threadIdx.x + k * kWgT, x = e % (GW / 4) * 4, y = e / (GW / 4) % WR, c = e / (GW / 4 * WR);
             if (e < NG) *reinterpret_cast<float4*>(gs + c * GCH + y * GW + x) = vg[k];
+            chk = not_finite(vg[k], chk);
         }
 #pragma unroll
         for (int k = 0; k < PI; ++k) {
             constexpr int Q = GW * STRIDE / 4;
             const int e = threadIdx.x + k * kWgT, x = e % Q * 4, y = e / Q % IR, c = e / (Q * IR);
             if (e < NI) *reinterpret_cast<float4*>(is + c * ICH + y * IW + 4 + x) = vi[k];
+            chk = not_finite(vi[k], chk);
         }
 #pragma unroll
         for (int k = 0; k < PE; ++k) {
             const int e = threadIdx.x + k * kWgT, y = e / 2 % IR, c = e / (2 * IR);
             if (e < NE && !(STRIDE == 2 && (e & 1))) is[c * ICH + y * IW + (e & 1 ? 4 + GW * STRIDE : 3)] = ve[k];
+            chk = fmaf(ve[k], 0.f, chk);
         }
-        __syncthreads();
+        if (__syncthreads_or(!(chk == 0.f))) {
+#pragma unroll 1
+            for (int q = 0; q < WR * GW; ++q) {
+                const int y = q / GW, x = q - y * GW;
+                const float g[2] = {gs[to * GCH + q], gs[(to + 16) * GCH + q]};
+                sb[0] += g[0];
+                sb[1] += g[1];
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) {
+                    const int iy = (y0 + y) * STRIDE + ky - 1;
+                    if (iy < 0 || iy >= hin) continue;
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) {
+                        const int ix = (xs + x) * STRIDE + kx - 1;
+                        if (ix < 0 || ix >= hin) continue;
+                        const int at = (y * STRIDE + ky) * IW + x * STRIDE + kx + 3;
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const float v = is[(tc + 16 * j) * ICH + at];
+#pragma unroll
+                            for (int i = 0; i < 2; ++i)
+                                if (g[i] != 0.f) acc[i][j][ky * 3 + kx] = fmaf(g[i], v, acc[i][j][ky * 3 + kx]);
+                        }
+                    }
+                }
+            }
+            continue;
+        }
 #pragma unroll 1
         for (int y = 0; y < WR; ++y) {
             const float* gp = gs + to * GCH + y * GW;
@@ -489,7 +529,8 @@ __global__ void __launch_bounds__(kWgT, 2) k_conv_wgrad(const float* __restrict_
 }
 
 // The same for the first layer (one input channel, stride 1): two output channels per warp, 16 per block, its
-// lanes over groups of four columns of a tile of 16 rows.  Bound by reading gout once.
+// lanes over groups of four columns of a tile of 16 rows.  Bound by reading gout once.  Which products count: as
+// above, the slow path for a group of columns whose gradients or a tile whose inputs are not all finite.
 constexpr int kW1Rows = 16, kW1C = 16;
 __global__ void __launch_bounds__(kWgT) k_conv_wgrad1(const float* __restrict__ gout, const float* __restrict__ in,
                                                       int B, int cout, int h, float* __restrict__ part) {
@@ -510,12 +551,15 @@ __global__ void __launch_bounds__(kWgT) k_conv_wgrad1(const float* __restrict__ 
         const int b = (int)(u / tiles), t = (int)(u - (long long)b * tiles);
         const int y0 = t / tiles_x * kW1Rows, xs = t % tiles_x * gw;
         __syncthreads();
+        float chk = 0.f;   // NaN once an input is not finite
         for (int i = threadIdx.x; i < (kW1Rows + 2) * iw; i += kWgT) {
             const int y = i / iw, x = i - y * iw;
             const int iy = y0 + y - 1, ix = xs + x - 1;
-            is[i] = iy >= 0 && iy < h && ix >= 0 && ix < h ? __ldg(in + ((size_t)b * h + iy) * h + ix) : 0.f;
+            const float v = iy >= 0 && iy < h && ix >= 0 && ix < h ? __ldg(in + ((size_t)b * h + iy) * h + ix) : 0.f;
+            is[i] = v;
+            chk = fmaf(v, 0.f, chk);
         }
-        __syncthreads();
+        const bool odd = __syncthreads_or(!(chk == 0.f));
         const int rows = min(kW1Rows, h - y0);
 #pragma unroll 2
         for (int e = lane; e < rows * q4; e += 32) {
@@ -540,6 +584,24 @@ __global__ void __launch_bounds__(kWgT) k_conv_wgrad1(const float* __restrict__ 
                 const float4 w = *reinterpret_cast<const float4*>(row);
                 const float2 w2 = *reinterpret_cast<const float2*>(row + 4);
                 v[ky][0] = w.x; v[ky][1] = w.y; v[ky][2] = w.z; v[ky][3] = w.w; v[ky][4] = w2.x; v[ky][5] = w2.y;
+            }
+            float gchk = 0.f;
+#pragma unroll
+            for (int c = 0; c < CW; ++c) gchk = not_finite(make_float4(g[c][0], g[c][1], g[c][2], g[c][3]), gchk);
+            if (odd || !(gchk == 0.f)) {
+#pragma unroll
+                for (int c = 0; c < CW; ++c)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+#pragma unroll
+                        for (int k = 0; k < 9; ++k) {
+                            const int iy = y0 + y + k / 3 - 1, ix = xs + x0 + x + k % 3 - 1;
+                            if (g[c][x] != 0.f && iy >= 0 && iy < h && ix >= 0 && ix < h)
+                                acc[c][k] = fmaf(g[c][x], v[k / 3][x + k % 3], acc[c][k]);
+                        }
+                        acc[c][9] += g[c][x];
+                    }
+                continue;
             }
 #pragma unroll
             for (int c = 0; c < CW; ++c)
