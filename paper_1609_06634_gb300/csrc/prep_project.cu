@@ -275,12 +275,14 @@ __device__ __forceinline__ float store_half_spectrum(const float2* F, const floa
     return amax;
 }
 
-// k != 0 of the half spectrum stands for w_kx of the full one's coefficients: 1 on the kx = 0 and kx = N/2
-// columns, 2 elsewhere (their Hermitian partners); 0 at DC.
+// w_kx |v|^2 of coefficient o of the half spectrum, w_kx = 1 on the kx = 0 and kx = N/2 columns and 2 elsewhere
+// (their Hermitian partners).  DC is left out, not multiplied by 0: it alone may be infinite (the sum of an
+// image whose other coefficients are within range).
 template <int N>
-__device__ __forceinline__ double half_weight(int o) {
+__device__ __forceinline__ double half_energy(int o, float2 v) {
     const int kx = o % Dft<N>::H;
-    return o == 0 ? 0.0 : (kx == 0 || kx == N / 2) ? 1.0 : 2.0;
+    const double m = (double)v.x * v.x + (double)v.y * v.y;
+    return o == 0 ? 0.0 : (kx == 0 || kx == N / 2) ? m : 2.0 * m;
 }
 
 // VEC: the images start on a 16-byte boundary (a caller's tensor may be a view that does not).
@@ -313,10 +315,7 @@ __global__ void __launch_bounds__(Dft<N>::T) k_prepare_images(const float* __res
     __syncthreads();
     c2c_columns_inplace<N>(sm);
     double e = 0.0, dummy = 0.0;
-    for (int o = threadIdx.x; o < N * H; o += T) {
-        const float2 v = sm.F[o];
-        e += half_weight<N>(o) * ((double)v.x * v.x + (double)v.y * v.y);
-    }
+    for (int o = threadIdx.x; o < N * H; o += T) e += half_energy<N>(o, sm.F[o]);
     block_sum2<T>(e, dummy, sm.red);
     const bool bad = !(A > 0.0) || !(e > 0.0);
     const float scale = bad ? 0.f : (float)(1.0 / sqrt(e));
@@ -597,10 +596,7 @@ constexpr double kSmall = 1e-12;
 template <int N>
 __device__ __forceinline__ double psf_energy64(const float2* F, const float* __restrict__ T) {
     double e = 0.0;
-    for (int o = threadIdx.x; o < N * Dft<N>::H; o += Dft<N>::T) {
-        const float2 v = c_scale(F[o], __ldg(T + o));
-        e += half_weight<N>(o) * ((double)v.x * v.x + (double)v.y * v.y);
-    }
+    for (int o = threadIdx.x; o < N * Dft<N>::H; o += Dft<N>::T) e += half_energy<N>(o, c_scale(F[o], __ldg(T + o)));
     return e;
 }
 
@@ -644,7 +640,8 @@ __global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(con
                     const int o = threadIdx.x + i * TH;
                     if (o < N * H) {
                         const int kx = o % H;
-                        const float2 v = c_scale(c_scale(sm.F[o], __ldg(Tc + o)), o == 0 ? 0.f : sc);
+                        float2 v = c_scale(c_scale(sm.F[o], __ldg(Tc + o)), sc);
+                        if (o == 0) v = make_float2(0.f, 0.f);   // DC (see half_energy)
                         const float w = kx == 0 || kx == N / 2 ? 1.f : 2.f;
                         add_square(hi, lo, v.x, w);
                         add_square(hi, lo, v.y, w);

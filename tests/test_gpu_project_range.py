@@ -1,0 +1,55 @@
+"""GPU: projections at the ends of the number range: weights whose sum overflows, atoms that are points,
+weights that are not finite."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def env():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1609_06634_gb300 as bioem
+    from paper_1609_06634_gb300 import build
+    build.build()
+    return bioem, bioem.Context(0)
+
+
+def _dev(x):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(x)).to("cuda:0")
+
+
+def _ball(rng, n, radius):
+    g = rng.standard_normal((n, 3))
+    g *= (radius * rng.random(n) ** (1 / 3) / np.linalg.norm(g, axis=1))[:, None]
+    return np.concatenate([g, np.ones((n, 1))], 1).astype(np.float32)
+
+
+@pytest.mark.parametrize("npix", [32, 96, 128, 192])
+def test_weights_whose_sum_overflows(env, npix):
+    """Weights of 2^116: their sum, the DC coefficient alone, exceeds the FP32 range, so ln L changes by ln of the
+    scale.  1e-3, the FP32 form's bound: the spectra's norms are near 2^127, and the FP32 factor that takes
+    them to 1 has lost bits to underflow."""
+    bioem, ctx = env
+    rng = np.random.default_rng(npix)
+    pixel, n, bits = 128.0 / npix, 5000, 116
+    assert n * 2.0 ** bits > float(np.finfo(np.float32).max)
+    atoms = _ball(rng, n, 40.0)
+    quats = rng.standard_normal((3, 4)).astype(np.float32)
+    ctfs = [(1.0e4, 0.1, 0.0, 300.0), (2.0e4, 0.2, 30.0, 300.0)]
+    im = bioem.prepare_images(ctx, _dev(rng.standard_normal((2, npix, npix)).astype(np.float32)), pixel)
+    out = []
+    for scale in (1.0, 2.0 ** bits):
+        a = atoms.copy()
+        a[:, 3] *= np.float32(scale)
+        ps = bioem.project_model(ctx, _dev(a), 1.5, _dev(quats), ctfs, npix, pixel)
+        out.append([x.cpu().numpy() for x in bioem.score_pairs(ctx, im, ps, 3)])
+        assert ctx.status() == 0
+    for one, two in zip(*out):
+        assert np.isfinite(one).all()
+        np.testing.assert_allclose(two, one - bits * np.log(2.0), rtol=0, atol=1e-3)
