@@ -347,6 +347,14 @@ __device__ __forceinline__ float pixel_mass(float t0, bool neg0, float t1, bool 
 // integral is exactly zero, with room for the rounding of the window's own bounds.
 constexpr float kErfcZero = 11.f, kWindow = 10.5f;
 
+// k_project's reach: kWindow, but one pixel (D) more for atoms that are points beside a pixel.  The bounds of a
+// window are rounded by up to 5e-5 pixels (N 2^-22), for which kWindow leaves 0.4 / D.  (Formed in the kernel,
+// in a register or in shared memory, it cost 3 % of 1024 maps at 128 px.)
+float window_reach(double sigma, double pixel) {
+    const double d = pixel / (sigma * 1.4142135623730951);
+    return d > 4096.0 ? (float)(kWindow + d) : kWindow;
+}
+
 // One orientation per block.  The image is cut into tiles of TR x TC pixels, LR x LC per lane (4 x 8 lanes);
 // a warp owns TPW tiles, one in each of TPW bands of rows and in different columns, so that dense and
 // empty parts of the projection even out.  Atoms are processed in chunks of 32 in order: a warp tabulates
@@ -391,7 +399,7 @@ __device__ __forceinline__ void load_vec(const float* src, float (&v)[V]) {
 template <int N>
 __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1) k_project(const float4* __restrict__ atoms, int n_atoms,
                                                            const float4* __restrict__ quats, double sigma,
-                                                           double pixel, float* __restrict__ out) {
+                                                           double pixel, float reach, float* __restrict__ out) {
     using C = ProjCfg<N>;
     constexpr int LR = C::LR, LC = C::LC, CH = C::CH, NW = C::NW;
     extern __shared__ __align__(16) float tab[];   // [2][CH][2][N]: gx, gy (gy carries the atom's weight)
@@ -432,10 +440,10 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
             ax.h = (float)x; ax.l = (float)(x - (double)ax.h);
             ay.h = (float)y; ay.l = (float)(y - (double)ay.h);
             w = p.w;
-            // boundary j has |u_j| < kWindow for (A - kWindow) / D < j < (A + kWindow) / D; pixel j has boundaries j, j + 1
+            // boundary j has |u_j| < reach for (A - reach) / D < j < (A + reach) / D; pixel j has boundaries j, j + 1
             auto window = [&](Axis& v) {
-                v.lo = max(0, (int)ceilf(fminf(fmaxf((v.h - kWindow) * inv_d, -1.e6f), 1.e6f)) - 1);
-                v.hi = min(N - 1, (int)floorf(fminf(fmaxf((v.h + kWindow) * inv_d, -1.e6f), 1.e6f)));
+                v.lo = max(0, (int)ceilf(fminf(fmaxf((v.h - reach) * inv_d, -1.e6f), 1.e6f)) - 1);
+                v.hi = min(N - 1, (int)floorf(fminf(fmaxf((v.h + reach) * inv_d, -1.e6f), 1.e6f)));
             };
             window(ax);
             window(ay);
@@ -1050,7 +1058,7 @@ int launch_project_n(bioem_ctx* ctx, const float* d_atoms, int n_atoms, double s
         bioem_launch_begin(ctx, KID_PROJECT);
         k_project<N><<<nb, ProjCfg<N>::T, ProjCfg<N>::SMEM, ctx->stream>>>(reinterpret_cast<const float4*>(d_atoms), n_atoms,
                                                         reinterpret_cast<const float4*>(d_quats) + q0, sigma_A,
-                                                        ps->pixel_A, d_I0);
+                                                        ps->pixel_A, window_reach(sigma_A, ps->pixel_A), d_I0);
         bioem_launch_end(ctx, KID_PROJECT);
         rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_project");
         if (rc) break;
@@ -1085,7 +1093,8 @@ int launch_synthetic_n(bioem_ctx* ctx, const float* d_atoms, int n_atoms, double
     }
     bioem_launch_begin(ctx, KID_PROJECT);
     k_project<N><<<n, ProjCfg<N>::T, ProjCfg<N>::SMEM, ctx->stream>>>(reinterpret_cast<const float4*>(d_atoms), n_atoms,
-                                                   reinterpret_cast<const float4*>(d_quats), sigma_A, pixel_A, d_I0);
+                                                   reinterpret_cast<const float4*>(d_quats), sigma_A, pixel_A,
+                                                   window_reach(sigma_A, pixel_A), d_I0);
     bioem_launch_end(ctx, KID_PROJECT);
     rc = bioem_check_cuda(ctx, cudaGetLastError(), "k_project");
     if (!rc && set_smem<N>((const void*)k_psf_real<N>, Fft<N>::SMEM)) rc = bioem_set_error(ctx, BIOEM_ERR_CUDA, "smem attribute");

@@ -53,3 +53,24 @@ def test_weights_whose_sum_overflows(env, npix):
     for one, two in zip(*out):
         assert np.isfinite(one).all()
         np.testing.assert_allclose(two, one - bits * np.log(2.0), rtol=0, atol=1e-3)
+
+
+IDENTITY = np.array([[1, 0, 0, 0]], dtype=np.float32)
+
+
+@pytest.mark.parametrize("npix", [32, 64, 96, 128, 192])
+@pytest.mark.parametrize("sigma_px", [1e-3, 1e-4, 1e-6, 1e-7, 1e-8])
+def test_atoms_that_are_points(env, npix, sigma_px):
+    """Atoms on pixel boundaries and up to 2^-8 pixels beside them, narrower than the FP32 spacing of their
+    positions in units of sigma.  The bound of the maps of any window: 2e-5 of the largest value."""
+    bioem, ctx = env
+    rng = np.random.default_rng(npix)
+    atoms = np.zeros((300, 4), dtype=np.float32)
+    atoms[:, :2] = rng.integers(2, npix - 2, (300, 2)) - npix / 2 - 0.5
+    atoms[150:, :2] += rng.choice([-1, 1], (150, 2)) * 2.0 ** -rng.integers(8, 18, (150, 1))
+    atoms[:, 3] = rng.uniform(0.5, 1.5, 300)
+    ctf = (0.0, 1.0, 0.0, 300.0)
+    got = bioem.synthetic_maps(ctx, _dev(atoms), sigma_px, _dev(IDENTITY), [ctf], npix, 1.0).cpu().numpy()[0]
+    want = oracle.apply_psf(oracle.project(atoms, IDENTITY[0], sigma_px, npix, 1.0), ctf, 1.0)
+    assert ctx.status() == 0
+    np.testing.assert_allclose(got, want, rtol=0, atol=2e-5 * np.abs(want).max())
