@@ -447,6 +447,13 @@ __global__ void __launch_bounds__(ProjCfg<N>::T, N <= 64 ? 4 : N <= 128 ? 2 : 1)
             };
             window(ax);
             window(ay);
+            if (!(fabsf(w) < INFINITY)) {
+                // inf or NaN times the zeros beside the window is NaN: the whole image for an atom whose rows
+                // come near it, so that the projection is found degenerate
+                const bool near_rows = floorf((ay.h - kErfcZero) * inv_d) - 2.f < N && ceilf((ay.h + kErfcZero) * inv_d) + 1.f >= 0.f;
+                ax.lo = ay.lo = 0;
+                ax.hi = ay.hi = near_rows ? N - 1 : -1;
+            }
         }
         pos[buf][lane][0] = ax;
         pos[buf][lane][1] = ay;

@@ -74,3 +74,22 @@ def test_atoms_that_are_points(env, npix, sigma_px):
     want = oracle.apply_psf(oracle.project(atoms, IDENTITY[0], sigma_px, npix, 1.0), ctf, 1.0)
     assert ctx.status() == 0
     np.testing.assert_allclose(got, want, rtol=0, atol=2e-5 * np.abs(want).max())
+
+
+@pytest.mark.parametrize("npix", [32, 96, 128, 192])
+@pytest.mark.parametrize("weight", [np.nan, np.inf, -np.inf])
+def test_weights_that_are_not_finite(env, npix, weight):
+    """An atom whose weight is not finite makes the projection degenerate (NUMERIC) and the map undefined
+    wherever it lies beside the image's columns: its weight meets the zeros there.  Far above or below the
+    image, where no row comes near it, it has no part in either."""
+    bioem, ctx = env
+    rng = np.random.default_rng(npix)
+    for x, y, part in ((0, 0, True), (5 * npix, 0, True), (0.5 * npix + 16.2, 3, True), (2, 0.5 * npix + 11.2, True),
+                       (0, 5 * npix, False), (-5 * npix, 5 * npix, False)):
+        atoms = rng.uniform(-8, 8, (40, 4)).astype(np.float32)
+        atoms[:, 3] = 1.0
+        atoms[7] = (x, y, 0.0, weight)
+        bioem.project_model(ctx, _dev(atoms), 1.0, _dev(IDENTITY), [(1.0e4, 0.1, 0.0, 300.0)], npix, 1.0)
+        assert ctx.status() == (bioem.ERR_NUMERIC if part else 0), (x, y)
+        got = bioem.synthetic_maps(ctx, _dev(atoms), 1.0, _dev(IDENTITY), [(1.0e4, 0.1, 0.0, 300.0)], npix, 1.0).cpu().numpy()
+        assert np.isfinite(got).any() != part and np.isfinite(got).all() != part, (x, y)
