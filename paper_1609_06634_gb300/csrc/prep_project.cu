@@ -816,8 +816,8 @@ __global__ void __launch_bounds__(Fft<N>::T, Fft<N>::MINB) k_psf_real(const floa
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = threadIdx.x; i < N; i += TH) tw[i] = g_tw[i];
     __syncthreads();
-    // rows: C = row 2p + i row 2p + 1 transformed, then taken apart into the halves 2 F (the factor
-    // is taken back at the end)
+    // rows: C = row 2p + i row 2p + 1 transformed, then taken apart into the halves F (halved before the sums,
+    // which would double the largest sum of an image that is within the FP32 range)
     const float* img = img0 + map * N * N;
     const int j = lane & 7, kA = j, kB = j ? 16 - j : 8;   // a lane's two residues k1, partners under k -> N - k
     for (int g = warp; g < N / 8; g += NW) {
@@ -844,8 +844,8 @@ __global__ void __launch_bounds__(Fft<N>::T, Fft<N>::MINB) k_psf_real(const floa
         dft<R, false>(v);
         __syncwarp();
         auto apart = [&](int k, float2 c, float2 d) {   // d = C(N - k)
-            buf[k] = make_float2(c.x + d.x, c.y - d.y);
-            buf[P + k] = make_float2(c.y + d.y, d.x - c.x);
+            buf[k] = make_float2(fmaf(0.5f, c.x, 0.5f * d.x), fmaf(0.5f, c.y, -0.5f * d.y));
+            buf[P + k] = make_float2(fmaf(0.5f, c.y, 0.5f * d.y), fmaf(0.5f, d.x, -0.5f * c.x));
         };
 #pragma unroll
         for (int k2 = 0; k2 < R / 2; ++k2) {
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(Fft<N>::T, Fft<N>::MINB) k_psf_real(const floa
     __syncthreads();
     // rows: C(k) = G_2p(k) + i G_2p+1(k) of the Hermitian rows G (the imaginary parts at k = 0 and N/2 do not
     // count), transformed back: its real and imaginary parts are the two rows of the map
-    constexpr float inv = 0.5f / ((float)N * N);
+    constexpr float inv = 1.f / ((float)N * N);
     float* o = out + map * N * N;
     for (int g = warp; g < N / 8; g += NW) {
         float2* const buf = F + (size_t)2 * (4 * g + (lane >> 3)) * P;

@@ -93,3 +93,17 @@ def test_weights_that_are_not_finite(env, npix, weight):
         assert ctx.status() == (bioem.ERR_NUMERIC if part else 0), (x, y)
         got = bioem.synthetic_maps(ctx, _dev(atoms), 1.0, _dev(IDENTITY), [(1.0e4, 0.1, 0.0, 300.0)], npix, 1.0).cpu().numpy()
         assert np.isfinite(got).any() != part and np.isfinite(got).all() != part, (x, y)
+
+
+@pytest.mark.parametrize("npix", [32, 64, 96, 128, 192])
+@pytest.mark.parametrize("top", [1e37, 2e38, 3e38])
+def test_maps_up_to_the_largest_numbers(env, npix, top):
+    """N^2 times the largest value of the map (what the unscaled inverse transform reaches) up to 3e38.  The
+    bound of the maps of any window: 2e-5 of the largest value."""
+    bioem, ctx = env
+    atoms = np.array([[1.3, -2.1, 0.0, 1.0]], dtype=np.float32)
+    want = -oracle.project(atoms, IDENTITY[0], 1.5, npix, 1.0)   # defocus 0, amplitude contrast 1: CTF = -1
+    atoms[0, 3] = top / (npix * npix * np.abs(want).max())
+    got = bioem.synthetic_maps(ctx, _dev(atoms), 1.5, _dev(IDENTITY), [(0.0, 1.0, 0.0, 300.0)], npix, 1.0).cpu().numpy()[0]
+    want *= float(atoms[0, 3])
+    np.testing.assert_allclose(got.astype(np.float64), want, rtol=0, atol=2e-5 * np.abs(want).max())
