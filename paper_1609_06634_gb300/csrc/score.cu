@@ -1172,7 +1172,9 @@ int run_waves(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, i
         ctx->rec_bytes = rec_need;
     }
     const int n_parts = pairs_mode ? 1 : reduce_parts(ctx, n_img, wave, nctf);
-    const size_t acc_need = reduce_bytes(n_img, n_parts);
+    // for the most parts that n_img images are ever cut into: a call captured in a graph must find the
+    // accumulators in place, whatever number of sets the earlier calls of as many images had
+    const size_t acc_need = sizeof(Acc) * ((size_t)n_img + 4 * (size_t)ctx->num_sms);
     if (!pairs_mode && ctx->acc_bytes < acc_need) {
         if (ctx->d_acc) cudaFreeAsync(ctx->d_acc, ctx->stream);
         ctx->d_acc = nullptr;
