@@ -595,6 +595,9 @@ __device__ __forceinline__ void score_tail(const Sm<C>& sm, const Job& job, int 
             acc = merge(acc, o, c1);   // merge orders its operands, so both lanes agree
         }
         const int p = p0 + jl;
+        // spectra of NaN leave no piece with a value, and which piece wins depends on the lanes: an empty record
+        // (ln L = -inf), as 32 lanes with fewer pieces gave
+        if (LPP < 32 && !(acc.t < INFINITY)) acc = Part{INFINITY, 0.f, 0x7fffffff};
         if (l == 0 && e < C::GPB * LPP && p < hi) {
             job.rec_t[p] = acc.t;
             job.rec_s[p] = acc.s;
