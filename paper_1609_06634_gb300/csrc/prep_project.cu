@@ -587,25 +587,35 @@ __global__ void k_ctf_table(const double* __restrict__ coef, int nctf, int N, do
     }
 }
 
-// (hi, lo) += w x^2 in FP32 pairs, w a power of two: the square and the sum with their rounding errors
-// (error-free transforms of Dekker and Knuth), the errors summed in lo.
-__device__ __forceinline__ void add_square(float& hi, float& lo, float x, float w) {
-    const float p0 = x * x, e = fmaf(x, x, -p0) * w, p = p0 * w;
-    const float s = hi + p, b = s - hi;
-    lo += (hi - (s - b)) + (p - b) + e;
-    hi = s;
+// a + b and its rounding error (Knuth)
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float s = a + b, t = s - a;
+    err = (a - (s - t)) + (b - t);
+    return s;
+}
+
+// hi + mid + lo += w x^2, w a power of two: the square and the sums with their rounding errors (error-free
+// transforms of Dekker and Knuth), to about 2^-66 of the sum for a spectrum's share of one thread.
+__device__ __forceinline__ void add_square(float& hi, float& mid, float& lo, float x, float w) {
+    const float p = x * x, e = fmaf(x, x, -p);
+    float e1, e2, e3;
+    hi = two_sum(hi, p * w, e1);
+    mid = two_sum(mid, e1, e2);
+    mid = two_sum(mid, e * w, e3);
+    lo += e2 + e3;
 }
 
 // One orientation per block: transform I0, and for every PSF c the energy B_c = sum_{k != 0} w_kx |F T_c|^2 (of
 // the FP32 products that are stored) and the normalised product.
 // GB300's float64 rate is 1/70 of its FP32 rate, and squaring every product in float64 (two conversions
-// and three operations) took most of the kernel's 1.5 us per orientation (128 px, 8 PSFs).  Each thread now
-// sums its squares in runs of kRun as FP32 pairs (relative error about 2^-46 per run, independent between
-// the ~800 runs of a spectrum, so 1e-16 of B) and adds the runs in float64.  The products are scaled by a
-// power of two so that the largest |F| is near 1; a B so small against it that squares may have lost bits
-// to underflow (below kSmall) is summed again in float64 throughout.
+// and three operations) took most of the kernel's 1.5 us per orientation (128 px, 8 PSFs). Each thread sums
+// its squares in FP32 triples, exact beyond float64's own rounding, and the threads' sums are added in float64 by
+// pairs: error of B 1.0e-16 (rms over models, PSFs and sizes), as with float64 throughout. (In FP32 pairs, restarted
+// every 11 coefficients, 1e-15: the energy lies in few coefficients, so the runs' errors do not average.)
+// The products are scaled by a power of two so that the largest |F| is near 1; a B so small against it that
+// squares may have lost bits to underflow (below kSmall) is summed again in float64 throughout.
 constexpr int kPsfChunk = 16;   // PSFs whose energies are reduced together
-constexpr int kRun = 11;
+constexpr int kUnroll = 11;
 constexpr double kSmall = 1e-12;
 
 template <int N>
@@ -625,6 +635,7 @@ __global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(con
     constexpr int H = Dft<N>::H, TH = Dft<N>::T, PER = Dft<N>::PER;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ double part[kPsfChunk][TH / 32];
+    __shared__ float scale[kPsfChunk];   // 1 / sqrt(B); -1 where B is to be summed in float64
     const DftSm<N> sm(smem);
     const int q = blockIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -646,54 +657,61 @@ __global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(con
         const int nc = min(kPsfChunk, nctf - c0);
         for (int c = 0; c < nc; ++c) {
             const float* Tc = T + (size_t)(c0 + c) * N * H;
-            double e = 0.0;
+            float hi = 0.f, mid = 0.f, lo = 0.f;
+#pragma unroll 1
+            for (int i0 = 0; i0 < PER; i0 += kUnroll) {
 #pragma unroll
-            for (int i0 = 0; i0 < PER; i0 += kRun) {
-                float hi = 0.f, lo = 0.f;
-#pragma unroll
-                for (int i = i0; i < i0 + kRun && i < PER; ++i) {
-                    const int o = threadIdx.x + i * TH;
+                for (int i = 0; i < kUnroll; ++i) {
+                    const int o = threadIdx.x + (i0 + i) * TH;
                     if (o < N * H) {
                         const int kx = o % H;
                         float2 v = c_scale(c_scale(sm.F[o], __ldg(Tc + o)), sc);
                         if (o == 0) v = make_float2(0.f, 0.f);   // DC (see half_energy)
                         const float w = kx == 0 || kx == N / 2 ? 1.f : 2.f;
-                        add_square(hi, lo, v.x, w);
-                        add_square(hi, lo, v.y, w);
+                        add_square(hi, mid, lo, v.x, w);
+                        add_square(hi, mid, lo, v.y, w);
                     }
                 }
-                e += (double)hi + (double)lo;
             }
+            double e = (double)hi + ((double)mid + (double)lo);
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
             if (lane == 0) part[c][warp] = e;
         }
         __syncthreads();
+        // the warps' sums, the scale and ln B of a PSF by one lane (float64 by every thread takes longer than the sums)
+        if (threadIdx.x < nc) {
+            const int c = threadIdx.x;
+            double t[TH / 32];
+#pragma unroll
+            for (int w = 0; w < TH / 32; ++w) t[w] = part[c][w];
+#pragma unroll
+            for (int n = TH / 64; n > 0; n /= 2)
+#pragma unroll
+                for (int w = 0; w < n; ++w) t[w] = t[2 * w] + t[2 * w + 1];
+            const bool sure = t[0] > kSmall && t[0] < INFINITY;
+            const double B = ldexp(t[0], 2 * ex);
+            scale[c] = sure ? (float)(1.0 / sqrt(B)) : -1.f;
+            if (sure) kB[(size_t)q * nctf + c0 + c] = -0.5 * log(B);
+        }
+        __syncthreads();
         for (int c = 0; c < nc; ++c) {
             const float* Tc = T + (size_t)(c0 + c) * N * H;
-            double B = part[c][0];
-            for (int w = 1; w < TH / 32; ++w) B += part[c][w];
-            if (B > kSmall && B < INFINITY) {
-                B = ldexp(B, 2 * ex);
-            } else {   // uniform over the block
-                double dummy = 0.0;
-                B = psf_energy64<N>(sm.F, Tc);
-                block_sum2<TH>(B, dummy, sm.red);
-            }
-            const bool bad = !(B > 0.0);   // B = n C_cc - C_c^2 (Plancherel)
             const size_t p = (size_t)q * nctf + c0 + c;
-            const float mx = block_max<TH>(store_half_spectrum<N>(sm.F, Tc, bad ? 0.f : (float)(1.0 / sqrt(B)),
-                                                                  spec + p * N * H),
-                                           reinterpret_cast<float*>(sm.red));
-            if (threadIdx.x == 0) {
-                amax[p] = mx;
-                if (bad) {
-                    atomicOr(status, BIOEM_DEV_NUMERIC);
-                    kB[p] = -INFINITY;
-                } else {
-                    kB[p] = -0.5 * log(B);
+            float sB = scale[c];
+            if (sB < 0.f) {   // uniform over the block
+                double B = psf_energy64<N>(sm.F, Tc), dummy = 0.0;
+                block_sum2<TH>(B, dummy, sm.red);
+                const bool bad = !(B > 0.0);   // B = n C_cc - C_c^2 (Plancherel)
+                sB = bad ? 0.f : (float)(1.0 / sqrt(B));
+                if (threadIdx.x == 0) {
+                    if (bad) atomicOr(status, BIOEM_DEV_NUMERIC);
+                    kB[p] = bad ? -INFINITY : -0.5 * log(B);
                 }
             }
+            const float mx = block_max<TH>(store_half_spectrum<N>(sm.F, Tc, sB, spec + p * N * H),
+                                           reinterpret_cast<float*>(sm.red));
+            if (threadIdx.x == 0) amax[p] = mx;
         }
     }
 }
