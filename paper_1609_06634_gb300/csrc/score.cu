@@ -838,15 +838,15 @@ __device__ double g_exp2[1 << kExpBits];   // uploaded with the twiddle tables
 
 // exp(x) for x in [-100, 0]: x = (256 q + j) ln2 / 256 + r, |r| <= ln2 / 512, exp(x) = 2^q 2^(j/256) e^r with the
 // Taylor series of e^r to r^4 (truncation below 4e-17), the table-driven scheme of Tang (ACM TOMS 15,
-// 1989).  ln2 / 256 as one float64 is 9e-20 off per step of 1 / 256: 5e-16 of the result at x = -16, where the
-// term is 1e-7 of the sum.  Eight float64 operations: the reductions below are bound by the float64 pipe (1/70
-// of the FP32 rate), so what can be an integer operation (comparisons, scaling) is one.
+// 1989), ln2 / 256 in two float64 numbers (with one the error grows with |x|, to 1.4e-15 at -36).  Within 1.1
+// ulp, as the library's exponential is within 1.  Nine float64 operations: the reductions below are bound by the
+// float64 pipe (1/70 of the FP32 rate), so what can be an integer operation (comparisons, scaling) is one.
 __device__ __forceinline__ double exp_neg(double x, const double* tab) {
     const double big = 6755399441055744.0;   // 1.5 * 2^52: adding it rounds to an integer in the low word
     const double kd = fma(x, 369.32993046757463, big);   // 256 / ln 2
     const int k = __double2loint(kd);
     const double n = kd - big;
-    const double r = fma(n, -0.0027076061740622863, x);   // ln 2 / 256
+    const double r = fma(n, -9.0587766165871077e-20, fma(n, -0.0027076061740622863, x));   // ln 2 / 256
     double p = fma(r, 1.0 / 24.0, 1.0 / 6.0);
     p = fma(r, p, 0.5);
     p = fma(r, p, 1.0);

@@ -52,3 +52,30 @@ extern "C" void sum_squares(const float* x, const float* w, int n, float* out) {
         exact = sum(Fraction(float(b)) * Fraction(float(a)) ** 2 for a, b in zip(x, w))
         got = sum(Fraction(float(v)) for v in out)
         assert abs(got - exact) <= exact / 2 ** 60
+
+
+def test_exponential_of_the_reductions(tmp_path):
+    """exp_neg over [-100, 0] against long double where that is wider, within 2.7e-16: half an ulp (2^-53) each of the
+    table's entry and of the last sum, and the series' truncation."""
+    if np.finfo(np.longdouble).nmant <= 52:
+        pytest.skip("no wider type")
+    lib = _library(str(tmp_path), '''
+static int __double2loint(double x) { int64_t b; memcpy(&b, &x, 8); return (int)(uint32_t)b; }
+static int __double2hiint(double x) { int64_t b; memcpy(&b, &x, 8); return (int)(b >> 32); }
+static double __hiloint2double(int h, int l) {
+    const int64_t b = (int64_t)((uint64_t)(uint32_t)h << 32 | (uint32_t)l); double x; memcpy(&x, &b, 8); return x;
+}
+static const int kExpBits = 8;
+''' + _function("score.cu", "exp_neg") + '''
+extern "C" void exps(const double* x, int n, double* y) {
+    double tab[256];
+    for (int j = 0; j < 256; ++j) tab[j] = exp2(j / 256.0);
+    for (int i = 0; i < n; ++i) y[i] = exp_neg(x[i], tab);
+}
+''')
+    rng = np.random.default_rng(4)
+    x = np.concatenate([-rng.uniform(0, 100, 200_000), -rng.uniform(0, 1, 50_000), [0.0, -100.0, -1e-300, -np.log(2.0)]])
+    y = np.empty_like(x)
+    lib.exps(x.ctypes.data_as(ctypes.c_void_p), len(x), y.ctypes.data_as(ctypes.c_void_p))
+    exact = np.exp(x.astype(np.longdouble))
+    assert float(np.abs((y - exact) / exact).max()) < 2.7e-16
