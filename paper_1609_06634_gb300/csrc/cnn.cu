@@ -991,6 +991,7 @@ __device__ void joint_log_norms(const float* q, int nq, const float* d, int nd, 
 // Bound by the sort's shared-memory passes: 0.5 log2(k)^2 of them, against one pass over all nq nd
 // scores for every bin picked before (k = 4096 of 18,432, 256 samples: 54.2 ms).
 constexpr int kTopT = 1024, kSelBits = 11;
+static_assert(kTopT == 32 * 32 && kT >= 32, "a warp scans the warps' counts");
 constexpr int kTopMaxK = 32768, kTopMaxBins = 65536;   // 6 bytes per sorted entry in shared memory; 16-bit bins
 
 // a before b: larger score first, then the lower bin
@@ -1099,19 +1100,30 @@ __global__ void __launch_bounds__(kTopT) k_topk_joint(const float* __restrict__ 
         }
     }
     __syncthreads();
-    if (split && t < 32) {   // equal scores at the threshold (shift = 0): the lowest bins
-        uint32_t at = s_taken;
+    if (split) {   // equal scores at the threshold (shift = 0): the lowest bins, kTopT at a time
+        uint32_t at = s_taken;   // rv is free since joint_log_norms: the warps' counts
+        uint32_t* count = reinterpret_cast<uint32_t*>(rv);
         const int total = nq * nd;
-        for (int j0 = 0; j0 < total && at < need; j0 += 32) {
-            const int j = j0 + lane;
+        for (int j0 = 0; j0 < total && at < need; j0 += kTopT) {   // uniform over the block
+            const int j = j0 + t;
             const bool tie = j < total && ord((q[j / nd] - lse) + dls[j % nd]) == prefix;
             const unsigned bal = __ballot_sync(0xffffffffu, tie);
-            const uint32_t my = at + __popc(bal & ((1u << lane) - 1u));
+            if (lane == 0) count[t >> 5] = __popc(bal);
+            __syncthreads();
+            uint32_t run = count[lane];   // kTopT / 32 = 32 warps
+            const uint32_t own = run;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, run, off);
+                if (lane >= off) run += v;
+            }
+            const uint32_t my = at + __shfl_sync(0xffffffffu, run - own, t >> 5) + __popc(bal & ((1u << lane) - 1u));
             if (tie && my < need) {
                 key[my] = prefix;
                 idx[my] = (uint16_t)j;
             }
-            at += __popc(bal);
+            at += __shfl_sync(0xffffffffu, run, 31);
+            __syncthreads();   // the counts have been read
         }
     }
     for (int i = need + t; i < n2; i += kTopT) { key[i] = 0u; idx[i] = 0xffffu; }   // after every score
