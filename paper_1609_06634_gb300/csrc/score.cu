@@ -915,9 +915,10 @@ __device__ __forceinline__ int lse_add4(Lse& a, const double (&m)[4], const floa
     return at;
 }
 
-__device__ __forceinline__ void exp_table(double* tab) {
-    for (int i = threadIdx.x; i < (1 << kExpBits); i += kRedThreads) tab[i] = g_exp2[i];
-}
+// The table, one entry per thread: loaded before a reduction's first terms, stored after them, so that a small
+// call waits once for both.
+static_assert((1 << kExpBits) == kRedThreads, "one entry of the table per thread");
+__device__ __forceinline__ double exp_entry() { return g_exp2[threadIdx.x]; }
 
 // The warp's sums and best set merged into every lane, lanes in a fixed order; bp = the lowest set of the maximum.
 __device__ __forceinline__ void warp_lse(Lse& a, int& bp, const double* tab) {
@@ -925,8 +926,10 @@ __device__ __forceinline__ void warp_lse(Lse& a, int& bp, const double* tab) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     const double mv = key_d(mx);
-    a.S = a.key != kKeyNone ? scaled_exp(a.S, a.M - mv, tab) : 0.0;
-    if (a.key != mx) bp = 0x7fffffff;
+    if (a.key != mx) {   // (exp(0) = 1; a small call has few lanes to scale)
+        a.S = a.key != kKeyNone ? scaled_exp(a.S, a.M - mv, tab) : 0.0;
+        bp = 0x7fffffff;
+    }
     a.M = mv;
     a.key = mx;
 #pragma unroll
@@ -981,10 +984,9 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_wave(
     const int w = blockIdx.x / n_parts, part = blockIdx.x - w * n_parts;
     const int q_all = wave_len / nctf, q_per = (q_all + n_parts - 1) / n_parts;
     const int q0 = min(part * q_per, q_all), q1 = min(q0 + q_per, q_all);
+    const double entry = exp_entry();
     const double ka = kA[w];
     const size_t base = (size_t)w * wave_len;
-    exp_table(tab);
-    __syncthreads();
     Lse a;
     int bp = 0x7fffffff;
     auto term = [&](int p, bool ok, double& m, float& sv) {
@@ -994,14 +996,24 @@ __global__ void __launch_bounds__(kRedThreads) k_reduce_wave(
     double m[4];
     float sv[4];
     if (!logP_orient) {
-        const int lo = q0 * nctf, hi = q1 * nctf;
-        for (int p = lo + threadIdx.x; p < hi; p += 4 * kRedThreads) {
+        const int hi = q1 * nctf;
+        int p = q0 * nctf + threadIdx.x;
+        auto terms = [&]() {
 #pragma unroll
             for (int i = 0; i < 4; ++i) term(p + i * kRedThreads, p + i * kRedThreads < hi, m[i], sv[i]);
+        };
+        terms();
+        tab[threadIdx.x] = entry;
+        __syncthreads();
+        while (p < hi) {
             const int at = lse_add4(a, m, sv, tab);
             if (at >= 0) bp = p + at * kRedThreads;
+            p += 4 * kRedThreads;
+            if (p < hi) terms();
         }
     } else {
+        tab[threadIdx.x] = entry;
+        __syncthreads();
         // an orientation per thread: its sum over the PSFs is an output and one term of the image's sum
         for (int ql = q0 + threadIdx.x; ql < q1; ql += kRedThreads) {
             Lse o;
@@ -1040,8 +1052,10 @@ __global__ void __launch_bounds__(kRedThreads) k_finalize(Acc* acc, const Acc* p
                                                           int* best_ctf, int* best_dx, int* best_dy, double* best_logL) {
     __shared__ double tab[1 << kExpBits];
     const int w = blockIdx.x * (kRedThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    exp_table(tab);
-    __syncthreads();
+    if (n_parts > 1) {
+        tab[threadIdx.x] = exp_entry();
+        __syncthreads();
+    }
     if (w >= n_img) return;
     Acc a{-INFINITY, 0.0, -INFINITY, 0x7fffffff, 0};
     if (lane < n_parts) a = (parts ? parts : acc)[(size_t)w * n_parts + lane];
@@ -1050,7 +1064,7 @@ __global__ void __launch_bounds__(kRedThreads) k_finalize(Acc* acc, const Acc* p
     Lse l;
     if (a.M > -INFINITY) { l.M = a.M; l.S = a.S; l.key = d_key(a.M); }
     int bp = a.bp;
-    warp_lse(l, bp, tab);
+    if (n_parts > 1) warp_lse(l, bp, tab);   // one part: lane 0 has it
     const int src = __ffs(__ballot_sync(0xffffffffu, bp != 0x7fffffff && a.bp == bp)) - 1;
     const int bd = __shfl_sync(0xffffffffu, a.bd, src < 0 ? 0 : src);
     if (lane != 0) return;
@@ -1681,27 +1695,34 @@ int seg_slots(bioem_ctx* ctx, const SegInstance& si, int* slots) {
 __global__ void __launch_bounds__(kRedThreads) k_reduce_multi(const SegDesc* __restrict__ segs, int n_segs,
                                                               float* __restrict__ out, int out_ld) {
     __shared__ double tab[1 << kExpBits];
+    const double entry = exp_entry();
     const long long row = blockIdx.x;
     const int g = find_seg(segs, n_segs, row, true);
     const SegDesc& sd = segs[g];
     const int w = (int)(row - sd.row_begin);
     const double ka = sd.kA[w];
     const double c1 = (double)sd.c1;
-    exp_table(tab);
-    __syncthreads();
     Lse a;
     int bp = 0x7fffffff;
     const size_t base = (size_t)w * sd.n_ps;
-    for (int p = threadIdx.x; p < sd.n_ps; p += 4 * kRedThreads) {
-        double m[4];
-        float sv[4];
+    double m[4];
+    float sv[4];
+    int p = threadIdx.x;
+    auto terms = [&]() {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int pi = p + i * kRedThreads;
             m[i] = pi < sd.n_ps ? ka + sd.kB[pi] + c1 * (double)sd.rec_t[base + pi] : -INFINITY;
             sv[i] = pi < sd.n_ps ? sd.rec_s[base + pi] : 0.f;
         }
+    };
+    terms();
+    tab[threadIdx.x] = entry;
+    __syncthreads();
+    while (p < sd.n_ps) {
         lse_add4(a, m, sv, tab);
+        p += 4 * kRedThreads;
+        if (p < sd.n_ps) terms();
     }
     block_lse(a, bp, tab);
     if (threadIdx.x == 0)
@@ -2178,21 +2199,28 @@ __global__ void __launch_bounds__(kRedThreads) k_fold_gathered(const int* __rest
                                                                double* __restrict__ acc, int first) {
     __shared__ double tab[1 << kExpBits];
     const int w = blockIdx.x;
+    const double entry = exp_entry();
     const int b0 = offsets[w], b1 = offsets[w + 1];
-    exp_table(tab);
-    __syncthreads();
     Lse a;
     int bp = 0x7fffffff;
-    for (int i0 = b0 + threadIdx.x; i0 < b1; i0 += 4 * kRedThreads) {
-        double m[4];
-        float sv[4];
+    double m[4];
+    float sv[4];
+    int i0 = b0 + threadIdx.x;
+    auto terms = [&]() {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = i0 + k * kRedThreads;
             m[k] = i < b1 ? kA[w] + kB[ps_idx[i]] + c1 * (double)rec_t[i] : -INFINITY;
             sv[k] = i < b1 ? rec_s[i] : 0.f;
         }
+    };
+    terms();
+    tab[threadIdx.x] = entry;
+    __syncthreads();
+    while (i0 < b1) {
         lse_add4(a, m, sv, tab);
+        i0 += 4 * kRedThreads;
+        if (i0 < b1) terms();
     }
     block_lse(a, bp, tab);
     if (threadIdx.x == 0) {
