@@ -790,6 +790,22 @@ k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int
     }
 }
 
+// Parts end on whole rounds of a block (NGROUP batches) where an image is one round and there are more
+// batches than blocks, or a few rounds and still about a round for every block.
+__host__ __device__ inline bool whole_rounds(int n_img, int batches, int groups, int grid) {
+    const int rounds = (batches + groups - 1) / groups;
+    return (long long)n_img * batches > grid && (rounds == 1 || (rounds < 4 && (long long)n_img * rounds * 8 >= 7ll * grid));
+}
+
+// Where a block's part of the work ends within an image of `len` sets (or batches), v of them into it: whole pieces of
+// q.  With few rounds per image a piece is what the groups do side by side: part of one takes as long, and a
+// block with the ends of two images waits for both.
+__device__ __noinline__ int part_end(long long v, int len, int q) {
+    if (v <= 0) return 0;
+    if (v >= len) return len;
+    return min(len, ((int)v + q / 2) / q * q);
+}
+
 // The wave's sets go by in phases of phase_sets, whose spectra stay in the L2.  Within a phase the (image, batch)
 // pairs, image by image, are split evenly over the blocks, counting a new image as kImageUnits batches
 // of a group (its load and the wait of the groups for one another): a block meets one image, or the end of one
@@ -797,7 +813,7 @@ k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int
 template <class C>
 __global__ void __launch_bounds__(C::THREADS, 1)
 k_score_phases(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int n_img,
-        const float2* __restrict__ ps_spec, int ps_begin, int ps_count, int phase_sets, int s, float c1,
+        const float2* __restrict__ ps_spec, int ps_begin, int ps_count, int phase_sets, int piece, int s, float c1,
         float* __restrict__ rec_t, float* __restrict__ rec_s, int* __restrict__ rec_d, int* __restrict__ status) {
     constexpr int kImageUnits = (6 * C::NGROUP + 5) / 10 > 0 ? (6 * C::NGROUP + 5) / 10 : 1;   // about 0.6 of a round
     extern __shared__ __align__(16) unsigned char smem[];
@@ -813,7 +829,11 @@ k_score_phases(const float2* __restrict__ gtw, const float2* __restrict__ img_sp
         for (int w = (int)(x0 / stride); w < n_img; ++w) {
             const long long at = (long long)w * stride + kImageUnits;   // of the image's first batch
             if (at >= x1) break;
-            const int u0 = (int)max(x0 - at, 0ll), u1 = (int)min(x1 - at, (long long)units);
+            int u0 = (int)max(x0 - at, 0ll), u1 = (int)min(x1 - at, (long long)units);
+            if (piece > 1) {
+                u0 = part_end(x0 - at, units, piece);
+                u1 = part_end(x1 - at, units, piece);
+            }
             if (u0 >= u1) continue;
             const size_t row = (size_t)w * ps_count;
             score_item<C>(sm, Job{gtw, img_spec + (size_t)w * C::N * C::H, nullptr, ps_spec, ps_begin, s, c1, rec_t + row,
@@ -1302,11 +1322,13 @@ int launch_score_records(bioem_ctx* ctx, const bioem_images* im, const bioem_pro
     const float c1f = 0.5f * (3.0f - (float)(C::N * C::N));
     if constexpr (C::PHASES) {
         const int phase = phase_sets<C>(n_img, wl, slots);
-        const long long units = (long long)n_img * ((phase + C::GPB - 1) / C::GPB);
+        const int per_img = ((phase < wl ? phase : wl) + C::GPB - 1) / C::GPB;
+        const long long units = (long long)n_img * per_img;
         const int grid = (int)(units < slots ? units : slots);
+        const int piece = whole_rounds(n_img, per_img, C::NGROUP, grid) ? C::NGROUP : 1;
         bioem_launch_begin(ctx, KID_SCORE);
         k_score_phases<C><<<grid, C::THREADS, C::SMEM, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, ps->d_spec,
-                                                                wbegin, wl, phase, max_shift, c1f, rec_t, rec_s, rec_d,
+                                                                wbegin, wl, phase, piece, max_shift, c1f, rec_t, rec_s, rec_d,
                                                                 ctx->d_status);
         bioem_launch_end(ctx, KID_SCORE);
     } else {
@@ -2164,6 +2186,7 @@ k_score_gathered(const float2* __restrict__ gtw, const float2* __restrict__ img_
         }
         next_w = w;
     }
+    const bool many = offsets[n_img] - offsets[0] > (long long)gridDim.x * GPB;
     for (;;) {
         __syncthreads();   // the previous image's readers of the job are done
         if (threadIdx.x == 0) {
@@ -2172,8 +2195,10 @@ k_score_gathered(const float2* __restrict__ gtw, const float2* __restrict__ img_
                 const long long at = start(w) + kImageSets;   // of the image's first set
                 if (at >= x1) break;
                 const int b0 = offsets[w], len = offsets[w + 1] - b0;
-                const int lo = (int)((max(x0 - at, 0ll) + GPB - 1) / GPB) * GPB;
-                const int hi = min(len, (int)((min(x1 - at, (long long)len) + GPB - 1) / GPB) * GPB);
+                const int rounds = (len + C::PB - 1) / C::PB;
+                const bool whole = many && (rounds == 1 || (rounds < 4 && (long long)n_img * rounds * 8 >= 7ll * gridDim.x));
+                const int piece = whole ? C::PB : GPB;
+                const int lo = part_end(x0 - at, len, piece), hi = part_end(x1 - at, len, piece);
                 if (lo >= hi) continue;
                 job = Job{gtw, img_spec + (size_t)w * C::N * C::H, ps_idx + b0, ps_spec, 0, s, c1, rec_t + b0, rec_s + b0,
                           rec_d + b0};
