@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(C::THREADS, 1)
 k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int n_img,
         const float2* __restrict__ ps_spec, int ps_begin, int ps_count, int chunk, int n_long, int n_items, int s, float c1,
         float* __restrict__ rec_t, float* __restrict__ rec_s, int* __restrict__ rec_d, int* __restrict__ status,
-        int* __restrict__ work) {
+        int* __restrict__ work, int fetch) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int next_item;
     const Sm<C> sm(smem);
@@ -774,7 +774,7 @@ k_score(const float2* __restrict__ gtw, const float2* __restrict__ img_spec, int
         auto first_set = [&](int c) { return c < n_long ? c * chunk : n_long * chunk + (c - n_long) * tail; };
         const int lo = first_set(ci);
         const int hi = min(first_set(ci + 1), ps_count);
-        if (threadIdx.x < 32) {
+        if (fetch && threadIdx.x < 32) {
             const long long nx = (long long)item + gridDim.x / 2;
             if (item < (int)gridDim.x) fetch_share<C>(ps_spec + (size_t)(ps_begin + lo) * C::N * C::H, hi - lo, w, n_img);
             if (nx < n_items) {
@@ -1345,12 +1345,18 @@ int launch_score_records(bioem_ctx* ctx, const bioem_images* im, const bioem_pro
         const long long n_items = n_chunks * n_img;
         if (n_items > 0x7fffffffll) return bioem_set_error(ctx, BIOEM_ERR_UNSUPPORTED_SIZE, "too many work items");
         const int grid = (int)(n_items < slots ? n_items : slots);
+        // no fetching ahead in a single round, where it repeats what the blocks are reading, nor where half a grid of
+        // items, n_img of which share a chunk, reaches further than the L2 keeps (192 px, 6912 sets, us with
+        // and without: 1 image 528 and 466, 2: 899 and 850, 3: 1259 and 1203, 5 (48 MB ahead): 1937 and 1931; 128 px,
+        // +-16 px: 1: 217 and 172, 3: 411 and 399, 8 (53 MB): 882 and 917)
+        const double ahead = 0.5 * grid / n_img * (double)chunk * (double)(sizeof(float2) * C::N * C::H);
+        const int fetch = n_items > slots && ahead < 60e6;
         bioem_launch_begin(ctx, KID_SCORE);
         if (cudaMemsetAsync(ctx->d_work, 0, sizeof(int), ctx->stream) != cudaSuccess)
             return bioem_check_cuda(ctx, cudaGetLastError(), "work counter");
         k_score<C><<<grid, C::THREADS, C::SMEM, ctx->stream>>>(bioem_twiddles(ctx, C::N), im->d_spec, n_img, ps->d_spec,
                                                                 wbegin, wl, (int)chunk, (int)n_long, (int)n_items, max_shift, c1f,
-                                                                rec_t, rec_s, rec_d, ctx->d_status, ctx->d_work);
+                                                                rec_t, rec_s, rec_d, ctx->d_status, ctx->d_work, fetch);
         bioem_launch_end(ctx, KID_SCORE);
     }
     return bioem_check_cuda(ctx, cudaGetLastError(), "k_score");
