@@ -2318,7 +2318,7 @@ __global__ void __launch_bounds__(kRedThreads) k_gathered_pairs_out(const int* _
 
 template <class C>
 int run_gathered(bioem_ctx* ctx, const bioem_images* im, const bioem_projset* ps, int max_shift, const int* offsets,
-                 const int* ps_idx, int nnz, int max_per_image, double* acc, int first, double* pair_lse) {
+                 const int* ps_idx, int nnz, double* acc, int first, double* pair_lse) {
     const int n_img = im->n_img;
     const size_t need = (size_t)nnz * 12;
     if (ctx->rec_bytes < need) {
@@ -2380,7 +2380,7 @@ static int gathered(bioem_ctx* ctx, const bioem_images* images, const bioem_proj
                                images->nx);
     if (images->n_img == 0) return BIOEM_OK;
     if (cudaSetDevice(ctx->device) != cudaSuccess) return bioem_set_error(ctx, BIOEM_ERR_CUDA, "cudaSetDevice");
-#define G(C) run_gathered<C>(ctx, images, projset, max_shift, d_offsets, d_ps_idx, nnz, max_per_image, d_acc, first, d_pair_lse)
+#define G(C) run_gathered<C>(ctx, images, projset, max_shift, d_offsets, d_ps_idx, nnz, d_acc, first, d_pair_lse)
     switch (images->nx) {
         case 32: return G(C32_4);
         case 64: return max_shift <= 4 ? G(C64_4) : G(C64_8);
