@@ -610,22 +610,31 @@ __global__ void k_ctf_table(const double* __restrict__ coef, int nctf, int N, do
     }
 }
 
-// a + b and its rounding error (Knuth)
-__device__ __forceinline__ float two_sum(float a, float b, float& err) {
-    const float s = a + b, t = s - a;
-    err = (a - (s - t)) + (b - t);
+// a + b and its rounding error (Knuth), two numbers side by side
+__device__ __forceinline__ float2 two_sum(float2 a, float2 b, float2& err) {
+    const float2 minus = make_float2(-1.f, -1.f);
+    const float2 s = __fadd2_rn(a, b), t = __ffma2_rn(a, minus, s);
+    err = __fadd2_rn(__ffma2_rn(__ffma2_rn(t, minus, s), minus, a), __ffma2_rn(t, minus, b));
     return s;
 }
 
-// hi + mid + lo += w x^2, w a power of two: the square and the sums with their rounding errors (error-free
-// transforms of Dekker and Knuth), to about 2^-66 of the sum for a spectrum's share of one thread.
-__device__ __forceinline__ void add_square(float& hi, float& mid, float& lo, float x, float w) {
-    const float p = x * x, e = fmaf(x, x, -p);
-    float e1, e2, e3;
-    hi = two_sum(hi, p * w, e1);
+// hi + mid + lo += w v^2 for both parts of v, w a power of two: the square and the sums with their rounding errors
+// (error-free transforms of Dekker and Knuth), to about 2^-66 of the sum for a spectrum's share of one thread.
+__device__ __forceinline__ void add_square(float2& hi, float2& mid, float2& lo, float2 v, float2 w) {
+    const float2 p = __fmul2_rn(v, v), e = __ffma2_rn(v, v, make_float2(-p.x, -p.y));
+    float2 e1, e2, e3;
+    hi = two_sum(hi, __fmul2_rn(p, w), e1);
     mid = two_sum(mid, e1, e2);
-    mid = two_sum(mid, e * w, e3);
-    lo += e2 + e3;
+    mid = two_sum(mid, __fmul2_rn(e, w), e3);
+    lo = __fadd2_rn(lo, __fadd2_rn(e2, e3));
+}
+
+// The sum of both parts, rounded to float64 (the two of hi and of mid are added exactly in FP32: each conversion to
+// float64 and each float64 sum takes as long as 70 FP32 ones).
+__device__ __forceinline__ double square_total(float2 hi, float2 mid, float2 lo) {
+    float2 e;   // of (hi, mid)
+    const float2 s = two_sum(make_float2(hi.x, mid.x), make_float2(hi.y, mid.y), e);
+    return (double)s.x + (((double)s.y + (double)e.x) + (double)(e.y + (lo.x + lo.y)));
 }
 
 // One orientation per block: transform I0, and for every PSF c the energy B_c = sum_{k != 0} w_kx |F T_c|^2 (of
@@ -680,7 +689,8 @@ __global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(con
         const int nc = min(kPsfChunk, nctf - c0);
         for (int c = 0; c < nc; ++c) {
             const float* Tc = T + (size_t)(c0 + c) * N * H;
-            float hi = 0.f, mid = 0.f, lo = 0.f;
+            const float2 none = make_float2(0.f, 0.f);
+            float2 hi = none, mid = none, lo = none;   // of the real and the imaginary parts
 #pragma unroll 1
             for (int i0 = 0; i0 < PER; i0 += kUnroll) {
 #pragma unroll
@@ -691,12 +701,11 @@ __global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(con
                         float2 v = c_scale(c_scale(sm.F[o], __ldg(Tc + o)), sc);
                         if (o == 0) v = make_float2(0.f, 0.f);   // DC (see half_energy)
                         const float w = kx == 0 || kx == N / 2 ? 1.f : 2.f;
-                        add_square(hi, mid, lo, v.x, w);
-                        add_square(hi, mid, lo, v.y, w);
+                        add_square(hi, mid, lo, v, make_float2(w, w));
                     }
                 }
             }
-            double e = (double)hi + ((double)mid + (double)lo);
+            double e = square_total(hi, mid, lo);
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
             if (lane == 0) part[c][warp] = e;

@@ -32,26 +32,38 @@ def _library(tmp_path, body: str):
 
 
 def test_squares_are_summed_beyond_float64(tmp_path):
-    """A thread's share of a spectrum (33 coefficients, values falling over six decades) as squares with weights 1
-    and 2: the three parts hold the sum to 2^-60, where float64's own rounding is 2^-53.  (Each square's
-    error and each sum's is kept but for the last part's rounding: 66 x 2^-24 of 2^-48.)"""
-    lib = _library(str(tmp_path), _function("prep_project.cu", "two_sum") + _function("prep_project.cu", "add_square") + '''
-extern "C" void sum_squares(const float* x, const float* w, int n, float* out) {
-    float hi = 0.f, mid = 0.f, lo = 0.f;
-    for (int i = 0; i < n; ++i) add_square(hi, mid, lo, x[i], w[i]);
-    out[0] = hi; out[1] = mid; out[2] = lo;
+    """A thread's share of a spectrum (33 coefficients, sizes over six decades) as squares with weights 1
+    and 2: the parts hold the sum to 2^-60, where float64's own rounding is 2^-53.  (Each square's
+    error and each sum's is kept but for the last part's rounding: 66 x 2^-24 of 2^-48.)  Their total in float64 is
+    rounded once, but for 2^-24 of a rounding."""
+    lib = _library(str(tmp_path), '''
+struct float2 { float x, y; };
+static float2 make_float2(float x, float y) { return float2{x, y}; }
+static float2 __fadd2_rn(float2 a, float2 b) { return {a.x + b.x, a.y + b.y}; }
+static float2 __fmul2_rn(float2 a, float2 b) { return {a.x * b.x, a.y * b.y}; }
+static float2 __ffma2_rn(float2 a, float2 b, float2 c) { return {fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)}; }
+''' + _function("prep_project.cu", "two_sum") + _function("prep_project.cu", "add_square") +
+                   _function("prep_project.cu", "square_total") + '''
+extern "C" double sum_squares(const float* x, const float* w, int n, float* out) {
+    float2 hi{0.f, 0.f}, mid = hi, lo = hi;
+    for (int i = 0; i < n; ++i) add_square(hi, mid, lo, float2{x[2 * i], x[2 * i + 1]}, float2{w[i], w[i]});
+    const float2 r[3] = {hi, mid, lo};
+    for (int k = 0; k < 3; ++k) { out[2 * k] = r[k].x; out[2 * k + 1] = r[k].y; }
+    return square_total(hi, mid, lo);
 }
 ''')
+    lib.sum_squares.restype = ctypes.c_double
     rng = np.random.default_rng(3)
     ptr = lambda a: a.ctypes.data_as(ctypes.c_void_p)
     for _ in range(200):
-        x = (rng.standard_normal(66) * 10.0 ** rng.uniform(-6, 0, 66)).astype(np.float32)
-        w = rng.integers(1, 3, 66).astype(np.float32)
-        out = np.empty(3, dtype=np.float32)
-        lib.sum_squares(ptr(x), ptr(w), 66, ptr(out))
-        exact = sum(Fraction(float(b)) * Fraction(float(a)) ** 2 for a, b in zip(x, w))
+        x = (rng.standard_normal(66) * 10.0 ** np.repeat(rng.uniform(-6, 0, 33), 2)).astype(np.float32)
+        w = rng.integers(1, 3, 33).astype(np.float32)
+        out = np.empty(6, dtype=np.float32)
+        total = lib.sum_squares(ptr(x), ptr(w), 33, ptr(out))
+        exact = sum(Fraction(float(b)) * Fraction(float(a)) ** 2 for a, b in zip(x, np.repeat(w, 2)))
         got = sum(Fraction(float(v)) for v in out)
         assert abs(got - exact) <= exact / 2 ** 60
+        assert abs(Fraction(total) - exact) <= exact * Fraction(101, 100) / 2 ** 53
 
 
 def test_exponential_of_the_reductions(tmp_path):
