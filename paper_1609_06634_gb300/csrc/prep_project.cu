@@ -366,7 +366,7 @@ float window_reach(double sigma, double pixel) {
 // Bound by issue (0.7 per cycle and scheduler) and the latency of erfc: ~540 warp instructions per atom at 128 px
 // (1.1 A), most of them for the tables' three passes and for 6.7 tiles' sums.  128 px, 5000 atoms, sigma 1.5 A, us per orientation: 7.1 when every boundary
 // of the image was tabulated for every atom and whole rows were summed, 3.4 with 8 warps of 4 tiles, 3.1
-// with 16 warps of 2, 2.9 with atoms taken by the warps that are free.
+// with 16 warps of 2, 2.7 with atoms taken by the warps that are free.
 template <int N>
 struct ProjCfg {
     static constexpr int LR = N == 32 ? 2 : 4, LC = LR;
@@ -377,8 +377,8 @@ struct ProjCfg {
     static_assert(TCOLS * TC == N && TROWS * TR == N && BAND * TCOLS == NW && TPW * BAND == TROWS, "tiles cover the image");
     static constexpr int T = 32 * NW;
     // Warps take the atoms they tabulate one by one, after their sums, so that those with sparse tiles tabulate
-    // more: 1024 maps at 128 px 4.79 -> 4.56 ms, 500 at 192 px 7.66 -> 5.18 ms.  At 96 px (two passes per
-    // atom) and below equal shares are as good or better: 2.35 against 2.48 ms for 1000 maps at 64 px.
+    // more: 1024 maps at 128 px 3.07 -> 2.78 ms, 500 at 192 px 5.59 -> 3.03 ms.  At 96 px (two passes per
+    // atom) and below equal shares are as good or better: 1000 maps 2.46 against 2.45 ms, at 64 px 1.51 against 1.61.
     static constexpr bool TAKE = N >= 128;
     static constexpr int CH = 32;                                  // atoms per chunk: one per lane of a ballot
     static constexpr size_t SM_TAB = (size_t)CH * 2 * N * sizeof(float);   // gx, gy rows of a chunk
@@ -647,7 +647,6 @@ __device__ __forceinline__ double square_total(float2 hi, float2 mid, float2 lo)
 // The products are scaled by a power of two so that the largest |F| is near 1; a B so small against it that
 // squares may have lost bits to underflow (below kSmall) is summed again in float64 throughout.
 constexpr int kPsfChunk = 16;   // PSFs whose energies are reduced together
-constexpr int kUnroll = 11;
 constexpr double kSmall = 1e-12;
 
 template <int N>
@@ -691,18 +690,17 @@ __global__ void __launch_bounds__(Dft<N>::T, N == 192 ? 1 : 2) k_psf_spectra(con
             const float* Tc = T + (size_t)(c0 + c) * N * H;
             const float2 none = make_float2(0.f, 0.f);
             float2 hi = none, mid = none, lo = none;   // of the real and the imaginary parts
-#pragma unroll 1
-            for (int i0 = 0; i0 < PER; i0 += kUnroll) {
+            // unrolled as a whole, so that the PSF's values are loaded ahead (in runs of 11, each waited for, the 128
+            // orientations x 8 PSFs of a re-ranking wave took 172 us instead of 119)
 #pragma unroll
-                for (int i = 0; i < kUnroll; ++i) {
-                    const int o = threadIdx.x + (i0 + i) * TH;
-                    if (o < N * H) {
-                        const int kx = o % H;
-                        float2 v = c_scale(c_scale(sm.F[o], __ldg(Tc + o)), sc);
-                        if (o == 0) v = make_float2(0.f, 0.f);   // DC (see half_energy)
-                        const float w = kx == 0 || kx == N / 2 ? 1.f : 2.f;
-                        add_square(hi, mid, lo, v, make_float2(w, w));
-                    }
+            for (int i = 0; i < PER; ++i) {
+                const int o = threadIdx.x + i * TH;
+                if (o < N * H) {
+                    const int kx = o % H;
+                    float2 v = c_scale(c_scale(sm.F[o], __ldg(Tc + o)), sc);
+                    if (o == 0) v = make_float2(0.f, 0.f);   // DC (see half_energy)
+                    const float w = kx == 0 || kx == N / 2 ? 1.f : 2.f;
+                    add_square(hi, mid, lo, v, make_float2(w, w));
                 }
             }
             double e = square_total(hi, mid, lo);

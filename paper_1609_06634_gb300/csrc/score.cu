@@ -993,8 +993,8 @@ __device__ __forceinline__ void acc_merge_prev(Acc& r, const Acc& prev) {
 // and, if requested, write the per-orientation posteriors of the share's orientations.  Parts are whole
 // orientations; an image is cut into enough of them to occupy the GPU (reduce_parts).  An image in one part
 // is folded in place (parts = prev = the running accumulators; prev null: the first wave).  Bound by the
-// float64 pipe (13 operations per record; 64 images x 6912 sets: 93 us as one block per image with the
-// library's exponential, 28 us so; 16 images with per-orientation output: 181 -> 15 us).
+// float64 pipe (14 operations per record; 64 images x 6912 sets: 93 us as one block per image with the
+// library's exponential, 33 us so; 16 images with per-orientation output: 181 -> 16 us).
 __global__ void __launch_bounds__(kRedThreads) k_reduce_wave(
     const float* __restrict__ rec_t, const float* __restrict__ rec_s, const int* __restrict__ rec_d,
     const double* __restrict__ kA, const double* __restrict__ kB, int ps_begin, int wave_len, int nctf,
@@ -1611,7 +1611,7 @@ extern "C" int bioem_score_noalloc(bioem_ctx* ctx, const bioem_images* images, c
 // launches of the sizes present are parallel branches of the graph, so that the blocks of the next
 // size start on the SMs that the previous size's blocks leave.  (One kernel that held all four sizes
 // gave every size the register count and the 256 threads of the largest: 19.2 ms for 4 models x 4
-// stacks, 1.03e6 pairs, against 16.1 ms so.)
+// stacks, 1.03e6 pairs; 16.1 ms by size, 13.9 with the instances' other changes.)
 #include <string>
 #include <vector>
 
