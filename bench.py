@@ -86,12 +86,13 @@ def kernel_source_sha(kernel: str) -> str:
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum, one-pass ncu captures), valid only for
 # the kernel source they were taken on (kernel_source_sha).
 #   k_score: per evaluated pair, from one launch of 2048 images x 4608 sets (above L2), scaled by
-#            pairs to the bench's launches (profiles/k_score_throughput.md).
+#            pairs to the bench's launches (profiles/k_score_throughput.md): an upper estimate, since a
+#            launch's chunks (478 sets) are larger than the capture's (384) and re-read the images less.
 #   k_score_gemm: per launch of the precision workloads (64 images x 6912 sets, +-4 px).
-K_SCORE_TRAFFIC = {"source_sha256": "67f77ea988b4d2ce701dc6cf4863691b2f57eb4d524e737f2c8d0bca9126f5c0", "bytes_per_pair": (2361264640 + 117821696) / (2048 * 4608)}
-K_SCORE_GEMM_TRAFFIC = {"source_sha256": "083bf58cd6cd1f4630508bfac27c7d80488b5d30f742979416b2b4b648b51731", "bytes_per_launch": {
-    '128/bf16x2': 3528212224, '128/fp16x2': 3795020800, '128/bf16x2_real': 3479105792, '128/fp16x2_real': 4123705344,
-    '64/bf16x2': 895100672, '64/fp16x2': 895214592, '64/bf16x2_real': 868046336, '64/fp16x2_real': 867884544}}
+K_SCORE_TRAFFIC = {"source_sha256": "d4121b68d1b3bf3c7df21dae9ced320642b03a1fceb93c68596c64da7fb3df02", "bytes_per_pair": (2363574784 + 117958912) / (2048 * 4608)}
+K_SCORE_GEMM_TRAFFIC = {"source_sha256": "489606e882a24d4f9fb111dbabb7e0224a7af213a3d80f9975998e05f7e206a7", "bytes_per_launch": {
+    '128/bf16x2': 3776552960, '128/fp16x2': 4476913920, '128/bf16x2_real': 3817636352, '128/fp16x2_real': 4565877760,
+    '64/bf16x2': 895163904, '64/fp16x2': 895484160, '64/bf16x2_real': 867652352, '64/fp16x2_real': 867508736}}
 K_SCORE_TC_TRAFFIC = {"source_sha256": "", "bytes_per_pair": None}
 
 

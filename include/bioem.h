@@ -262,11 +262,12 @@ int bioem_autotune_load(const char* cache_path, int* n_taken, int* n_skipped);
 /* Scoring of per-image lists of parameter sets (the paper has no counterpart: it scores every
  * image on the full grid; this serves proposals that restrict each image to a few grid cells).
  * Image w is scored against projset sets d_ps_idx[d_offsets[w] .. d_offsets[w+1]) (CSR, device
- * int arrays), every displacement |d| <= max_shift, and the results are folded into d_acc [n_img][2] float64 device = running (max, sum exp(. - max)) of
- * ln L over everything scored so far; first != 0 overwrites d_acc instead of folding into it.
- * bioem_acc_logP turns the accumulators into ln P: d_logP[w] = max + ln sum - log_norm (pass
- * log_norm = ln(number of sets scored per image x S)).  Calling it over several projection sets
- * (waves of grid cells) accumulates one posterior.  max_per_image must not be negative and has no
+ * int arrays), every displacement |d| <= max_shift, and the results are folded into d_acc
+ * [n_img][2] float64 device = running (max, sum exp(. - max)) of ln L over everything scored so
+ * far; first != 0 overwrites d_acc instead of folding into it.  bioem_acc_logP turns the
+ * accumulators into ln P: d_logP[w] = max + ln sum - log_norm (pass log_norm = ln(number of sets
+ * scored per image x S)).  Calling it over several projection sets (waves of grid cells)
+ * accumulates one posterior.  max_per_image must not be negative and has no
  * other part: the work is divided by the lists' lengths in d_offsets. */
 int bioem_score_gathered(bioem_ctx* ctx, const bioem_images* images, const bioem_projset* projset, int max_shift,
                          const int* d_offsets, const int* d_ps_idx, int nnz, int max_per_image, double* d_acc,
